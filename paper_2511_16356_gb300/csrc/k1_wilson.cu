@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(kLaneWalkerBlock) k_wilson(GraphView g, WaveVi
     int phase = kSeek;
     bool stopped = false;
     bool rejected = false;
+    bool failed = false;  // its words are unfinished: flagged -1, never traversed
 
     // Every iteration: phase-specific arithmetic, then ONE gather (the word of
     // one vertex, with its record when the lane may walk from it), then
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(kLaneWalkerBlock) k_wilson(GraphView g, WaveVi
             }
             if ((!kReject && ++steps > step_cap) || w_count(wu) + 1 >= (1u << 25)) {
                 atomicOr(w.err, kErrStepLimit);
+                failed = true;
                 break;
             }
             a = v;
@@ -156,6 +158,7 @@ __global__ void __launch_bounds__(kLaneWalkerBlock) k_wilson(GraphView g, WaveVi
                 u = w_next(wa);
                 if (len > n || u < 0 || u >= n) {  // a path longer than n means corrupt state
                     atomicOr(w.err, kErrBadTree);
+                    failed = true;
                     break;
                 }
             }
@@ -192,7 +195,7 @@ __global__ void __launch_bounds__(kLaneWalkerBlock) k_wilson(GraphView g, WaveVi
     if (done_flag) {
         // publish the finished tree (its depth + 1) after its words and order
         __threadfence_system();
-        done_flag[t] = maxd + 1;
+        done_flag[t] = failed ? -1 : maxd + 1;
     }
 }
 
@@ -333,6 +336,7 @@ __global__ void __launch_bounds__(kWarpWalkerBlock, 24)
     int64_t pos = rs_q ? (int64_t)rs_pos[t] : w.pos0;   // warp-uniform, ord[0 .. pos) placed
     bool bad = false;
     bool rejected = false;  // warp-uniform
+    bool failed = false;    // warp-uniform: unfinished words, flagged -1
 
     for (int64_t it = 0;; ++it) {
         // ---- hand out start vertices to idle lanes
@@ -350,6 +354,7 @@ __global__ void __launch_bounds__(kWarpWalkerBlock, 24)
         // the warp notices within 8 iterations
         if (it > iter_cap || ((it & 7) == 0 && __any_sync(kFull, bad))) {
             if (lane == 0) atomicOr(w.err, bad ? kErrBadTree : kErrIterLimit);
+            failed = true;
             break;
         }
         if constexpr (kReject) {
@@ -576,6 +581,7 @@ __global__ void __launch_bounds__(kWarpWalkerBlock, 24)
         }
         return;
     }
+    failed = failed || __any_sync(kFull, bad);
     if (done_flag) {
         // publish the finished tree (its depth + 1) to the host, after every
         // lane's words and order entries are visible
@@ -583,7 +589,7 @@ __global__ void __launch_bounds__(kWarpWalkerBlock, 24)
         __syncwarp();
         if (lane == 0) {
             __threadfence_system();
-            done_flag[t] = md + 1;
+            done_flag[t] = failed ? -1 : md + 1;
         }
     }
 }

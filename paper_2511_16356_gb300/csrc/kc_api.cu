@@ -405,9 +405,6 @@ void ensure_pipeline(kc_graph *g, int64_t B) {
     if (B <= g->done_cap) return;
     hfree(g->h_done);
     hfree(g->h_map);
-    hfree(g->h_segtab);
-    dfree(g->d_segtab);
-    dfree(g->d_segx);
     dfree(g->d_map);
     g->h_done = g->h_map = g->d_done = nullptr;
     g->done_cap = 0;
