@@ -479,9 +479,11 @@ inline unsigned blk(int64_t x, int t) { return (unsigned)((x + t - 1) / t); }
 }  // namespace
 
 cudaError_t launch_edge_pre_init(int64_t n, int64_t B, int32_t u, int32_t v, uint64_t *word,
-                                 int32_t *ord, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(word, 0, sizeof(uint64_t) * (size_t)(B * n), s);
-    if (e != cudaSuccess) return e;
+                                 int32_t *ord, bool cleared, cudaStream_t s) {
+    if (cleared) {
+        cudaError_t e = cudaMemsetAsync(word, 0, sizeof(uint64_t) * (size_t)(B * n), s);
+        if (e != cudaSuccess) return e;
+    }
     k_edge_pre_init<<<blk(B, 128), 128, 0, s>>>(n, B, u, v, word, ord);
     return cudaGetLastError();
 }

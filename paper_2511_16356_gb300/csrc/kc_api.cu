@@ -369,11 +369,52 @@ int fast_traversal(const kc_graph *g) {
     return (g->ttf_variant == KC_TTF_SCAN && g->n >= (1 << 16)) ? kTravLeafUp : kTravChunked;
 }
 
+// Whether waves run the one-walker kernels with arrows drawn ahead (k1_solo.cu)
+// in place of the handle's walker: always for LANE, and under AUTO on
+// long-diameter graphs, where 32 walkers of a tree mostly wait for one another
+// (40000-vertex grid, walk in ms with 32 walkers / one: 64 trees 192 / 114, 500
+// trees 348 / 184, 4000 trees 590 / 316).  On graphs of low diameter the 32
+// walkers spread and stay faster (20000-vertex random graph: 24 / 28 ms).
+bool use_solo(const kc_graph *g) {
+    if (kc_host::queue_bits(g->max_deg) > kc_host::kMaxQueueBits) return false;
+    if (g->walker == KC_WALK_LANE) return true;
+    return g->walker == KC_WALK_WARP && g->auto_walker &&
+           g->ttf_variant == KC_TTF_BIT;
+}
+
+// Words of k1_solo.cu with the arrow queues of `root`'s trees (-1: no vertex in
+// the tree).  A long-diameter graph departs a dozen times from a vertex, the
+// others once or twice: their first queues stay short.
+void init_queues(kc_graph *g, const GraphView &gv, const WaveView &w, const int64_t *sids,
+                 int32_t root, cudaStream_t s) {
+    KC_CK(g, launch_queue_init(gv, w, g->seed, sids, root, kc_host::queue_bits(g->max_deg),
+                               g->ttf_variant == KC_TTF_BIT ? 32 : 2, s));
+}
+
+// Words and order of a wave before its walk, rooted at g->root.
+void init_wave(kc_graph *g, const GraphView &gv, const WaveView &w, const Carved &c, bool solo) {
+    if (solo) init_queues(g, gv, w, c.sids, g->root, g->stream);
+    else KC_CK(g, launch_wave_init(gv, w, g->stream));
+}
+
+// Error bits of a walk that ran k1_solo.cu after which the wave is repeated with
+// the handle's own walker: a departure count past its field, or (when the
+// 32-walker kernel stands behind AUTO, whose cap bounds each walker and not
+// the tree) the step cap.
+bool solo_retry(const kc_graph *g, uint32_t err) {
+    return (err & kErrCountField) ||
+           ((err & kErrStepLimit) && g->walker == KC_WALK_WARP);
+}
+
 // Wilson's algorithm for the B trees of `w` (words and order already
-// initialised, w.pos0 vertices placed) with the handle's walker.
-void run_wilson(kc_graph *g, const GraphView &gv, const WaveView &w, const Carved &c) {
+// initialised for it, w.pos0 vertices placed) with k1_solo.cu or the handle's
+// walker.
+void run_wilson(kc_graph *g, const GraphView &gv, const WaveView &w, const Carved &c, bool solo) {
     const int64_t cap = step_cap_of(g);
-    if (g->walker == KC_WALK_LANE) {
+    if (solo) {
+        KC_CK(g, launch_wilson_queue(gv, w, g->seed, c.sids,
+                                     kc_host::queue_bits(g->max_deg), cap, false, g->num_sms, g->stream));
+    } else if (g->walker == KC_WALK_LANE) {
         KC_CK(g, launch_wilson(gv, w, g->seed, c.sids, cap, g->stream));
     } else if (g->walker == KC_WALK_WARP) {
         KC_CK(g, launch_wilson_warp(gv, w, g->seed, c.sids, g->d_sorder, cap, g->stream));
@@ -394,7 +435,9 @@ void run_wilson(kc_graph *g, const GraphView &gv, const WaveView &w, const Carve
     }
 }
 
-int wilson_launches(const kc_graph *g) { return g->walker == KC_WALK_HYBRID ? 2 : 1; }
+int wilson_launches(const kc_graph *g, bool solo) {
+    return !solo && g->walker == KC_WALK_HYBRID ? 2 : 1;
+}
 
 // One full sampling pass over sample ids [sid0, sid0 + B): walk, traverse,
 // evaluate f.  Leaves per-tree results in the carved workspace.
@@ -422,7 +465,8 @@ void ensure_pipeline(kc_graph *g, int64_t B) {
 // slowest trees waits for the end of the walk.
 // With reject, the walk abandons trees past cfg.reject_steps departures; they
 // flag -1 and are left out of the chunks (their f stays 0, their steps -1).
-void run_wave_pipelined(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool reject = false) {
+// Returns false when the wave has to be repeated without k1_solo.cu.
+bool run_wave_pipelined(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool reject, bool solo) {
     ensure_pipeline(g, B);
     GraphView gv = view_of(g);
     Carved c = carve(g, p);
@@ -451,14 +495,18 @@ void run_wave_pipelined(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool reje
     KC_CK(g, launch_iota(c.sids, sid0, B, s1));
     {
         Phase ph(g, g->t_init);
-        KC_CK(g, launch_wave_init(gv, w, s1));
+        init_wave(g, gv, w, c, solo);
         ph.done(1);
     }
     cudaEvent_t ev_ready = event(), ev_w0 = event(), ev_w1 = event();
     KC_CK(g, cudaEventRecord(ev_ready, s1));
     KC_CK(g, cudaStreamWaitEvent(s2, ev_ready, 0));
     KC_CK(g, cudaEventRecord(ev_w0, s1));
-    if (g->walker == KC_WALK_LANE) {
+    if (solo) {
+        KC_CK(g, launch_wilson_queue(gv, w, g->seed, c.sids, kc_host::queue_bits(g->max_deg),
+                                     reject ? g->cfg.reject_steps : step_cap_of(g), reject,
+                                     g->num_sms, s1, g->d_done));
+    } else if (g->walker == KC_WALK_LANE) {
         if (reject)
             KC_CK(g, launch_wilson_reject(gv, w, g->seed, c.sids, nullptr, g->cfg.reject_steps,
                                           s1, g->d_done));
@@ -563,6 +611,7 @@ void run_wave_pipelined(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool reje
     }
     uint32_t hdr[2] = {0, 0};
     KC_CK(g, copy_sync(g, hdr, g->d_err, sizeof(hdr), cudaMemcpyDeviceToHost));
+    if (solo && solo_retry(g, hdr[0])) return false;
     if (hdr[0] & kErrStepLimit) {
         g->last_error = "Wilson walk exceeded the step cap";
         throw Fail{KC_ERR_STEP_LIMIT};
@@ -571,6 +620,7 @@ void run_wave_pipelined(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool reje
         g->last_error = "inconsistent tree state, walker iteration cap or traversal stack overflow";
         throw Fail{KC_ERR_CUDA};
     }
+    return true;
 }
 
 void run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = false) {
@@ -580,7 +630,8 @@ void run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
         B > 1 &&
         (B > p.BT || g->n >= (1 << 16))) {
         try {
-            run_wave_pipelined(g, p, B, sid0);
+            if (!run_wave_pipelined(g, p, B, sid0, false, use_solo(g)))
+                run_wave_pipelined(g, p, B, sid0, false, false);
         } catch (Fail &) {
             // let both streams drain before the workspace is reused
             cudaStreamSynchronize(g->stream);
@@ -593,21 +644,24 @@ void run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
     Carved c = carve(g, p);
     WaveView w = c.wv;
     w.B = B;
-    KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
     KC_CK(g, launch_iota(c.sids, sid0, B, g->stream));
     reset_segtab(g, B);
-    {
-        Phase ph(g, g->t_init);
-        KC_CK(g, launch_wave_init(gv, w, g->stream));
-        ph.done(1);
-    }
-    {
-        Phase ph(g, g->t_wilson);
-        run_wilson(g, gv, w, c);
-        ph.done(wilson_launches(g));
-    }
     uint32_t hdr[2] = {0, 0};
-    KC_CK(g, copy_sync(g, hdr, g->d_err, sizeof(hdr), cudaMemcpyDeviceToHost));
+    for (bool solo = use_solo(g);; solo = false) {
+        KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
+        {
+            Phase ph(g, g->t_init);
+            init_wave(g, gv, w, c, solo);
+            ph.done(1);
+        }
+        {
+            Phase ph(g, g->t_wilson);
+            run_wilson(g, gv, w, c, solo);
+            ph.done(wilson_launches(g, solo));
+        }
+        KC_CK(g, copy_sync(g, hdr, g->d_err, sizeof(hdr), cudaMemcpyDeviceToHost));
+        if (!solo || !solo_retry(g, hdr[0])) break;
+    }
     if (hdr[0] & kErrStepLimit) {
         g->last_error = "Wilson walk exceeded the step cap";
         throw Fail{KC_ERR_STEP_LIMIT};
@@ -929,6 +983,7 @@ void edit_graph(kc_graph *g, int32_t u, int32_t v, bool insert) {
         throw Fail{KC_ERR_CUDA};
     }
     g->m += insert ? 1 : -1;
+    g->max_deg += insert ? 1 : 0;
     g->host_csr_stale = true;
     KC_CK(g, launch_build_records(view_of(g), g->d_rec, g->d_deg, g->stream));
     g->t_update.launches += 4;
@@ -1050,26 +1105,33 @@ void resample_slots(kc_graph *g, const std::vector<int64_t> &slots, bool cond, i
         const int64_t b = std::min<int64_t>(chunk, (int64_t)(slots.size() - c0));
         KC_CK(g, cudaMemcpyAsync(ub.slots, slots.data() + c0, sizeof(int64_t) * b,
                                  cudaMemcpyHostToDevice, g->stream));
-        KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
         Carved c = carve(g, p);
         WaveView w = c.wv;
         w.B = b;
+        w.pos0 = cond ? 2 : 1;
         KC_CK(g, launch_iota(c.sids, g->next_sid, b, g->stream));
-        if (cond) {
-            KC_CK(g, launch_edge_pre_init(g->n, b, u, v, w.word, w.ord, g->stream));
-            w.pos0 = 2;
-        } else {
-            KC_CK(g, launch_wave_init(gv, w, g->stream));
-            w.pos0 = 1;
+        for (bool solo = use_solo(g);; solo = false) {
+            KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
+            if (cond) {
+                if (solo) init_queues(g, gv, w, c.sids, -1, g->stream);
+                KC_CK(g, launch_edge_pre_init(g->n, b, u, v, w.word, w.ord, !solo, g->stream));
+            } else {
+                init_wave(g, gv, w, c, solo);
+            }
+            run_wilson(g, gv, w, c, solo);
+            g->t_update.launches += wilson_launches(g, solo);
+            if (!solo) break;
+            uint32_t err = 0;
+            KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
+            if (!solo_retry(g, err)) break;
         }
-        run_wilson(g, gv, w, c);
         KC_CK(g, launch_words_to_slots(g->n, b, w.word, ub.slots, g->d_parents, g->root,
                                        cond ? v : -1, g->d_err, g->stream));
         KC_CK(g, launch_scatter_results(ub.slots, b, nullptr, w.steps, c.sids, g->d_f,
                                         g->d_steps, g->d_sid, g->stream));
         check_err(g, "resample");
         g->next_sid += b;
-        g->t_update.launches += 4 + wilson_launches(g);
+        g->t_update.launches += 4;
         std::vector<int64_t> part(slots.begin() + c0, slots.begin() + c0 + b);
         for (int64_t x : part) g->h_modified[(size_t)x] = 1;
         refresh_slots(g, part);
@@ -1309,27 +1371,34 @@ void run_wave_reject(kc_graph *g, Plan &p, int64_t B, int64_t sid0) {
     Carved c = carve(g, p);
     WaveView w = c.wv;
     w.B = B;
-    KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
     KC_CK(g, cudaMemsetAsync(w.f, 0, sizeof(int64_t) * (size_t)B, g->stream));
     KC_CK(g, launch_iota(c.sids, sid0, B, g->stream));
     reset_segtab(g, B);
-    {
-        Phase ph(g, g->t_init);
-        KC_CK(g, launch_wave_init(gv, w, g->stream));
-        ph.done(1);
-    }
-    {
-        Phase ph(g, g->t_wilson);
-        if (g->walker == KC_WALK_LANE)
-            KC_CK(g, launch_wilson_reject(gv, w, g->seed, c.sids, nullptr, g->cfg.reject_steps,
-                                          g->stream));
-        else
-            KC_CK(g, launch_wilson_warp_reject(gv, w, g->seed, c.sids, g->d_sorder,
-                                               g->cfg.reject_steps, g->stream));
-        ph.done(1);
-    }
     uint32_t hdr[2] = {0, 0};
-    KC_CK(g, copy_sync(g, hdr, g->d_err, sizeof(hdr), cudaMemcpyDeviceToHost));
+    for (bool solo = use_solo(g);; solo = false) {
+        KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
+        {
+            Phase ph(g, g->t_init);
+            init_wave(g, gv, w, c, solo);
+            ph.done(1);
+        }
+        {
+            Phase ph(g, g->t_wilson);
+            if (solo)
+                KC_CK(g, launch_wilson_queue(gv, w, g->seed, c.sids,
+                                             kc_host::queue_bits(g->max_deg),
+                                             g->cfg.reject_steps, true, g->num_sms, g->stream));
+            else if (g->walker == KC_WALK_LANE)
+                KC_CK(g, launch_wilson_reject(gv, w, g->seed, c.sids, nullptr,
+                                              g->cfg.reject_steps, g->stream));
+            else
+                KC_CK(g, launch_wilson_warp_reject(gv, w, g->seed, c.sids, g->d_sorder,
+                                                   g->cfg.reject_steps, g->stream));
+            ph.done(1);
+        }
+        KC_CK(g, copy_sync(g, hdr, g->d_err, sizeof(hdr), cudaMemcpyDeviceToHost));
+        if (!solo || !solo_retry(g, hdr[0])) break;
+    }
     if (hdr[0] & kErrStepLimit) {
         // a single vertex's departure counter filled its 25 bits
         g->last_error = "Wilson walk exceeded the per-vertex departure limit";
@@ -1423,7 +1492,8 @@ void do_sample_reject(kc_graph *g, int64_t ntrees) {
             }
             if (B > 1 && (B > p.BT || g->n >= (1 << 16))) {
                 try {
-                    run_wave_pipelined(g, p, B, g->next_sid, true);
+                    if (!run_wave_pipelined(g, p, B, g->next_sid, true, use_solo(g)))
+                        run_wave_pipelined(g, p, B, g->next_sid, true, false);
                 } catch (Fail &) {
                     // let both streams drain before the workspace is reused
                     cudaStreamSynchronize(g->stream);
@@ -1556,6 +1626,7 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
             std::vector<const int64_t *> sids;
             std::vector<const int32_t *> sorders;
             std::vector<int64_t> caps;
+            std::vector<int32_t> qbits;
             std::vector<int32_t> idx;  // graph of each table row
             std::vector<int64_t> bs;
             for (int32_t i = 0; i < count; ++i) {
@@ -1566,55 +1637,101 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                 WaveView w = c.wv;
                 w.B = B;
                 const GraphView v = view_of(g);
-                KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), s0));
                 KC_CK(g, launch_iota(c.sids, g->next_sid, B, s0));
-                KC_CK(g, launch_wave_init(v, w, s0));
                 gv.push_back(v);
                 wv.push_back(w);
                 seeds.push_back(g->seed);
                 sids.push_back(c.sids);
                 sorders.push_back(g->d_sorder);
                 caps.push_back(step_cap_of(g));
+                qbits.push_back(kc_host::queue_bits(g->max_deg));
                 idx.push_back(i);
                 bs.push_back(B);
             }
             if (idx.empty()) break;
             const size_t G = idx.size();
-            // trees of different graphs interleaved, so a launch mixes sizes
-            std::vector<int2> entry;
-            int64_t most = 0;
-            for (int64_t b : bs) most = std::max(most, b);
-            for (int64_t t = 0; t < most; ++t)
-                for (size_t k = 0; k < G; ++k)
-                    if (t < bs[k]) entry.push_back(make_int2((int)k, (int)t));
-            const size_t bytes = sizeof(GraphView) * G + sizeof(WaveView) * G + 8 * G * 4 +
-                                 sizeof(int2) * entry.size() + 256 * 8;
-            kc_graph *g0 = gs[0];
-            KC_CK(g0, cudaMallocAsync(&d_tab, bytes, s0));
-            char *base = (char *)d_tab;
-            size_t off = 0;
-            auto put = [&](const void *src, size_t nb) {
-                void *dst = base + off;
-                KC_CK(g0, cudaMemcpyAsync(dst, src, nb, cudaMemcpyHostToDevice, s0));
-                off += (nb + 255) & ~size_t(255);
-                return dst;
-            };
-            MultiWalk mw;
-            mw.graphs = (const GraphView *)put(gv.data(), sizeof(GraphView) * G);
-            mw.waves = (const WaveView *)put(wv.data(), sizeof(WaveView) * G);
-            mw.seeds = (const uint64_t *)put(seeds.data(), 8 * G);
-            mw.sids = (const int64_t *const *)put(sids.data(), 8 * G);
-            mw.sorders = (const int32_t *const *)put(sorders.data(), 8 * G);
-            mw.step_caps = (const int64_t *)put(caps.data(), 8 * G);
-            mw.entry = (const int2 *)put(entry.data(), sizeof(int2) * entry.size());
-            mw.count = (int64_t)entry.size();
-            {
-                Phase ph(g0, g0->t_wilson);
-                KC_CK(g0, launch_wilson_warp_multi(mw, s0));
-                ph.done(1);
+            // graphs that run one walker per tree (k1_solo.cu) and graphs that run
+            // 32, a launch each: the former's trees longest first, so that no long
+            // tree starts last, the latter's interleaved, so that a launch mixes sizes
+            std::vector<char> solo(G);
+            for (size_t k = 0; k < G; ++k) solo[k] = use_solo(gs[idx[k]]) ? 1 : 0;
+            std::vector<size_t> by_work(G);
+            for (size_t k = 0; k < G; ++k) by_work[k] = k;
+            std::stable_sort(by_work.begin(), by_work.end(), [&](size_t x, size_t y) {
+                auto len = [&](size_t k) {  // long-diameter graphs walk ~8 times as far
+                    const kc_graph *g = gs[idx[k]];
+                    return g->n * (g->ttf_variant == KC_TTF_BIT ? 8 : 1);
+                };
+                return len(x) > len(y);
+            });
+            int64_t most = 0, total = 0;
+            for (int64_t b : bs) {
+                most = std::max(most, b);
+                total += b;
             }
-            KC_CK(g0, cudaFreeAsync(d_tab, s0));
-            d_tab = nullptr;
+            kc_graph *g0 = gs[0];
+            std::vector<int2> entry;
+            for (bool again = true; again;) {
+                std::vector<int2> e_warp;
+                entry.clear();
+                for (size_t k : by_work)
+                    for (int64_t t = 0; solo[k] && t < bs[k]; ++t)
+                        entry.push_back(make_int2((int)k, (int)t));
+                for (int64_t t = 0; t < most; ++t)
+                    for (size_t k = 0; k < G; ++k)
+                        if (!solo[k] && t < bs[k]) e_warp.push_back(make_int2((int)k, (int)t));
+                const int64_t n_solo = (int64_t)entry.size();
+                entry.insert(entry.end(), e_warp.begin(), e_warp.end());
+                for (size_t k = 0; k < G; ++k) {
+                    kc_graph *g = gs[idx[k]];
+                    KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), s0));
+                    if (solo[k])
+                        init_queues(g, gv[k], wv[k], sids[k], g->root, s0);
+                    else KC_CK(g, launch_wave_init(gv[k], wv[k], s0));
+                }
+                const size_t bytes = sizeof(GraphView) * G + sizeof(WaveView) * G + 8 * G * 5 +
+                                     sizeof(int2) * entry.size() + 256 * 8;
+                KC_CK(g0, cudaMallocAsync(&d_tab, bytes, s0));
+                char *base = (char *)d_tab;
+                size_t off = 0;
+                auto put = [&](const void *src, size_t nb) {
+                    void *dst = base + off;
+                    KC_CK(g0, cudaMemcpyAsync(dst, src, nb, cudaMemcpyHostToDevice, s0));
+                    off += (nb + 255) & ~size_t(255);
+                    return dst;
+                };
+                MultiWalk mw;
+                mw.graphs = (const GraphView *)put(gv.data(), sizeof(GraphView) * G);
+                mw.waves = (const WaveView *)put(wv.data(), sizeof(WaveView) * G);
+                mw.seeds = (const uint64_t *)put(seeds.data(), 8 * G);
+                mw.sids = (const int64_t *const *)put(sids.data(), 8 * G);
+                mw.sorders = (const int32_t *const *)put(sorders.data(), 8 * G);
+                mw.step_caps = (const int64_t *)put(caps.data(), 8 * G);
+                mw.queue_bits = (const int32_t *)put(qbits.data(), 4 * G);
+                mw.entry = (const int2 *)put(entry.data(), sizeof(int2) * entry.size());
+                {
+                    Phase ph(g0, g0->t_wilson);
+                    mw.count = n_solo;
+                    KC_CK(g0, launch_wilson_queue_multi(mw, s0));
+                    mw.entry += n_solo;
+                    mw.count = total - n_solo;
+                    KC_CK(g0, launch_wilson_warp_multi(mw, s0));
+                    ph.done((n_solo > 0 ? 1 : 0) + (n_solo < total ? 1 : 0));
+                }
+                KC_CK(g0, cudaFreeAsync(d_tab, s0));
+                d_tab = nullptr;
+                again = false;  // a graph whose count fields or step cap did not hold
+                for (size_t k = 0; k < G; ++k) {
+                    if (!solo[k]) continue;
+                    uint32_t err = 0;
+                    KC_CK(g0, copy_sync(g0, &err, gs[idx[k]]->d_err, sizeof(err),
+                                        cudaMemcpyDeviceToHost));
+                    if (!(err & (kErrCountField | kErrStepLimit))) continue;
+                    for (char &c : solo) c = 0;
+                    again = true;
+                    break;
+                }
+            }
             // per graph: walk errors, BIT stacks, sub-wave buffers zeroed; the
             // graphs whose wave is one sub-wave get one batched traversal and TTF
             // launch, the others their own launches
@@ -1886,8 +2003,11 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
         const cudaMemcpyKind kind = cfg.inputs_on_device ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost;
         KC_CK(g, copy_sync(g, g->h_row_off.data(), row_off, sizeof(int64_t) * (n + 1), kind));
         if (g->h_row_off[0] != 0) throw Fail{KC_ERR_INVALID_ARG};
-        for (int64_t v = 0; v < n; ++v)
-            if (g->h_row_off[v + 1] < g->h_row_off[v]) throw Fail{KC_ERR_INVALID_ARG};
+        for (int64_t v = 0; v < n; ++v) {
+            const int64_t d = g->h_row_off[v + 1] - g->h_row_off[v];
+            if (d < 0) throw Fail{KC_ERR_INVALID_ARG};
+            g->max_deg = std::max(g->max_deg, d);
+        }
         const int64_t twom = g->h_row_off[n];
         if (twom % 2 != 0 || twom == 0) throw Fail{twom == 0 ? KC_ERR_DISCONNECTED : KC_ERR_NOT_SYMMETRIC};
         g->m = twom / 2;
@@ -1998,6 +2118,7 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
             walker = (cfg.reject_steps > 0 && !cfg.autotune && variant == KC_TTF_BIT)
                          ? KC_WALK_LANE : KC_WALK_WARP;
         g->walker = walker;
+        g->auto_walker = cfg.walker == KC_WALK_AUTO && !cfg.autotune;
     } catch (Fail &f) {
         kc_graph_destroy(g);
         return f.st;

@@ -176,6 +176,10 @@ __host__ __device__ __forceinline__ uint64_t w_make(int32_t next, uint32_t count
 constexpr uint32_t kErrStepLimit = 1u;
 constexpr uint32_t kErrBadTree = 2u;
 constexpr uint32_t kErrIterLimit = 4u;
+constexpr uint32_t kErrCountField = 8u;  // k1_solo.cu: repeat the wave with k1_wilson.cu
+
+// departures of one vertex at which every sampler stops
+constexpr uint32_t kWalkCountMask = (1u << 25) - 1u;
 
 // ---------------------------------------------------------------------------
 // Device views
@@ -256,6 +260,7 @@ struct kc_graph {
     int device = 0;
     cudaStream_t stream = nullptr;
     int64_t n = 0, m = 0;
+    int64_t max_deg = 0;  // largest degree (an upper bound after deletions)
     // device graph
     int64_t *d_row_off = nullptr;
     int32_t *d_col = nullptr;
@@ -265,6 +270,7 @@ struct kc_graph {
     int32_t *d_p0 = nullptr, *d_level0 = nullptr, *d_in0 = nullptr, *d_out0 = nullptr;
     int32_t ttf_variant = KC_TTF_SCAN;
     int32_t walker = KC_WALK_WARP;
+    bool auto_walker = false;  // walker is AUTO's choice: a wave may run k1_solo.cu instead
     // host copy of the graph (validated CSR, needed by updates)
     std::vector<int64_t> h_row_off;
     std::vector<int32_t> h_col;
@@ -368,6 +374,7 @@ struct MultiWalk {
     const int64_t *const *sids = nullptr;
     const int32_t *const *sorders = nullptr;
     const int64_t *step_caps = nullptr;
+    const int32_t *queue_bits = nullptr;  // k1_solo.cu only
     const int2 *entry = nullptr;
     int64_t count = 0;
 };
@@ -410,6 +417,18 @@ __device__ __forceinline__ bool pick_tree(const MultiSub &ms, const GraphView &g
 cudaError_t launch_traverse_multi(const MultiSub &ms, cudaStream_t s);
 cudaError_t launch_ttf_scan_multi(const MultiSub &ms, int64_t max_n, cudaStream_t s);
 cudaError_t launch_ttf_bit_multi(const MultiSub &ms, cudaStream_t s);
+// k1_solo.cu: one walker per tree with the arrows drawn ahead into queues of
+// `bits`-bit neighbour indices (kc_host::queue_bits, at most kMaxQueueBits).
+// The wave's words are initialised by launch_queue_init, with up to first_slots
+// arrows a vertex (root < 0: no vertex is in the tree yet), instead of
+// launch_wave_init.  step_cap bounds a tree's departures: with reject a tree past
+// it gets steps = -1 (and done flag -1), otherwise kErrStepLimit.
+cudaError_t launch_queue_init(const GraphView &g, WaveView w, uint64_t seed, const int64_t *sids,
+                              int32_t root, int bits, int first_slots, cudaStream_t s);
+cudaError_t launch_wilson_queue(const GraphView &g, WaveView w, uint64_t seed,
+                                const int64_t *sids, int bits, int64_t step_cap, bool reject,
+                                int64_t num_sms, cudaStream_t s, int32_t *done_flag = nullptr);
+cudaError_t launch_wilson_queue_multi(const MultiWalk &mw, cudaStream_t s);
 cudaError_t launch_wilson(const GraphView &g, WaveView w, uint64_t seed, const int64_t *sids,
                           int64_t step_cap, cudaStream_t s, const int32_t *sorder = nullptr,
                           int32_t *rs_q = nullptr, int32_t *rs_pos = nullptr,
@@ -454,8 +473,10 @@ cudaError_t launch_words_from_parents(int64_t n, int64_t B, const int32_t *paren
                                       uint64_t *word, cudaStream_t s);
 
 // Sample maintenance (k6_update.cu) and effective resistance (k8_resistance.cu).
+// the edge (u, v) in the tree of every word array, u -> v; cleared: the other words
+// are zeroed first
 cudaError_t launch_edge_pre_init(int64_t n, int64_t B, int32_t u, int32_t v, uint64_t *word,
-                                 int32_t *ord, cudaStream_t s);
+                                 int32_t *ord, bool cleared, cudaStream_t s);
 cudaError_t launch_words_to_slots(int64_t n, int64_t B, const uint64_t *word, const int64_t *slot,
                                   int32_t *pool_parents, int32_t r, int32_t top, uint32_t *err,
                                   cudaStream_t s);

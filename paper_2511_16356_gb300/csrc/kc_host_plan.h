@@ -98,4 +98,28 @@ inline int64_t reject_wave_size(int64_t need, int64_t drawn, int64_t accepted, d
     return (int64_t)std::ceil(want + 3.0 * sd) + 8;
 }
 
+// Arrow queues of the one-walker kernels (k1_solo.cu): bits of a neighbour index
+// in a graph of largest degree max_deg, and how many arrows a queue of
+// kQueueWidth bits holds behind the last one taken and before its end mark.  At
+// most kMaxQueueBits bits leave room for one.
+constexpr int kQueueWidth = 17;
+constexpr int kMaxQueueBits = (kQueueWidth - 1) / 2;
+constexpr int queue_bits(int64_t max_deg) {
+    int b = 1;
+    while (b < 63 && ((int64_t)1 << b) < max_deg) ++b;
+    return b;
+}
+constexpr int queue_slots(int bits) { return (kQueueWidth - 1 - bits) / bits; }
+
+// Lanes per tree of those kernels for a wave of B trees (32, 16 or 8): one tree
+// per warp while all are resident (28 an SM), as it has the shortest chain per
+// departure; then as many trees per warp as make them resident (40 and 96 an
+// SM).  350x350 grid under a cap of 13 n departures, walk in ms for 32 / 16 / 8
+// lanes: 3044 trees 347 / 469 / 645, 4522 trees 549 / 508 / 666, 8929 trees
+// 904 / 975 / 726, 17672 trees 1579 / 1551 / 1423.
+inline int queue_group(int64_t B, int64_t num_sms) {
+    const int64_t per_sm = (B + std::max<int64_t>(num_sms, 1) - 1) / std::max<int64_t>(num_sms, 1);
+    return per_sm <= 28 ? 32 : (per_sm <= 40 ? 16 : 8);
+}
+
 }  // namespace kc_host

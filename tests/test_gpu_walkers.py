@@ -55,3 +55,39 @@ def test_segment_tables_survive_a_later_pipelined_wave(grid260):
         G.sample(5, 64)
         G.sample(5, 4)
         _check(grid260, G.samples(), 5, 0, 68)
+
+
+SMALL = {
+    "K2": lambda: S.complete(2), "K3": lambda: S.complete(3), "star40": lambda: S.star(40),
+    "cycle500": lambda: S.cycle(500),  # paths of more than 32 vertices are committed in chunks
+    "er300": lambda: S.er_lcc(300, 0.02, 7), "grid17x13": lambda: S.grid_perturbed(17, 13, 0.25, 3),
+    "cl3000": lambda: S.chung_lu(3000, 2.1, 8.0, 5),
+}
+
+
+@pytest.mark.parametrize("name,trees", [(k, 40) for k in SMALL] +
+                         [("K3", 100000), ("star40", 3000), ("er300", 5000),
+                          ("grid17x13", 9800), ("er300", 20000), ("grid17x13", 40000)])
+def test_arrows_drawn_ahead_match_oracle(name, trees):
+    """One walker per tree, one to 32 trees per warp (40 trees up to 40000)."""
+    g = SMALL[name]()
+    with kc.KemenyGraph.from_graph(g, _cfg(walker=kc.KC_WALK_LANE)) as G:
+        G.sample(17, trees)
+        _check(g, G.samples(), 17, 0, trees)
+
+
+@pytest.mark.parametrize("name,trees", [("cycle500", 64), ("grid17x13", 4000)])
+def test_arrows_drawn_ahead_reject_match_oracle(name, trees):
+    """Rejection by walk length, one tree and several trees per warp."""
+    g = SMALL[name]()
+    t0 = O.tau0(g)
+    _, st = O.sample_batch(g, t0, 23, 0, 256)
+    cap = int(np.quantile(st, 0.6))
+    ids, f_ref, st_ref = O.accepted_samples(lambda a, c: O.sample_batch(g, t0, 23, a, c), cap,
+                                            trees, block=2 * trees)
+    with kc.KemenyGraph.from_graph(g, _cfg(walker=kc.KC_WALK_LANE, reject_steps=cap)) as G:
+        G.sample(23, trees)
+        got = G.samples()
+    assert np.array_equal(got["sid"], ids)
+    assert np.array_equal(got["steps"], st_ref)
+    assert np.array_equal(got["f"], f_ref)
