@@ -35,20 +35,6 @@ constexpr uint32_t kQueue = (1u << kc_host::kQueueWidth) - 1u;
 constexpr uint32_t kOneMore = 1u << kc_host::kQueueWidth;  // one departure in the high half
 constexpr uint32_t kMostDepartures = (1u << (31 - kc_host::kQueueWidth)) - 1u;
 
-// neighbour number k of a record; kDeg4: the graph's degrees are at most 4
-template <bool kDeg4>
-__device__ __forceinline__ int32_t nbr_of(const VRec &r, uint32_t k,
-                                          const int32_t *__restrict__ col) {
-    if (!kDeg4 && k >= (uint32_t)kInline) {
-        const uint64_t off = (uint64_t)r.off_lo | ((uint64_t)r.off_hi << 32);
-        return col[off + k];
-    }
-    const int32_t lo = (k & 1u) ? r.nbr[1] : r.nbr[0];
-    const int32_t hi = (k & 1u) ? r.nbr[3] : r.nbr[2];
-    const int32_t x = (k & 2u) ? hi : lo;
-    return !kDeg4 && (k & 4u) ? r.nbr[4] : x;
-}
-
 // Words of every tree of the wave: the first `slots` arrows of each vertex, the
 // root (if any) in the tree.  A thread keeps one vertex's record for kInitTrees
 // trees.
@@ -331,16 +317,6 @@ __global__ void __launch_bounds__(32, kGroup == 32 ? 28 : (kGroup == 16 ? 20 : 2
         }
         __syncwarp();
     }
-}
-
-PhiloxKeys host_keys(uint64_t seed) {
-    PhiloxKeys K;
-    uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-    for (int i = 0; i < 10; ++i, k0 += kPhiloxW0, k1 += kPhiloxW1) {
-        K.k0[i] = k0;
-        K.k1[i] = k1;
-    }
-    return K;
 }
 
 }  // namespace

@@ -1,0 +1,265 @@
+// Spanning trees of low-diameter graphs by cycle popping, and f(tau) of each tree
+// in the same block (Sec. 2.2; Theorem 3).
+//
+// Wilson's algorithm pops the cycles of stacks of arrows (vertex u's k-th arrow is
+// bounded(seed, u, k, sample, WALK, deg u)); popping them in any order gives the
+// same tree and the same number of arrows.  Here a block takes a tree: every
+// vertex shows its first arrow, all cycles of that map are found and their
+// vertices shown their next arrows, and so on until none is left.  On a
+// low-diameter graph the first map holds most of the tree -- a random graph of
+// 2000 vertices pops about 0.5 n arrows in some 20 rounds, a power-law graph of a
+// million 0.09 n in 10 to 80 -- where a walk is a chain of n loads and more.
+//
+// A cycle is found by its leader, the smallest active vertex on it (active: its
+// arrow is new; every cycle holds one).  An active vertex a follows the arrows
+// until a settled vertex (one known to lead to the root: then so does a, and
+// its path is settled), an active vertex below a (which then leads, if anything
+// does), a itself, or an active vertex met before (Brent's rule: a cycle of larger
+// vertices that does not hold a).  Settled paths are never followed again, so all
+// rounds together settle each vertex once.
+//
+// k_pop_small keeps the tree in shared memory: 14 bytes a vertex.
+#include <algorithm>
+
+#include "kc_common.cuh"
+#include "kc_host_plan.h"
+
+namespace kc {
+
+namespace {
+
+constexpr unsigned kFull = 0xFFFFFFFFu;
+
+// Vertex word in shared memory: target (16 bits), pops (14), settled, active
+constexpr uint32_t kActive = 1u << 31;
+constexpr uint32_t kSettled = 1u << 30;
+constexpr uint32_t kTarget = 0xFFFFu;
+constexpr uint32_t kSmallMostPops = 0x3FFFu;
+
+// The length of the cycle that active vertex a leads, or 0 (see above).
+__device__ __forceinline__ uint32_t led_cycle(volatile uint32_t *nx, uint32_t a) {
+    uint32_t x = nx[a] & kTarget;
+    uint32_t saved = 0xFFFFFFFFu, met = 0, power = 1, len = 1;
+    for (;; ++len) {
+        const uint32_t w = nx[x];
+        if (w >= kSettled) {
+            if (w & kSettled) break;
+            if (x <= a) return x == a ? len : 0;
+            if (x == saved) return 0;
+            if (++met == power) {
+                saved = x;
+                power <<= 1;
+                met = 0;
+            }
+        }
+        x = w & kTarget;
+    }
+    // a leads to the root: settle its path (others may settle parts of it too)
+    x = a;
+    for (uint32_t w = nx[x]; !(w & kSettled); w = nx[x]) {
+        nx[x] = w | kSettled;
+        x = w & kTarget;
+    }
+    return 0;
+}
+
+template <int kThreads, bool kMulti>
+__global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 12 : (kThreads <= 256 ? 6 : 1))
+    k_pop_small(PopTask one, const PopTask *__restrict__ tasks, const int2 *__restrict__ entry) {
+    const int64_t t = kMulti ? (int64_t)entry[blockIdx.x].y : (int64_t)blockIdx.x;
+    const PopTask task = kMulti ? tasks[entry[blockIdx.x].x] : one;
+    const GraphView &g = task.g;
+    const uint32_t n = (uint32_t)g.n, root = (uint32_t)task.root;
+    const uint32_t sample = (uint32_t)task.sids[t];
+    const uint32_t tid = threadIdx.x;
+    const VRec *__restrict__ rec = g.rec;
+
+    extern __shared__ uint32_t smem[];
+    uint32_t *nx = smem;       // [n] the map
+    uint32_t *acc = smem + n;  // [n] the two lists of active vertices; then reports, jumps
+    uint32_t *vol = smem + 2 * n;
+    uint16_t *size = reinterpret_cast<uint16_t *>(smem + 3 * n);
+    uint16_t *list = reinterpret_cast<uint16_t *>(acc), *fresh = list + n;
+    __shared__ uint32_t s_count[2];
+    __shared__ unsigned long long s_f;
+
+    // arrow number `count` of v
+    auto arrow = [&](uint32_t v, uint32_t count) {
+        const VRec r = load_rec(rec + v);
+        const uint32_t k = bounded_draw_k(task.keys, task.seed, v, count, sample, kTagWalk,
+                                          (uint32_t)r.deg);
+        return (uint32_t)nbr_of<false>(r, k, g.col);
+    };
+    for (uint32_t v = tid; v < n; v += kThreads) {
+        uint32_t x = root | kSettled;
+        if (v != root && (int32_t)v != task.fixed) x = arrow(v, 0) | kActive;
+        nx[v] = x;
+    }
+    if (tid < 2) s_count[tid] = 0;
+    if (tid == 0) s_f = 0;
+    __syncthreads();
+
+    // ---- rounds: leaders list their cycles, the cycles' arrows are replaced
+    uint32_t active = n;  // round 0: every vertex
+    int64_t pops = 0;
+    int end = 0;
+    for (int round = 0;; ++round) {
+        for (uint32_t i = tid; i < active; i += kThreads) {
+            const uint32_t a = round == 0 ? i : list[i];
+            if (nx[a] & kSettled) continue;
+            const uint32_t len = led_cycle(nx, a);
+            if (len == 0) continue;
+            uint32_t x = a, at = atomicAdd(&s_count[round & 1], len);
+            do {
+                fresh[at++] = (uint16_t)x;
+                x = nx[x] & kTarget;
+            } while (x != a);
+        }
+        __syncthreads();
+        const uint32_t found = s_count[round & 1];
+        for (uint32_t i = tid; i < active; i += kThreads) {
+            const uint32_t a = round == 0 ? i : list[i];
+            nx[a] &= ~kActive;
+        }
+        if (tid == 0) s_count[(round + 1) & 1] = 0;
+        if (found == 0) break;
+        pops += found;
+        if (pops + (int64_t)n - task.placed > task.step_cap) {
+            end = kErrStepLimit;
+            break;
+        }
+        __syncthreads();
+        bool full = false;
+        for (uint32_t i = tid; i < found; i += kThreads) {
+            const uint32_t v = fresh[i];
+            const uint32_t c = ((nx[v] >> 16) & kSmallMostPops) + 1;
+            nx[v] = arrow(v, c) | (c << 16) | kActive;
+            full = full || c >= kSmallMostPops;
+        }
+        if (__syncthreads_or(full)) {
+            end = kErrCountField;
+            break;
+        }
+        active = found;
+        uint16_t *const swap = list;
+        list = fresh;
+        fresh = swap;
+    }
+    __syncthreads();
+    if (end) {  // uniform
+        if (tid == 0) {
+            atomicOr(task.err, (uint32_t)end);
+            task.steps[t] = -1;
+        }
+        return;
+    }
+    if (tid == 0) task.steps[t] = pops + (int64_t)n - task.placed;
+    if (task.par)
+        for (uint32_t v = tid; v < n; v += kThreads)
+            task.par[t * n + v] = v == root ? -1 : (int32_t)(nx[v] & kTarget);
+    if (!task.f) return;
+
+    // ---- sizes, volumes and preorder.  acc of a vertex: unreported children
+    // (high half) and sizes reported (low half); the child that reports last goes
+    // on with its parent.  After its own report it holds the vertex's preorder
+    // relative to an ancestor: offset (high half) and that ancestor (low half).
+    for (uint32_t v = tid; v < n; v += kThreads) {
+        acc[v] = 0;
+        vol[v] = (uint32_t)g.deg[v];
+    }
+    __syncthreads();
+    for (uint32_t v = tid; v < n; v += kThreads)
+        if (v != root) atomicAdd(&acc[nx[v] & kTarget], 1u << 16);
+    __syncthreads();
+    for (uint32_t v = tid; v < n; v += kThreads) {
+        if (*(volatile uint32_t *)&acc[v] != 0u) continue;  // has children
+        uint32_t x = v, sx = 1;
+        while (x != root) {
+            const uint32_t p = nx[x] & kTarget;
+            size[x] = (uint16_t)sx;
+            atomicAdd(&vol[p], *(volatile uint32_t *)&vol[x]);
+            __threadfence_block();
+            const uint32_t old = atomicAdd(&acc[p], sx - (1u << 16));
+            acc[x] = (((old & 0xFFFFu) + 1u) << 16) | p;
+            if ((old >> 16) != 1u) break;  // siblings still to report
+            __threadfence_block();
+            sx = 1u + (old & 0xFFFFu) + sx;
+            x = p;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) acc[root] = root;
+    __syncthreads();
+    // pointer jumping in place: a pair is read and written whole, and holds at
+    // any time
+    for (uint32_t v = tid; v < n; v += kThreads) {
+        volatile uint32_t *pairs = acc;
+        uint32_t p = pairs[v];
+        while ((p & kTarget) != root) {
+            const uint32_t q = pairs[p & kTarget];
+            p = (((p >> 16) + (q >> 16)) << 16) | (q & kTarget);
+            pairs[v] = p;
+        }
+    }
+    __syncthreads();
+
+    // ---- f: every vertex walks up tau0 (as k_ttf_scan)
+    long long contrib = 0;
+    for (uint32_t v = tid; v < n; v += kThreads) {
+        if (v == root) continue;
+        const uint32_t inv = acc[v] >> 16;
+        long long q = 0;
+        uint32_t x = v;
+        for (int it = 0; x != root && it <= g.ecc; ++it) {
+            const uint32_t p0x = (uint32_t)g.p0[x];
+            if ((nx[x] & kTarget) == p0x) {
+                if (inv - (acc[x] >> 16) < size[x]) q += g.twom - (int64_t)vol[x];
+            } else if (p0x != root && (nx[p0x] & kTarget) == x) {
+                if (inv - (acc[p0x] >> 16) < size[p0x]) q -= g.twom - (int64_t)vol[p0x];
+            }
+            x = p0x;
+        }
+        contrib += (long long)g.deg[v] * q;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) contrib += __shfl_down_sync(kFull, contrib, o);
+    if ((tid & 31) == 0 && contrib != 0) atomicAdd(&s_f, (unsigned long long)contrib);
+    __syncthreads();
+    if (tid == 0) task.f[t] = (int64_t)s_f;
+}
+
+template <int kThreads, bool kMulti>
+cudaError_t launch_small(const PopTask &one, const PopTask *tasks, const int2 *entry,
+                         int64_t blocks, int64_t max_n, cudaStream_t s) {
+    const size_t bytes = kc_host::pop_small_bytes(max_n);
+    const cudaError_t e = cudaFuncSetAttribute(k_pop_small<kThreads, kMulti>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)bytes);
+    if (e != cudaSuccess) return e;
+    k_pop_small<kThreads, kMulti><<<(unsigned)blocks, kThreads, bytes, s>>>(one, tasks, entry);
+    return cudaGetLastError();
+}
+
+template <bool kMulti>
+cudaError_t launch_small_any(const PopTask &one, const PopTask *tasks, const int2 *entry,
+                             int64_t blocks, int64_t max_n, cudaStream_t s) {
+    if (blocks <= 0) return cudaSuccess;
+    switch (kc_host::pop_small_threads(max_n)) {
+        case 128: return launch_small<128, kMulti>(one, tasks, entry, blocks, max_n, s);
+        case 256: return launch_small<256, kMulti>(one, tasks, entry, blocks, max_n, s);
+        default: return launch_small<1024, kMulti>(one, tasks, entry, blocks, max_n, s);
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_pop_small(const PopTask &task, int64_t B, cudaStream_t s) {
+    return launch_small_any<false>(task, nullptr, nullptr, B, task.g.n, s);
+}
+
+cudaError_t launch_pop_small_multi(const PopTask *tasks, const int2 *entry, int64_t count,
+                                   int64_t max_n, cudaStream_t s) {
+    return launch_small_any<true>(PopTask{}, tasks, entry, count, max_n, s);
+}
+
+}  // namespace kc

@@ -29,13 +29,14 @@ __global__ void k_edge_pre_init(int64_t n, int64_t B, int32_t u, int32_t v, uint
     ord[t * n + 1] = u;
 }
 
-// dst[slot[t]][x] = parent of x in wave tree t
-__global__ void k_words_to_slots(int64_t n, int64_t B, const uint64_t *word, const int64_t *slot,
-                                 int32_t *pool_parents) {
+// dst[slot[t]][x] = parent of x in wave tree t, from its words or (word null) its
+// parent array
+__global__ void k_words_to_slots(int64_t n, int64_t B, const uint64_t *word, const int32_t *par,
+                                 const int64_t *slot, int32_t *pool_parents) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= B * n) return;
     const int64_t t = k / n, x = k - t * n;
-    pool_parents[slot[t] * n + x] = w_next(word[k]);
+    pool_parents[slot[t] * n + x] = word ? w_next(word[k]) : par[k];
 }
 
 // reverse the parent chain from r up to the old root `top` in each slot tree
@@ -488,10 +489,10 @@ cudaError_t launch_edge_pre_init(int64_t n, int64_t B, int32_t u, int32_t v, uin
     return cudaGetLastError();
 }
 
-cudaError_t launch_words_to_slots(int64_t n, int64_t B, const uint64_t *word, const int64_t *slot,
-                                  int32_t *pool_parents, int32_t r, int32_t top, uint32_t *err,
-                                  cudaStream_t s) {
-    k_words_to_slots<<<blk(B * n, 256), 256, 0, s>>>(n, B, word, slot, pool_parents);
+cudaError_t launch_words_to_slots(int64_t n, int64_t B, const uint64_t *word, const int32_t *par,
+                                  const int64_t *slot, int32_t *pool_parents, int32_t r,
+                                  int32_t top, uint32_t *err, cudaStream_t s) {
+    k_words_to_slots<<<blk(B * n, 256), 256, 0, s>>>(n, B, word, par, slot, pool_parents);
     if (top >= 0) k_reroot_slots<<<blk(B, 128), 128, 0, s>>>(n, B, slot, pool_parents, r, top, err);
     return cudaGetLastError();
 }

@@ -382,6 +382,42 @@ bool use_solo(const kc_graph *g) {
            g->ttf_variant == KC_TTF_BIT;
 }
 
+// Whether AUTO draws the trees of a low-diameter graph by cycle popping in shared
+// memory (k4_pop.cu), which also evaluates f.
+bool use_pop(const kc_graph *g) {
+    if (g->walker != KC_WALK_WARP || !g->auto_walker || g->ttf_variant != KC_TTF_SCAN ||
+        2 * g->m >= ((int64_t)1 << 32))
+        return false;
+    const int64_t root_deg = g->h_row_off[(size_t)g->root + 1] - g->h_row_off[(size_t)g->root];
+    return kc_host::pop_small(g->n, 2 * g->m, root_deg);
+}
+
+// The trees of wave w (sample ids c.sids): steps, and f unless they are only to be
+// stored (store: their parents, [w.B][n]).  fixed >= 0: the trees hold the edge
+// (fixed, root) and are rooted at `root`.
+PopTask pop_task(const kc_graph *g, const GraphView &gv, const WaveView &w, const int64_t *sids,
+                 int32_t root, int32_t fixed, bool want_f, int32_t *store) {
+    PopTask k;
+    k.g = gv;
+    k.root = root;
+    k.fixed = fixed;
+    k.placed = fixed >= 0 ? 2 : 1;
+    k.seed = g->seed;
+    k.keys = host_keys(g->seed);
+    k.step_cap = step_cap_of(g);
+    k.sids = sids;
+    k.steps = w.steps;
+    k.f = want_f ? w.f : nullptr;
+    k.par = store;
+    k.err = w.err;
+    return k;
+}
+
+// Where the parents of the next B trees of the pool go when trees are kept.
+int32_t *pool_slot(const kc_graph *g) {
+    return g->cfg.keep_trees ? g->d_parents + g->pool * g->n : nullptr;
+}
+
 // Words of k1_solo.cu with the arrow queues of `root`'s trees (-1: no vertex in
 // the tree).  A long-diameter graph departs a dozen times from a vertex, the
 // others once or twice: their first queues stay short.
@@ -623,7 +659,26 @@ bool run_wave_pipelined(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool reje
     return true;
 }
 
-void run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = false) {
+// Returns whether the trees' parents are in the pool already (k4_pop.cu).
+bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = false) {
+    if (!canonical && !g->tuning && use_pop(g)) {
+        const Carved c = carve(g, p);
+        WaveView w = c.wv;
+        w.B = B;
+        KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
+        KC_CK(g, launch_iota(c.sids, sid0, B, g->stream));
+        {
+            Phase ph(g, g->t_wilson);
+            KC_CK(g, launch_pop_small(pop_task(g, view_of(g), w, c.sids, g->root, -1, true,
+                                               pool_slot(g)),
+                                      B, g->stream));
+            ph.done(1);
+        }
+        uint32_t err = 0;
+        KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
+        if (!err) return true;
+        if (!solo_retry(g, err)) throw Fail{KC_ERR_CUDA};
+    }
     // pipelining pays when traversal and TTF take long enough to hide: several
     // sub-waves, or large graphs; short waves of small graphs run straight
     if (!canonical && !g->tuning && (g->walker == KC_WALK_WARP || g->walker == KC_WALK_LANE) &&
@@ -638,7 +693,7 @@ void run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
             if (g->stream2) cudaStreamSynchronize(g->stream2);
             throw;
         }
-        return;
+        return false;
     }
     GraphView gv = view_of(g);
     Carved c = carve(g, p);
@@ -704,6 +759,7 @@ void run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
         g->last_error = "inconsistent tree state or traversal stack overflow";
         throw Fail{KC_ERR_CUDA};
     }
+    return false;
 }
 
 
@@ -1110,7 +1166,18 @@ void resample_slots(kc_graph *g, const std::vector<int64_t> &slots, bool cond, i
         w.B = b;
         w.pos0 = cond ? 2 : 1;
         KC_CK(g, launch_iota(c.sids, g->next_sid, b, g->stream));
-        for (bool solo = use_solo(g);; solo = false) {
+        bool pop = use_pop(g);
+        if (pop) {
+            KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
+            KC_CK(g, launch_pop_small(pop_task(g, gv, w, c.sids, cond ? v : g->root,
+                                               cond ? u : -1, false, w.ord),
+                                      b, g->stream));
+            g->t_update.launches += 1;
+            uint32_t err = 0;
+            KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
+            pop = !solo_retry(g, err);
+        }
+        for (bool solo = use_solo(g); !pop; solo = false) {
             KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
             if (cond) {
                 if (solo) init_queues(g, gv, w, c.sids, -1, g->stream);
@@ -1125,8 +1192,9 @@ void resample_slots(kc_graph *g, const std::vector<int64_t> &slots, bool cond, i
             KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
             if (!solo_retry(g, err)) break;
         }
-        KC_CK(g, launch_words_to_slots(g->n, b, w.word, ub.slots, g->d_parents, g->root,
-                                       cond ? v : -1, g->d_err, g->stream));
+        KC_CK(g, launch_words_to_slots(g->n, b, pop ? nullptr : w.word, w.ord, ub.slots,
+                                       g->d_parents, g->root, cond ? v : -1, g->d_err,
+                                       g->stream));
         KC_CK(g, launch_scatter_results(ub.slots, b, nullptr, w.steps, c.sids, g->d_f,
                                         g->d_steps, g->d_sid, g->stream));
         check_err(g, "resample");
@@ -1312,16 +1380,16 @@ PoolSums reduce_pool(kc_graph *g) {
 
 // One wave of B trees appended to the pool.
 void sample_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0) {
-    run_wave(g, p, B, sid0);
+    const bool stored = run_wave(g, p, B, sid0);
     Carved c = carve(g, p);
     WaveView w = c.wv;
     w.B = B;
     {
         Phase ph(g, g->t_reduce);
+        const bool words = g->cfg.keep_trees && !stored;
         KC_CK(g, launch_pool_append(w, g->pool, g->d_f, g->d_w, g->d_steps, g->d_sid, c.sids,
-                                    g->cfg.keep_trees ? g->d_parents : nullptr, g->n,
-                                    g->stream));
-        ph.done(g->cfg.keep_trees ? 2 : 1);
+                                    words ? g->d_parents : nullptr, g->n, g->stream));
+        ph.done(words ? 2 : 1);
     }
     for (int64_t k = 0; k < B; ++k) g->h_modified[(size_t)(g->pool + k)] = 0;
     g->pool += B;
@@ -1650,11 +1718,15 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
             }
             if (idx.empty()) break;
             const size_t G = idx.size();
-            // graphs that run one walker per tree (k1_solo.cu) and graphs that run
-            // 32, a launch each: the former's trees longest first, so that no long
-            // tree starts last, the latter's interleaved, so that a launch mixes sizes
-            std::vector<char> solo(G);
-            for (size_t k = 0; k < G; ++k) solo[k] = use_solo(gs[idx[k]]) ? 1 : 0;
+            // graphs whose trees a block each pops (k4_pop.cu, a launch for each block
+            // size), graphs that run one walker per tree (k1_solo.cu) and graphs that
+            // run 32, a launch each: longest trees first, so that none starts last, the
+            // last kind's interleaved, so that a launch mixes sizes
+            std::vector<char> solo(G), pop(G);
+            for (size_t k = 0; k < G; ++k) {
+                solo[k] = use_solo(gs[idx[k]]) ? 1 : 0;
+                pop[k] = use_pop(gs[idx[k]]) ? 1 : 0;
+            }
             std::vector<size_t> by_work(G);
             for (size_t k = 0; k < G; ++k) by_work[k] = k;
             std::stable_sort(by_work.begin(), by_work.end(), [&](size_t x, size_t y) {
@@ -1664,33 +1736,47 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                 };
                 return len(x) > len(y);
             });
-            int64_t most = 0, total = 0;
-            for (int64_t b : bs) {
-                most = std::max(most, b);
-                total += b;
-            }
+            int64_t most = 0;
+            for (int64_t b : bs) most = std::max(most, b);
             kc_graph *g0 = gs[0];
             std::vector<int2> entry;
             for (bool again = true; again;) {
-                std::vector<int2> e_warp;
+                struct PopClass {
+                    int64_t first, count, max_n;
+                };
+                std::vector<PopClass> classes;
+                std::vector<PopTask> tasks(G);
                 entry.clear();
+                for (size_t k : by_work) {  // largest first: classes are contiguous
+                    kc_graph *g = gs[idx[k]];
+                    if (!pop[k]) continue;
+                    tasks[k] = pop_task(g, gv[k], wv[k], sids[k], g->root, -1, true,
+                                        pool_slot(g));
+                    if (classes.empty() || kc_host::pop_small_threads(classes.back().max_n) !=
+                                               kc_host::pop_small_threads(g->n))
+                        classes.push_back({(int64_t)entry.size(), 0, g->n});
+                    classes.back().count += bs[k];
+                    for (int64_t t = 0; t < bs[k]; ++t) entry.push_back(make_int2((int)k, (int)t));
+                }
+                const int64_t n_pop = (int64_t)entry.size();
                 for (size_t k : by_work)
                     for (int64_t t = 0; solo[k] && t < bs[k]; ++t)
                         entry.push_back(make_int2((int)k, (int)t));
+                const int64_t n_solo = (int64_t)entry.size() - n_pop;
                 for (int64_t t = 0; t < most; ++t)
                     for (size_t k = 0; k < G; ++k)
-                        if (!solo[k] && t < bs[k]) e_warp.push_back(make_int2((int)k, (int)t));
-                const int64_t n_solo = (int64_t)entry.size();
-                entry.insert(entry.end(), e_warp.begin(), e_warp.end());
+                        if (!solo[k] && !pop[k] && t < bs[k])
+                            entry.push_back(make_int2((int)k, (int)t));
+                const int64_t n_warp = (int64_t)entry.size() - n_pop - n_solo;
                 for (size_t k = 0; k < G; ++k) {
                     kc_graph *g = gs[idx[k]];
                     KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), s0));
-                    if (solo[k])
-                        init_queues(g, gv[k], wv[k], sids[k], g->root, s0);
+                    if (pop[k]) continue;
+                    if (solo[k]) init_queues(g, gv[k], wv[k], sids[k], g->root, s0);
                     else KC_CK(g, launch_wave_init(gv[k], wv[k], s0));
                 }
-                const size_t bytes = sizeof(GraphView) * G + sizeof(WaveView) * G + 8 * G * 5 +
-                                     sizeof(int2) * entry.size() + 256 * 8;
+                const size_t bytes = (sizeof(GraphView) + sizeof(WaveView) + sizeof(PopTask)) * G +
+                                     8 * G * 5 + sizeof(int2) * entry.size() + 256 * 9;
                 KC_CK(g0, cudaMallocAsync(&d_tab, bytes, s0));
                 char *base = (char *)d_tab;
                 size_t off = 0;
@@ -1708,26 +1794,32 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                 mw.sorders = (const int32_t *const *)put(sorders.data(), 8 * G);
                 mw.step_caps = (const int64_t *)put(caps.data(), 8 * G);
                 mw.queue_bits = (const int32_t *)put(qbits.data(), 4 * G);
+                const PopTask *d_tasks = (const PopTask *)put(tasks.data(), sizeof(PopTask) * G);
                 mw.entry = (const int2 *)put(entry.data(), sizeof(int2) * entry.size());
                 {
                     Phase ph(g0, g0->t_wilson);
+                    for (const PopClass &c : classes)
+                        KC_CK(g0, launch_pop_small_multi(d_tasks, mw.entry + c.first, c.count,
+                                                         c.max_n, s0));
+                    mw.entry += n_pop;
                     mw.count = n_solo;
                     KC_CK(g0, launch_wilson_queue_multi(mw, s0));
                     mw.entry += n_solo;
-                    mw.count = total - n_solo;
+                    mw.count = n_warp;
                     KC_CK(g0, launch_wilson_warp_multi(mw, s0));
-                    ph.done((n_solo > 0 ? 1 : 0) + (n_solo < total ? 1 : 0));
+                    ph.done((int)classes.size() + (n_solo > 0 ? 1 : 0) + (n_warp > 0 ? 1 : 0));
                 }
                 KC_CK(g0, cudaFreeAsync(d_tab, s0));
                 d_tab = nullptr;
                 again = false;  // a graph whose count fields or step cap did not hold
                 for (size_t k = 0; k < G; ++k) {
-                    if (!solo[k]) continue;
+                    if (!solo[k] && !pop[k]) continue;
                     uint32_t err = 0;
                     KC_CK(g0, copy_sync(g0, &err, gs[idx[k]]->d_err, sizeof(err),
                                         cudaMemcpyDeviceToHost));
                     if (!(err & (kErrCountField | kErrStepLimit))) continue;
                     for (char &c : solo) c = 0;
+                    for (char &c : pop) c = 0;
                     again = true;
                     break;
                 }
@@ -1754,6 +1846,7 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                 if (hdr[0]) throw Fail{KC_ERR_CUDA};
                 if (p.bit) ensure_stack(g, p, hdr[1]);
                 cv[k] = carve(g, p);
+                if (pop[k]) continue;  // f is there
                 WaveView w = cv[k].wv;
                 w.B = B;
                 const GraphView v = view_of(g);
@@ -1834,7 +1927,8 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                 WaveView w = cv[k].wv;
                 w.B = B;
                 KC_CK(g, launch_pool_append(w, g->pool, g->d_f, g->d_w, g->d_steps, g->d_sid,
-                                            cv[k].sids, g->cfg.keep_trees ? g->d_parents : nullptr,
+                                            cv[k].sids,
+                                            g->cfg.keep_trees && !pop[k] ? g->d_parents : nullptr,
                                             g->n, s0));
                 uint32_t hdr[2] = {0, 0};
                 KC_CK(g, copy_sync(g, hdr, g->d_err, sizeof(hdr), cudaMemcpyDeviceToHost));

@@ -63,6 +63,16 @@ __device__ __forceinline__ PhiloxKeys philox_keys(uint64_t seed) {
     }
     return K;
 }
+// the same on the host, for kernel arguments
+inline PhiloxKeys host_keys(uint64_t seed) {
+    PhiloxKeys K;
+    uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    for (int i = 0; i < 10; ++i, k0 += kPhiloxW0, k1 += kPhiloxW1) {
+        K.k0[i] = k0;
+        K.k1[i] = k1;
+    }
+    return K;
+}
 // philox4x32_10 with the round keys precomputed
 __device__ __forceinline__ void philox4x32_10_k(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                                                 const PhiloxKeys &K, uint32_t out[4]) {
@@ -152,6 +162,21 @@ __device__ __forceinline__ VRec load_rec(const VRec *p) {
     r.nbr[3] = (int32_t)b.z;
     r.nbr[4] = (int32_t)b.w;
     return r;
+}
+
+// neighbour number k of a record by a select, the column array from the inlined
+// ones on; kDeg4: the graph's degrees are at most 4
+template <bool kDeg4>
+__device__ __forceinline__ int32_t nbr_of(const VRec &r, uint32_t k,
+                                          const int32_t *__restrict__ col) {
+    if (!kDeg4 && k >= (uint32_t)kInline) {
+        const uint64_t off = (uint64_t)r.off_lo | ((uint64_t)r.off_hi << 32);
+        return col[off + k];
+    }
+    const int32_t lo = (k & 1u) ? r.nbr[1] : r.nbr[0];
+    const int32_t hi = (k & 1u) ? r.nbr[3] : r.nbr[2];
+    const int32_t x = (k & 2u) ? hi : lo;
+    return !kDeg4 && (k & 4u) ? r.nbr[4] : x;
 }
 
 // ---------------------------------------------------------------------------
@@ -429,6 +454,26 @@ cudaError_t launch_wilson_queue(const GraphView &g, WaveView w, uint64_t seed,
                                 const int64_t *sids, int bits, int64_t step_cap, bool reject,
                                 int64_t num_sms, cudaStream_t s, int32_t *done_flag = nullptr);
 cudaError_t launch_wilson_queue_multi(const MultiWalk &mw, cudaStream_t s);
+// k4_pop.cu: cycle popping, a block per tree.
+struct PopTask {
+    GraphView g;
+    int32_t root;             // root of the trees (g.root, or the head of a fixed edge)
+    int32_t fixed;            // >= 0: vertex whose arrow is the root and never drawn
+    int32_t placed;           // vertices that draw no arrow: 1, with a fixed edge 2
+    uint64_t seed;
+    PhiloxKeys keys;          // of the seed
+    int64_t step_cap;         // departures of a tree past which it fails (kErrStepLimit)
+    const int64_t *sids;      // [B]
+    int64_t *steps;           // [B]
+    int64_t *f;               // [B], or null: trees only
+    int32_t *par;             // [B][n] parents (-1 at the root), or null
+    uint32_t *err;
+};
+// n at most kc_host::kPopSmallMax, 2m < 2^32: trees and f from shared memory
+cudaError_t launch_pop_small(const PopTask &task, int64_t B, cudaStream_t s);
+// entries (task, tree) of a device table of tasks; max_n: their largest n
+cudaError_t launch_pop_small_multi(const PopTask *tasks, const int2 *entry, int64_t count,
+                                   int64_t max_n, cudaStream_t s);
 cudaError_t launch_wilson(const GraphView &g, WaveView w, uint64_t seed, const int64_t *sids,
                           int64_t step_cap, cudaStream_t s, const int32_t *sorder = nullptr,
                           int32_t *rs_q = nullptr, int32_t *rs_pos = nullptr,
@@ -477,9 +522,11 @@ cudaError_t launch_words_from_parents(int64_t n, int64_t B, const int32_t *paren
 // are zeroed first
 cudaError_t launch_edge_pre_init(int64_t n, int64_t B, int32_t u, int32_t v, uint64_t *word,
                                  int32_t *ord, bool cleared, cudaStream_t s);
-cudaError_t launch_words_to_slots(int64_t n, int64_t B, const uint64_t *word, const int64_t *slot,
-                                  int32_t *pool_parents, int32_t r, int32_t top, uint32_t *err,
-                                  cudaStream_t s);
+// parents of wave trees into pool slots, from their words or (word null) from the
+// parent arrays par; top >= 0: re-rooted from top to r
+cudaError_t launch_words_to_slots(int64_t n, int64_t B, const uint64_t *word, const int32_t *par,
+                                  const int64_t *slot, int32_t *pool_parents, int32_t r,
+                                  int32_t top, uint32_t *err, cudaStream_t s);
 cudaError_t launch_contains_edge(int64_t n, int64_t P, const int32_t *pool_parents, int32_t u,
                                  int32_t v, uint8_t *flag, cudaStream_t s);
 cudaError_t launch_select(uint64_t seed, uint32_t seq, int64_t N, int64_t k, uint8_t *taken,

@@ -122,4 +122,20 @@ inline int queue_group(int64_t B, int64_t num_sms) {
     return per_sm <= 28 ? 32 : (per_sm <= 40 ? 16 : 8);
 }
 
+// Cycle popping in shared memory (k_pop_small): its bytes for n vertices (two
+// words, a volume and a 16-bit size each; vertex ids are 16 bits), the largest n
+// (227 KB a block, less its static part) and the threads of a block.
+constexpr size_t pop_small_bytes(int64_t n) { return (size_t)n * 12 + ((size_t)n * 2 + 3) / 4 * 4; }
+constexpr int64_t kPopSmallMax = 16000;
+// Whether popping pays: its rounds follow the longest loops, which are long where
+// the first walk is -- the walk to the root takes about 2m / deg(root) departures.
+// Power-law graphs (a hub as the root): 10000 vertices, 500 trees 5.26 -> 1.27 ms
+// against 32 walkers and their traversal.  Sparse random graphs: 2000 vertices,
+// 2000 trees 3.9 -> 3.5 ms, even at 15000 vertices (24.0 / 23.8 ms) and behind when
+// blocks of many sizes share a call.
+inline bool pop_small(int64_t n, int64_t twom, int64_t root_deg) {
+    return n <= kPopSmallMax && (n <= 4096 || 16 * (twom / std::max<int64_t>(root_deg, 1)) <= n);
+}
+inline int pop_small_threads(int64_t n) { return n <= 1024 ? 128 : (n <= 4096 ? 256 : 1024); }
+
 }  // namespace kc_host

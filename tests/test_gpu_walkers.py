@@ -91,3 +91,30 @@ def test_arrows_drawn_ahead_reject_match_oracle(name, trees):
     assert np.array_equal(got["sid"], ids)
     assert np.array_equal(got["steps"], st_ref)
     assert np.array_equal(got["f"], f_ref)
+
+
+@pytest.mark.parametrize("n", [2, 3, 31, 33, 1024, 1025, 4096, 4097, 16000, 16001])
+def test_popped_trees_match_oracle(n):
+    """Cycle popping in shared memory (up to 16000 vertices; past them the walkers),
+    at the edges of its block sizes: f, step counts and a kept tree."""
+    g = S.complete(n) if n < 4 else S.complete_bipartite(min(25, n // 2), n - min(25, n // 2))
+    t0 = O.tau0(g)
+    with kc.KemenyGraph.from_graph(g, _cfg(keep_trees=1)) as G:
+        G.sample(41, 20)
+        G.sample(41, 13)
+        _check(g, G.samples(), 41, 0, 33)
+        for k in (0, 32):
+            tr, ref = G.tree(k), O.tree(g, t0, 41, k)
+            for key in ("parent", "depth", "din", "dout", "vol"):
+                assert np.array_equal(tr[key], getattr(ref, key)), key
+
+
+def test_popped_trees_at_the_step_cap():
+    """A tree past the cap is left to the 32-walker kernel, whose cap is per walker."""
+    g = SMALL["er300"]()
+    with kc.KemenyGraph.from_graph(g, _cfg(step_cap=400)) as G:  # S is about 540
+        G.sample(3, 40)
+        _check(g, G.samples(), 3, 0, 40)
+    with kc.KemenyGraph.from_graph(g, _cfg(step_cap=5)) as G:
+        st = kc.kc_sample(G.h, 3, 40, check=False)
+        assert kc.STATUS[st] == "KC_ERR_STEP_LIMIT"

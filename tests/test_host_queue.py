@@ -1,5 +1,5 @@
-"""Arrow queues of the one-walker kernels (csrc/kc_host_plan.h), compiled with the
-host C++ compiler."""
+"""Arrow queues of the one-walker kernels and block shapes of cycle popping
+(csrc/kc_host_plan.h), compiled with the host C++ compiler."""
 import ctypes
 import os
 import shutil
@@ -16,6 +16,10 @@ extern "C" int hq_bits(int64_t d) { return kc_host::queue_bits(d); }
 extern "C" int hq_slots(int b) { return kc_host::queue_slots(b); }
 extern "C" int hq_group(int64_t B, int64_t sms) { return kc_host::queue_group(B, sms); }
 extern "C" int hq_max_bits() { return kc_host::kMaxQueueBits; }
+extern "C" uint64_t hq_pop_bytes(int64_t n) { return kc_host::pop_small_bytes(n); }
+extern "C" int hq_pop_threads(int64_t n) { return kc_host::pop_small_threads(n); }
+extern "C" int hq_pop(int64_t n, int64_t twom, int64_t d) { return kc_host::pop_small(n, twom, d); }
+extern "C" int64_t hq_pop_max() { return kc_host::kPopSmallMax; }
 extern "C" int hq_width() { return kc_host::kQueueWidth; }
 """
 
@@ -32,6 +36,11 @@ def queue(tmp_path_factory):
     lib = ctypes.CDLL(str(d / "shim.so"))
     lib.hq_bits.argtypes = [ctypes.c_int64]
     lib.hq_group.argtypes = [ctypes.c_int64, ctypes.c_int64]
+    lib.hq_pop_bytes.restype = ctypes.c_uint64
+    lib.hq_pop_max.restype = ctypes.c_int64
+    for f in (lib.hq_pop_bytes, lib.hq_pop_threads):
+        f.argtypes = [ctypes.c_int64]
+    lib.hq_pop.argtypes = [ctypes.c_int64] * 3
     return lib
 
 
@@ -50,3 +59,15 @@ def test_arrow_queues_fit_their_words(queue):
 def test_every_wave_size_has_a_group(queue):
     got = [queue.hq_group(B, 152) for B in range(1, 20000)]
     assert set(got) == {32, 16, 8} and got == sorted(got, reverse=True)
+
+
+def test_popped_trees_fit_a_block(queue):
+    """14 bytes a vertex within 227 KB less the static part, ids in 16 bits."""
+    top = queue.hq_pop_max()
+    assert top < 1 << 16 and queue.hq_pop_bytes(top) + 64 <= 227 * 1024
+    for n in (2, 3, 1024, 1025, 4096, 4097, top):
+        assert 14 * n <= queue.hq_pop_bytes(n) <= 14 * n + 2
+        assert queue.hq_pop_threads(n) in (128, 256, 1024)
+        assert queue.hq_pop(n, 10 * n, n - 1)
+    assert not queue.hq_pop(top + 1, 10 * top, top)
+    assert not queue.hq_pop(8000, 64000, 20) and queue.hq_pop(4000, 32000, 20)
