@@ -31,8 +31,10 @@ namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-template <bool kMulti>
-__global__ void __launch_bounds__(256) k_ttf_scan(GraphView g_in, WaveView w_in, MultiSub ms) {
+// kPar: parents from their arrays, else from the walker words
+template <bool kMulti, bool kPar>
+__global__ void __launch_bounds__(256) k_ttf_scan(GraphView g_in, WaveView w_in, MultiSub ms,
+                                                  ParTrees trees) {
     GraphView g;
     WaveView w;
     int64_t t;
@@ -40,6 +42,8 @@ __global__ void __launch_bounds__(256) k_ttf_scan(GraphView g_in, WaveView w_in,
     const int64_t n = g.n;
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t *__restrict__ word = w.word + wave_tree(w, t) * n;
+    const int32_t *__restrict__ par = kPar ? trees.par + (trees.slot ? trees.slot[t] : t) * n
+                                           : nullptr;
     const int32_t *__restrict__ din = w.din + t * n;
     const int32_t *__restrict__ size = w.size + t * n;
     const int64_t *__restrict__ vol = w.vol + t * n;
@@ -52,11 +56,11 @@ __global__ void __launch_bounds__(256) k_ttf_scan(GraphView g_in, WaveView w_in,
         int32_t x = (int32_t)v;
         for (int it = 0; x != r && it <= g.ecc; ++it) {
             const int32_t p0x = g.p0[x];
-            const int32_t px = w_next(word[x]);
+            const int32_t px = kPar ? par[x] : w_next(word[x]);
             if (px == p0x) {
                 const int32_t inx = din[x];
                 if (inx <= inv && inv <= inx + size[x] - 1) q += twom - vol[x];
-            } else if (p0x != r && w_next(word[p0x]) == x) {
+            } else if (p0x != r && (kPar ? par[p0x] : w_next(word[p0x])) == x) {
                 const int32_t inw = din[p0x];
                 if (inw <= inv && inv <= inw + size[p0x] - 1) q -= twom - vol[p0x];
             }
@@ -354,7 +358,16 @@ cudaError_t launch_ttf_scan(const GraphView &g, WaveView w, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)((g.n + 255) / 256), (unsigned)w.B);
-    k_ttf_scan<false><<<grid, 256, 0, s>>>(g, w, MultiSub{});
+    k_ttf_scan<false, false><<<grid, 256, 0, s>>>(g, w, MultiSub{}, ParTrees{});
+    return cudaGetLastError();
+}
+
+cudaError_t launch_ttf_scan_parents(const GraphView &g, WaveView w, ParTrees trees,
+                                    cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(w.f, 0, sizeof(int64_t) * (size_t)w.B, s);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)((g.n + 255) / 256), (unsigned)w.B);
+    k_ttf_scan<false, true><<<grid, 256, 0, s>>>(g, w, MultiSub{}, trees);
     return cudaGetLastError();
 }
 
@@ -381,7 +394,7 @@ cudaError_t launch_ttf_scan_multi(const MultiSub &ms, int64_t max_n, cudaStream_
         part.entry = ms.entry + r0;
         part.count = std::min<int64_t>(65535, ms.count - r0);
         dim3 grid((unsigned)((max_n + 255) / 256), (unsigned)part.count);
-        k_ttf_scan<true><<<grid, 256, 0, s>>>(GraphView{}, WaveView{}, part);
+        k_ttf_scan<true, false><<<grid, 256, 0, s>>>(GraphView{}, WaveView{}, part, ParTrees{});
     }
     return cudaGetLastError();
 }

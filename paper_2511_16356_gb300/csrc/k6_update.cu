@@ -7,10 +7,12 @@
 //  - preparation of retained trees for the traversal passes: children lists,
 //    then a warp-per-tree breadth-first pass giving depths and a parent-first
 //    order;
-//  - link-cut (ISM insertion) and cut-link (ISM deletion), one warp per tree;
+//  - link-cut (ISM insertion) and cut-link (ISM deletion);
 //  - weight rescaling with sums in a fixed order (bit-reproducible).
 // The random choices follow the oracle's contract: tags select / link-cut /
 // cut-link with counters (update seq, draw index or pool index, 0).
+#include <algorithm>
+
 #include "kc_common.cuh"
 
 namespace kc {
@@ -179,18 +181,26 @@ __global__ void __launch_bounds__(128) k_bfs_order(int64_t n, int64_t B, int32_t
     if (tail != n && lane == 0) atomicOr(err, kErrBadTree);
 }
 
-// ---- link-cut / cut-link, one warp per selected tree -----------------------
+// ---- link-cut / cut-link ------------------------------------------------------
+// Three steps over the selected trees: k_cut_choose (a warp a tree) finds the
+// subtree that moves, k_cross_count counts the crossing edges in chunks of
+// preorder positions with a block a chunk, and k_link_finish / k_cut_finish (a
+// warp a tree) move the subtree.  The count is what the work is -- up to half the
+// graph's edges a tree -- and with one warp a tree it took 28 (link-cut) and 51 ms
+// (cut-link) for some 165 trees of 10^5 vertices.
+constexpr int kCrossChunk = 256;  // preorder positions of a block
+
 struct TransformIn {
     int64_t n;
     const int64_t *row_off;   // G'
     const int32_t *col;
-    const uint64_t *word;     // [B][n] parent + depth of the old tree
     const int32_t *din;       // [B][n] DFN of the old tree
     const int32_t *size;      // [B][n]
     const int32_t *pre;       // [B][n] preorder -> vertex
-    int32_t *scratch;         // [B][>= n] int32 per tree (cut-link's per-position counts)
+    int32_t *scratch;         // [B][2n] int32: crossing edges of each chunk
+    CutChoice *choice;        // [B]
     const int64_t *slot;      // [B] pool index of each tree
-    int32_t *pool_parents;    // [P][n] written in place
+    int32_t *pool_parents;    // [P][n] the old trees, written in place
     double *factor;           // [B] d_old / d_new
     int32_t r, u, v;
     uint64_t seed;
@@ -198,13 +208,22 @@ struct TransformIn {
     uint32_t *err;
 };
 
-__device__ int64_t tree_dist(const uint64_t *wd, int32_t a, int32_t b, int64_t n) {
+__device__ __forceinline__ bool in_subtree(const int32_t *din, const int32_t *size, int32_t x,
+                                           int32_t y) {  // y in Sub(x)
+    return (uint32_t)(din[y] - din[x]) < (uint32_t)size[x];
+}
+
+// hops from a up to the lowest ancestor whose subtree holds b (returned in a)
+__device__ int64_t climb_to(const int32_t *par, const int32_t *din, const int32_t *size, int32_t &a,
+                            int32_t b, int64_t n) {
     int64_t d = 0;
-    int32_t da = (int32_t)w_count(wd[a]), db = (int32_t)w_count(wd[b]);
-    for (int64_t it = 0; it < 2 * n + 2 && a != b; ++it) {
-        if (da >= db) { a = w_next(wd[a]); --da; } else { b = w_next(wd[b]); --db; }
-        ++d;
-    }
+    for (; d <= n && !in_subtree(din, size, a, b); ++d) a = par[a];
+    return d;
+}
+
+__device__ int64_t hops_up(const int32_t *par, int32_t a, int32_t top, int64_t n) {
+    int64_t d = 0;
+    for (; d <= n && a != top; ++d) a = par[a];
     return d;
 }
 
@@ -222,91 +241,116 @@ __device__ void reroot_chain(int32_t *p, int32_t x, int32_t top, int32_t attach,
     atomicOr(err, kErrBadTree);
 }
 
-__global__ void __launch_bounds__(128) k_link_cut(TransformIn a, int64_t B) {
-    const int lane = threadIdx.x & 31;
-    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// The root x of the subtree that moves: link-cut draws an edge of the cycle that
+// (u, v) closes (numbered from u up to the lowest common ancestor, then from v);
+// cut-link has the end of (u, v) below the other.
+__global__ void k_cut_choose(TransformIn a, int64_t B, bool insert) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= B) return;
     const int64_t n = a.n;
-    const uint64_t *wd = a.word + t * n;
+    const int32_t *par = a.pool_parents + a.slot[t] * n;
     const int32_t *din = a.din + t * n;
-    const int32_t *sz = a.size + t * n;
-    const int32_t *pre = a.pre + t * n;
-    // path u..v: climb to the lowest common ancestor
-    int32_t x = -1, side = -1;
-    int64_t d_old = 0;
-    if (lane == 0) {
-        int32_t p = a.u, q = a.v;
-        int32_t dp = (int32_t)w_count(wd[p]), dq = (int32_t)w_count(wd[q]);
-        while (dp > dq) { p = w_next(wd[p]); --dp; }
-        while (dq > dp) { q = w_next(wd[q]); --dq; }
-        while (p != q) { p = w_next(wd[p]); q = w_next(wd[q]); }
-        const int64_t du = (int64_t)w_count(wd[a.u]) - w_count(wd[p]);
-        const int64_t dvv = (int64_t)w_count(wd[a.v]) - w_count(wd[p]);
-        d_old = du + dvv;
-        const int64_t k = (int64_t)bounded_draw(a.seed, a.seq, (uint32_t)a.slot[t], 0, kTagLinkCut,
-                                                (uint32_t)d_old);
-        if (k < du) {
-            x = a.u;
-            for (int64_t i = 0; i < k; ++i) x = w_next(wd[x]);
-            side = a.u;
-        } else {
-            x = a.v;
-            for (int64_t i = 0; i < k - du; ++i) x = w_next(wd[x]);
-            side = a.v;
-        }
-        reroot_chain(a.pool_parents + a.slot[t] * n, side, x, side == a.u ? a.v : a.u, n, a.err);
+    const int32_t *size = a.size + t * n;
+    CutChoice c;
+    c.d_old = 0;
+    if (insert) {
+        int32_t top = a.u;
+        const int64_t du = climb_to(par, din, size, top, a.v, n);
+        const int64_t dv = hops_up(par, a.v, top, n);
+        c.d_old = du + dv;
+        int64_t k = (int64_t)bounded_draw(a.seed, a.seq, (uint32_t)a.slot[t], 0, kTagLinkCut,
+                                          (uint32_t)c.d_old);
+        c.side = k < du ? a.u : a.v;
+        c.x = c.side;
+        for (k = k < du ? k : k - du; k > 0; --k) c.x = par[c.x];
+    } else {
+        c.x = par[a.u] == a.v ? a.u : a.v;
+        c.side = c.x == a.u ? a.v : a.u;  // the old parent
     }
-    x = __shfl_sync(kFull, x, 0);
-    // edges of G' other than e that cross Sub(tau, x): an edge crosses the cut
-    // from either side, so the scan runs over the smaller side (the preorder
-    // positions of Sub(tau, x), or all the others)
-    const int32_t lo = din[x], hi = din[x] + sz[x] - 1;
-    const bool inside = 2 * (int64_t)sz[x] <= n;
-    const int64_t span = inside ? (int64_t)sz[x] : n - sz[x];
-    long long cross = 0;
-    for (int64_t k = lane; k < span; k += 32) {
-        const int64_t q = inside ? lo + k : (k < lo ? k : k + sz[x]);
-        const int32_t y = pre[q];
-        for (int64_t e = a.row_off[y]; e < a.row_off[y + 1]; ++e) {
-            const int32_t z = a.col[e];
-            const int32_t dz = din[z];
-            if ((dz >= lo && dz <= hi) == inside) continue;  // both ends on the scanned side
-            if ((y == a.u && z == a.v) || (y == a.v && z == a.u)) continue;
-            ++cross;
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cross += __shfl_down_sync(kFull, cross, o);
-    if (lane == 0) a.factor[t] = cross > 0 ? (double)d_old / (double)cross : 0.0;
+    a.choice[t] = c;
 }
 
-__global__ void __launch_bounds__(128) k_cut_link(TransformIn a, int64_t B) {
+// Crossing edges of the cut around Sub(x), from the preorder positions of Sub(x),
+// or (smaller_side) of the rest where that is smaller: a warp a vertex, a block a
+// chunk of positions.  Link-cut leaves out the new edge (u, v) itself.
+__global__ void __launch_bounds__(256) k_cross_count(TransformIn a, bool insert) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t n = a.n, t = blockIdx.y;
+    const int32_t *__restrict__ din = a.din + t * n;
+    const int32_t *__restrict__ pre = a.pre + t * n;
+    const int32_t x = a.choice[t].x;
+    const int32_t lo = din[x], sz = a.size[t * n + x];
+    const bool inside = !insert || 2 * (int64_t)sz <= n;
+    const int64_t span = inside ? (int64_t)sz : n - sz;
+    __shared__ int32_t part[8];
+    for (int64_t chunk = blockIdx.x; chunk * kCrossChunk < span; chunk += gridDim.x) {
+        int32_t cross = 0;
+        for (int i = warp; i < kCrossChunk; i += 8) {
+            const int64_t k = chunk * kCrossChunk + i;
+            if (k >= span) break;
+            const int32_t y = pre[inside ? lo + k : (k < lo ? k : k + sz)];
+            for (int64_t e = a.row_off[y] + lane; e < a.row_off[y + 1]; e += 32) {
+                const int32_t z = a.col[e];
+                if (((uint32_t)(din[z] - lo) < (uint32_t)sz) == inside) continue;
+                if (insert && ((y == a.u && z == a.v) || (y == a.v && z == a.u))) continue;
+                ++cross;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) cross += __shfl_down_sync(kFull, cross, o);
+        if (lane == 0) part[warp] = cross;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int32_t all = 0;
+            for (int i = 0; i < 8; ++i) all += part[i];
+            a.scratch[t * 2 * n + chunk] = all;
+        }
+        __syncthreads();
+    }
+}
+
+__device__ __forceinline__ long long warp_sum(long long x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+    return x;
+}
+
+__global__ void __launch_bounds__(128) k_link_finish(TransformIn a, int64_t B) {
     const int lane = threadIdx.x & 31;
     const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (t >= B) return;
     const int64_t n = a.n;
-    const uint64_t *wd = a.word + t * n;
-    const int32_t *din = a.din + t * n;
-    const int32_t *sz = a.size + t * n;
-    const int32_t *pre = a.pre + t * n;
-    const int32_t c = (w_next(wd[a.u]) == a.v) ? a.u : a.v;
-    const int32_t qv = (c == a.u) ? a.v : a.u;
-    const int32_t lo = din[c], hi = din[c] + sz[c] - 1;
-    // count crossing edges (G' no longer has e) from the smaller side of the
-    // cut: the preorder positions of Sub(tau, c), or all the others
-    const bool inside = 2 * (int64_t)sz[c] <= n;
-    const int64_t span = inside ? (int64_t)sz[c] : n - sz[c];
+    const CutChoice c = a.choice[t];
+    const int32_t sz = a.size[t * n + c.x];
+    const int64_t span = 2 * (int64_t)sz <= n ? (int64_t)sz : n - sz;
     long long cross = 0;
-    for (int64_t kq = lane; kq < span; kq += 32) {
-        const int64_t q = inside ? lo + kq : (kq < lo ? kq : kq + sz[c]);
-        const int32_t y = pre[q];
-        for (int64_t e = a.row_off[y]; e < a.row_off[y + 1]; ++e) {
-            const int32_t dz = din[a.col[e]];
-            if ((dz >= lo && dz <= hi) != inside) ++cross;
-        }
+    for (int64_t i = lane; i * kCrossChunk < span; i += 32) cross += a.scratch[t * 2 * n + i];
+    cross = warp_sum(cross);
+    if (lane == 0) {
+        reroot_chain(a.pool_parents + a.slot[t] * n, c.side, c.x, c.side == a.u ? a.v : a.u, n,
+                     a.err);
+        a.factor[t] = cross > 0 ? (double)c.d_old / (double)cross : 0.0;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cross += __shfl_xor_sync(kFull, cross, o);
+}
+
+// The k-th crossing edge in (preorder position of the inside end, outside end
+// ascending) order: its chunk, then its position, then its place in the row.
+__global__ void __launch_bounds__(128) k_cut_finish(TransformIn a, int64_t B) {
+    const int lane = threadIdx.x & 31;
+    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (t >= B) return;
+    const int64_t n = a.n;
+    int32_t *par = a.pool_parents + a.slot[t] * n;
+    const int32_t *din = a.din + t * n;
+    const int32_t *size = a.size + t * n;
+    const int32_t *pre = a.pre + t * n;
+    const int32_t *cnt = a.scratch + t * 2 * n;
+    const CutChoice c = a.choice[t];
+    const int32_t lo = din[c.x], sz = size[c.x];
+    const int64_t chunks = ((int64_t)sz + kCrossChunk - 1) / kCrossChunk;
+    long long cross = 0;
+    for (int64_t i = lane; i < chunks; i += 32) cross += cnt[i];
+    cross = warp_sum(cross);
     if (cross <= 0) {
         if (lane == 0) atomicOr(a.err, kErrBadTree);
         return;
@@ -316,106 +360,55 @@ __global__ void __launch_bounds__(128) k_cut_link(TransformIn a, int64_t B) {
         k = (long long)bounded_draw(a.seed, a.seq, (uint32_t)a.slot[t], 0, kTagCutLink,
                                     (uint32_t)cross);
     k = __shfl_sync(kFull, k, 0);
-    // find the k-th crossing edge in (preorder position of the inside end,
-    // outside end ascending) order
-    int32_t ia = -1, ob = -1;
-    long long before = 0;
-    if (!inside) {
-        // the outside is smaller: tally each inside position's crossing edges
-        // from the outside (atomics in L2), then scan the tallies in order
-        int32_t *cnt = a.scratch + t * n;
-        for (int64_t i = lane; i < sz[c]; i += 32) __stcg(cnt + i, 0);
-        __threadfence_block();
-        __syncwarp();
-        for (int64_t kq = lane; kq < span; kq += 32) {
-            const int64_t q = kq < lo ? kq : kq + sz[c];
-            const int32_t y = pre[q];
-            for (int64_t e = a.row_off[y]; e < a.row_off[y + 1]; ++e) {
-                const int32_t dz = din[a.col[e]];
-                if (dz >= lo && dz <= hi) atomicAdd(cnt + (dz - lo), 1);
-            }
-        }
-        __threadfence_block();
-        __syncwarp();
-        int64_t hit = -1;  // inside position (from lo) holding the k-th edge
-        long long hit_start = 0;
-        for (int64_t base = 0; base < sz[c] && hit < 0; base += 32) {
-            const int64_t i = base + lane;
-            const long long mine = i < sz[c] ? (long long)__ldcg(cnt + i) : 0;
-            long long incl = mine;
-#pragma unroll
-            for (int s2 = 1; s2 < 32; s2 <<= 1) {
-                const long long yv = __shfl_up_sync(kFull, incl, s2);
-                if (lane >= s2) incl += yv;
-            }
-            const long long start = before + incl - mine;
-            const unsigned hb = __ballot_sync(kFull, mine > 0 && k >= start && k < start + mine);
-            if (hb) {
-                const int src = __ffs(hb) - 1;
-                hit = base + src;
-                hit_start = __shfl_sync(kFull, start, src);
-            }
-            before += __shfl_sync(kFull, incl, 31);
-        }
-        if (lane == 0 && hit >= 0) {
-            const int32_t y = pre[lo + hit];
-            long long idx = hit_start;
-            for (int64_t e = a.row_off[y]; e < a.row_off[y + 1]; ++e) {
-                const int32_t z = a.col[e];
-                const int32_t dz = din[z];
-                if (dz >= lo && dz <= hi) continue;
-                if (idx == k) { ia = y; ob = z; break; }
-                ++idx;
-            }
-        }
-    }
-    for (int64_t base = lo; inside && base <= hi; base += 32) {
-        const int64_t q = base + lane;
-        int32_t y = -1;
-        long long mine = 0;
-        if (q <= hi) {
-            y = pre[q];
-            for (int64_t e = a.row_off[y]; e < a.row_off[y + 1]; ++e) {
-                const int32_t dz = din[a.col[e]];
-                if (dz < lo || dz > hi) ++mine;
-            }
-        }
+    int64_t chunk = -1;
+    for (int64_t base = 0; base < chunks && chunk < 0; base += 32) {
+        const int64_t i = base + lane;
+        const long long mine = i < chunks ? (long long)cnt[i] : 0;
         long long incl = mine;
 #pragma unroll
-        for (int s = 1; s < 32; s <<= 1) {
-            const long long yv = __shfl_up_sync(kFull, incl, s);
-            if (lane >= s) incl += yv;
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
         }
-        const long long total = __shfl_sync(kFull, incl, 31);
-        const long long start = before + incl - mine;
-        const bool here = mine > 0 && k >= start && k < start + mine;
-        const unsigned hb = __ballot_sync(kFull, here);
-        if (hb) {
-            if (here) {
-                long long idx = start;
-                for (int64_t e = a.row_off[y]; e < a.row_off[y + 1]; ++e) {
-                    const int32_t z = a.col[e];
-                    const int32_t dz = din[z];
-                    if (dz >= lo && dz <= hi) continue;
-                    if (idx == k) { ia = y; ob = z; break; }
-                    ++idx;
-                }
+        const unsigned hit = __ballot_sync(kFull, k >= incl - mine && k < incl);
+        if (hit) {
+            const int src = __ffs(hit) - 1;
+            chunk = base + src;
+            k -= __shfl_sync(kFull, incl - mine, src);
+        } else {
+            k -= __shfl_sync(kFull, incl, 31);
+        }
+    }
+    int32_t ia = -1, ob = -1;
+    for (int64_t i = chunk * kCrossChunk; chunk >= 0 && i < sz && ia < 0; ++i) {
+        if (i >= (chunk + 1) * kCrossChunk) break;
+        const int32_t y = pre[lo + i];
+        for (int64_t e0 = a.row_off[y]; e0 < a.row_off[y + 1]; e0 += 32) {
+            int32_t z = -1;
+            bool out = false;
+            if (e0 + lane < a.row_off[y + 1]) {
+                z = a.col[e0 + lane];
+                out = (uint32_t)(din[z] - lo) >= (uint32_t)sz;
             }
-            const int src = __ffs(hb) - 1;
-            ia = __shfl_sync(kFull, ia, src);
-            ob = __shfl_sync(kFull, ob, src);
-            break;
+            const unsigned m = __ballot_sync(kFull, out);
+            if (k < __popc(m)) {
+                const int src = __fns(m, 0, (int)k + 1);
+                ia = y;
+                ob = __shfl_sync(kFull, z, src);
+                break;
+            }
+            k -= __popc(m);
         }
-        before += total;
     }
     if (lane == 0) {
         if (ia < 0) {
             atomicOr(a.err, kErrBadTree);
             return;
         }
-        const int64_t d_new = ((int64_t)w_count(wd[ia]) - w_count(wd[c])) + 1 +
-                              tree_dist(wd, ob, qv, n);
-        reroot_chain(a.pool_parents + a.slot[t] * n, ia, c, ob, n, a.err);
+        int32_t top = ob;  // path ob .. the old parent, both outside Sub(x)
+        const int64_t up = climb_to(par, din, size, top, c.side, n);
+        const int64_t d_new = hops_up(par, ia, c.x, n) + 1 + up + hops_up(par, c.side, top, n);
+        reroot_chain(par, ia, c.x, ob, n, a.err);
         a.factor[t] = (double)cross / (double)d_new;
     }
 }
@@ -531,18 +524,18 @@ cudaError_t launch_prepare_from_parents(int64_t n, int64_t B, int32_t root,
 }
 
 cudaError_t launch_link_cut(const int64_t *row_off, const int32_t *col, WaveView w,
-                            const int64_t *slot, int32_t *pool_parents, double *factor, int32_t r,
-                            int32_t u, int32_t v, uint64_t seed, uint32_t seq, bool insert,
-                            cudaStream_t s) {
+                            const int64_t *slot, int32_t *pool_parents, double *factor,
+                            CutChoice *choice, int32_t r, int32_t u, int32_t v, uint64_t seed,
+                            uint32_t seq, bool insert, cudaStream_t s) {
     TransformIn a;
     a.n = w.n;
     a.row_off = row_off;
     a.col = col;
-    a.word = w.word;
     a.din = w.din;
     a.size = w.size;
     a.pre = w.aux;
     a.scratch = reinterpret_cast<int32_t *>(w.vol);  // 8n bytes per tree, unused here
+    a.choice = choice;
     a.slot = slot;
     a.pool_parents = pool_parents;
     a.factor = factor;
@@ -552,8 +545,12 @@ cudaError_t launch_link_cut(const int64_t *row_off, const int32_t *col, WaveView
     a.seed = seed;
     a.seq = seq;
     a.err = w.err;
-    if (insert) k_link_cut<<<blk(w.B * 32, 128), 128, 0, s>>>(a, w.B);
-    else k_cut_link<<<blk(w.B * 32, 128), 128, 0, s>>>(a, w.B);
+    k_cut_choose<<<blk(w.B, 32), 32, 0, s>>>(a, w.B, insert);
+    const dim3 grid((unsigned)std::min<int64_t>((w.n + kCrossChunk - 1) / kCrossChunk, 2048),
+                    (unsigned)w.B);
+    k_cross_count<<<grid, 256, 0, s>>>(a, insert);
+    if (insert) k_link_finish<<<blk(w.B * 32, 128), 128, 0, s>>>(a, w.B);
+    else k_cut_finish<<<blk(w.B * 32, 128), 128, 0, s>>>(a, w.B);
     return cudaGetLastError();
 }
 

@@ -1062,6 +1062,7 @@ void sync_host_csr(kc_graph *g) {
 struct UpdBuf {
     int64_t *slots;   // [P]
     double *factor;   // [P]
+    CutChoice *cut;   // [P]
     int64_t *sel;     // [P]
     uint8_t *flags;   // [P]
     uint8_t *taken;   // [P]
@@ -1070,7 +1071,8 @@ struct UpdBuf {
 
 UpdBuf upd_buf(kc_graph *g) {
     const size_t P = (size_t)std::max<int64_t>(g->pool, 1);
-    const size_t need = align256(8 * P) * 3 + align256(P) * 2 + 256;
+    const size_t need =
+        align256(8 * P) * 3 + align256(sizeof(CutChoice) * P) + align256(P) * 2 + 256;
     if (need > g->ub_bytes) {
         if (g->d_ub) cudaFree(g->d_ub);
         g->d_ub = nullptr;
@@ -1084,6 +1086,8 @@ UpdBuf upd_buf(kc_graph *g) {
     b += align256(8 * P);
     u.factor = (double *)b;
     b += align256(8 * P);
+    u.cut = (CutChoice *)b;
+    b += align256(sizeof(CutChoice) * P);
     u.sel = (int64_t *)b;
     b += align256(8 * P);
     u.flags = (uint8_t *)b;
@@ -1123,22 +1127,30 @@ void refresh_slots(kc_graph *g, const std::vector<int64_t> &slots) {
         Carved c = carve(g, p);
         WaveView w = c.wv;
         w.B = b;
+        if (!p.bit) {  // any valid DFN serves the tau0 scan
+            const ParTrees trees{g->d_parents, ub.slots};
+            int nl = 0;
+            KC_CK(g, launch_traverse_parents(gv, w, trees, false, -1, -1, false, g->stream, &nl));
+            KC_CK(g, launch_ttf_scan_parents(gv, w, trees, g->stream));
+            KC_CK(g, launch_scatter_results(ub.slots, b, w.f, nullptr, nullptr, g->d_f,
+                                            g->d_steps, g->d_sid, g->stream));
+            g->t_update.launches += nl + 2;
+            check_err(g, "refresh");
+            continue;
+        }
         KC_CK(g, launch_prepare_from_parents(g->n, b, g->root, g->d_parents, ub.slots, w,
                                              g->stream));
         uint32_t hdr[2] = {0, 0};
         KC_CK(g, cudaMemcpyAsync(hdr, g->d_err, sizeof(hdr), cudaMemcpyDeviceToHost, g->stream));
         KC_CK(g, cudaStreamSynchronize(g->stream));
         if (hdr[0]) check_err(g, "refresh");
-        if (p.bit) {
-            ensure_stack(g, p, hdr[1]);
-            c = carve(g, p);
-            w = c.wv;
-            w.B = b;
-        }
+        ensure_stack(g, p, hdr[1]);
+        c = carve(g, p);
+        w = c.wv;
+        w.B = b;
         int nl = 0;
-        KC_CK(g, launch_traverse(gv, w, p.bit, g->stream, &nl, fast_traversal(g)));
-        if (p.bit) KC_CK(g, launch_ttf_bit(gv, w, g->stream));
-        else KC_CK(g, launch_ttf_scan(gv, w, g->stream));
+        KC_CK(g, launch_traverse(gv, w, true, g->stream, &nl, fast_traversal(g)));
+        KC_CK(g, launch_ttf_bit(gv, w, g->stream));
         KC_CK(g, launch_scatter_results(ub.slots, b, w.f, nullptr, nullptr, g->d_f, g->d_steps,
                                         g->d_sid, g->stream));
         g->t_update.launches += nl + 6;
@@ -1224,20 +1236,18 @@ void transform_slots(kc_graph *g, const std::vector<int64_t> &slots, bool insert
         Carved c = carve(g, p);
         WaveView w = c.wv;
         w.B = b;
-        KC_CK(g, launch_prepare_from_parents(g->n, b, g->root, g->d_parents, ub.slots, w,
-                                             g->stream));
         // link-cut reads the DFN only to test subtree membership, so any valid
-        // DFN serves (the warp-per-tree pass); cut-link picks the k-th crossing
-        // edge in the id-ordered preorder, which the canonical pass gives
+        // DFN serves; cut-link picks the k-th crossing edge in the id-ordered
+        // preorder, and its trees hold the edge that the graph has lost
         int nl = 0;
-        KC_CK(g, launch_traverse(gv, w, true, g->stream, &nl,
-                                 insert ? kTravChunked : kTravCanonical));
+        KC_CK(g, launch_traverse_parents(gv, w, ParTrees{g->d_parents, ub.slots}, !insert,
+                                         insert ? -1 : u, insert ? -1 : v, true, g->stream, &nl));
         KC_CK(g, launch_link_cut(g->d_row_off, g->d_col, w, ub.slots, g->d_parents, ub.factor,
-                                 g->root, u, v, g->seed, (uint32_t)g->update_seq, insert,
+                                 ub.cut, g->root, u, v, g->seed, (uint32_t)g->update_seq, insert,
                                  g->stream));
         KC_CK(g, launch_scale_slots(g->d_w, ub.slots, ub.factor, b, g->stream));
         check_err(g, insert ? "link-cut" : "cut-link");
-        g->t_update.launches += nl + 7;
+        g->t_update.launches += nl + 4;
         std::vector<int64_t> part(slots.begin() + c0, slots.begin() + c0 + b);
         for (int64_t x : part) g->h_modified[(size_t)x] = 1;
     }

@@ -502,6 +502,21 @@ cudaError_t launch_wilson_warp_reject(const GraphView &g, WaveView w, uint64_t s
 enum : int { kTravCanonical = 0, kTravChunked = 1, kTravLeafUp = 2 };
 cudaError_t launch_traverse(const GraphView &g, WaveView w, bool want_preorder, cudaStream_t s,
                             int *launches = nullptr, int mode = kTravCanonical);
+// Trees by their parent arrays: parent of v in tree t is par[(slot ? slot[t] : t) n + v].
+struct ParTrees {
+    const int32_t *par = nullptr;
+    const int64_t *slot = nullptr;
+};
+// Order-free traversal (k2_parents.cu): w.size, w.vol and w.din (by_id: the DFN with
+// children in ascending id, else some valid one), w.aux the preorder if wanted;
+// w.word is scratch.  (eu, ev): an edge that the trees may hold and the graph does
+// not (eu < 0: none), needed with by_id.  w.B at most 65535.
+cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool by_id,
+                                    int32_t eu, int32_t ev, bool want_preorder, cudaStream_t s,
+                                    int *launches = nullptr);
+// f by the tau0 scan of trees traversed that way
+cudaError_t launch_ttf_scan_parents(const GraphView &g, WaveView w, ParTrees trees,
+                                    cudaStream_t s);
 cudaError_t launch_ttf_scan(const GraphView &g, WaveView w, cudaStream_t s);
 cudaError_t launch_ttf_bit(const GraphView &g, WaveView w, cudaStream_t s);
 // f of the sub-wave's trees from segments that each start from the DFS state
@@ -534,10 +549,18 @@ cudaError_t launch_select(uint64_t seed, uint32_t seq, int64_t N, int64_t k, uin
 cudaError_t launch_prepare_from_parents(int64_t n, int64_t B, int32_t root,
                                         const int32_t *pool_parents, const int64_t *slot,
                                         WaveView w, cudaStream_t s);
+// What link-cut / cut-link does to a tree: Sub(x) moves, hung up by `side` (link-cut:
+// the end of the new edge inside Sub(x); cut-link: x's old parent).
+struct CutChoice {
+    int32_t x, side;
+    int64_t d_old;  // link-cut: length of the cycle less the new edge
+};
+// w.din, w.size and w.aux (preorder) of the trees at `slot` (launch_traverse_parents;
+// cut-link: by_id); w.vol is scratch
 cudaError_t launch_link_cut(const int64_t *row_off, const int32_t *col, WaveView w,
-                            const int64_t *slot, int32_t *pool_parents, double *factor, int32_t r,
-                            int32_t u, int32_t v, uint64_t seed, uint32_t seq, bool insert,
-                            cudaStream_t s);
+                            const int64_t *slot, int32_t *pool_parents, double *factor,
+                            CutChoice *choice, int32_t r, int32_t u, int32_t v, uint64_t seed,
+                            uint32_t seq, bool insert, cudaStream_t s);
 cudaError_t launch_scale_slots(double *w, const int64_t *slot, const double *factor, int64_t B,
                                cudaStream_t s);
 cudaError_t launch_weight_rescale(double *w, const uint8_t *flag, int64_t P, double *sums,
