@@ -18,7 +18,17 @@
 // vertices that does not hold a).  Settled paths are never followed again, so all
 // rounds together settle each vertex once.
 //
-// k_pop_small keeps the tree in shared memory: 14 bytes a vertex.
+// k_pop_small keeps the tree in shared memory: 14 bytes a vertex.  Larger trees
+// stay in memory: the first arrows (k_first_arrows) and the cycles of the first map
+// (k_first_cycles) are passes over all vertices of all trees, the rounds after it,
+// which touch a tenth of the vertices where the root is a hub, a block per tree
+// (k_pop_rounds); the traversal is that of k2_parents.cu.  What bounds it is the
+// rate of random sectors, about ten a vertex with the traversal.
+//
+// Measured (GB300, power-law graphs of mean degree 17, against 32 walkers a tree
+// and their traversal): 2 million vertices, 384 trees 830 -> 160 ms (rounds 43,
+// first cycles 16, first arrows 5; traversal 65, tau0 scan 10); 10000 vertices in
+// shared memory, 500 trees 5.26 -> 1.27 ms.
 #include <algorithm>
 
 #include "kc_common.cuh"
@@ -228,6 +238,147 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 12 : (kThreads <= 
     if (tid == 0) task.f[t] = (int64_t)s_f;
 }
 
+// ---- larger trees, in memory ------------------------------------------------
+// Vertex word: target (low half); pops, settled (bit 30), active (bit 31).
+__device__ __forceinline__ uint64_t large_arrow(const PopTask &task, uint32_t sample, uint32_t v,
+                                                uint32_t count) {
+    const VRec r = load_rec(task.g.rec + v);
+    const uint32_t k = bounded_draw_k(task.keys, task.seed, v, count, sample, kTagWalk,
+                                      (uint32_t)r.deg);
+    return (uint32_t)nbr_of<false>(r, k, task.g.col);
+}
+
+constexpr int kFirstTrees = 4;  // trees for which a thread keeps a vertex's record
+__global__ void __launch_bounds__(256) k_first_arrows(PopTask task, int64_t B, uint64_t *words) {
+    const int64_t n = task.g.n;
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= n) return;
+    const VRec r = load_rec(task.g.rec + v);
+    const int64_t t0 = (int64_t)blockIdx.y * kFirstTrees;
+    const int64_t t1 = t0 + kFirstTrees < B ? t0 + kFirstTrees : B;
+    for (int64_t t = t0; t < t1; ++t) {
+        uint64_t x = (uint64_t)(uint32_t)task.root | (uint64_t)kSettled << 32;
+        if (v != task.root && v != task.fixed) {
+            const uint32_t k = bounded_draw_k(task.keys, task.seed, (uint32_t)v, 0,
+                                              (uint32_t)task.sids[t], kTagWalk, (uint32_t)r.deg);
+            x = (uint32_t)nbr_of<false>(r, k, task.g.col);
+        }
+        words[t * n + v] = x;
+    }
+}
+
+// As led_cycle; kFirst: every vertex is active.
+template <bool kFirst>
+__device__ __forceinline__ int32_t led_cycle_large(uint64_t *word, int32_t a) {
+    int32_t x = w_next(word[a]);
+    int32_t saved = -1, len = 1;
+    uint32_t met = 0, power = 1;
+    for (;; ++len) {
+        const uint64_t w = word[x];
+        const uint32_t hi = (uint32_t)(w >> 32);
+        if (kFirst || hi >= kSettled) {
+            if (hi & kSettled) break;
+            if (x <= a) return x == a ? len : 0;
+            if (x == saved) return 0;
+            if (++met == power) {
+                saved = x;
+                power <<= 1;
+                met = 0;
+            }
+        }
+        x = w_next(w);
+    }
+    x = a;
+    for (uint64_t w = word[x]; !((w >> 32) & kSettled); w = word[x]) {
+        word[x] = w | (uint64_t)kSettled << 32;
+        x = w_next(w);
+    }
+    return 0;
+}
+
+__device__ __forceinline__ void list_cycle(const uint64_t *word, int32_t *list, uint32_t at,
+                                           int32_t a) {
+    int32_t x = a;
+    do {
+        list[at++] = x;
+        x = w_next(word[x]);
+    } while (x != a);
+}
+
+__global__ void __launch_bounds__(256) k_first_cycles(int64_t n, uint64_t *words, int32_t *lists,
+                                                      unsigned long long *found) {
+    const int64_t t = blockIdx.y;
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint64_t *word = words + t * n;
+    if (v >= n || ((word[v] >> 32) & kSettled)) return;
+    const int32_t len = led_cycle_large<true>(word, (int32_t)v);
+    if (len)
+        list_cycle(word, lists + t * n, (uint32_t)atomicAdd(found + t, (unsigned long long)len),
+                   (int32_t)v);
+}
+
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, 1024 / kThreads)
+    k_pop_rounds(PopTask task, uint64_t *words, int32_t *lists0, int32_t *lists1,
+                 const unsigned long long *found0) {
+    const int64_t t = blockIdx.x, n = task.g.n;
+    const uint32_t sample = (uint32_t)task.sids[t], tid = threadIdx.x;
+    uint64_t *word = words + t * n;
+    int32_t *list = lists0 + t * n, *fresh = lists1 + t * n;
+    __shared__ uint32_t s_count[2];
+    uint32_t active = (uint32_t)found0[t];
+    int64_t pops = 0;
+    int end = 0;
+    if (tid < 2) s_count[tid] = 0;
+    for (int round = 0; active > 0; ++round) {
+        pops += active;
+        if (pops + n - task.placed > task.step_cap) {
+            end = kErrStepLimit;
+            break;
+        }
+        __syncthreads();
+        bool full = false;
+        for (uint32_t i = tid; i < active; i += kThreads) {
+            const int32_t v = list[i];
+            const uint32_t c = (uint32_t)(word[v] >> 32) + 1;
+            word[v] = large_arrow(task, sample, (uint32_t)v, c) | (uint64_t)(c | kActive) << 32;
+            full = full || c >= kWalkCountMask;
+        }
+        if (__syncthreads_or(full)) {
+            end = kErrCountField;
+            break;
+        }
+        for (uint32_t i = tid; i < active; i += kThreads) {
+            const int32_t a = list[i];
+            if ((word[a] >> 32) & kSettled) continue;
+            const int32_t len = led_cycle_large<false>(word, a);
+            if (len) list_cycle(word, fresh, atomicAdd(&s_count[round & 1], (uint32_t)len), a);
+        }
+        __syncthreads();
+        for (uint32_t i = tid; i < active; i += kThreads)
+            word[list[i]] &= ~((uint64_t)kActive << 32);
+        active = s_count[round & 1];
+        if (tid == 0) s_count[(round + 1) & 1] = 0;
+        int32_t *const swap = list;
+        list = fresh;
+        fresh = swap;
+    }
+    if (tid == 0) {
+        if (end) atomicOr(task.err, (uint32_t)end);
+        task.steps[t] = end ? -1 : pops + n - task.placed;
+    }
+}
+
+// parents of the finished maps, and the words zeroed for the traversal
+__global__ void __launch_bounds__(256) k_take_parents(int64_t n, int64_t B, int32_t root,
+                                                      uint64_t *words, int32_t *par) {
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= B * n) return;
+    const int32_t p = w_next(words[k]);
+    words[k] = 0;
+    par[k] = k % n == root ? -1 : p;
+}
+
 template <int kThreads, bool kMulti>
 cudaError_t launch_small(const PopTask &one, const PopTask *tasks, const int2 *entry,
                          int64_t blocks, int64_t max_n, cudaStream_t s) {
@@ -260,6 +411,25 @@ cudaError_t launch_pop_small(const PopTask &task, int64_t B, cudaStream_t s) {
 cudaError_t launch_pop_small_multi(const PopTask *tasks, const int2 *entry, int64_t count,
                                    int64_t max_n, cudaStream_t s) {
     return launch_small_any<true>(PopTask{}, tasks, entry, count, max_n, s);
+}
+
+cudaError_t launch_pop_large(const PopTask &task, int64_t B, uint64_t *words, int32_t *lists0,
+                             int32_t *lists1, int64_t *found, int64_t num_sms, cudaStream_t s) {
+    const int64_t n = task.g.n;
+    const cudaError_t e = cudaMemsetAsync(found, 0, sizeof(int64_t) * (size_t)B, s);
+    if (e != cudaSuccess) return e;
+    unsigned long long *count = reinterpret_cast<unsigned long long *>(found);
+    const unsigned rows = (unsigned)((n + 255) / 256);
+    k_first_arrows<<<dim3(rows, (unsigned)((B + kFirstTrees - 1) / kFirstTrees)), 256, 0, s>>>(
+        task, B, words);
+    k_first_cycles<<<dim3(rows, (unsigned)B), 256, 0, s>>>(n, words, lists0, count);
+    if (B <= num_sms)
+        k_pop_rounds<1024><<<(unsigned)B, 1024, 0, s>>>(task, words, lists0, lists1, count);
+    else
+        k_pop_rounds<256><<<(unsigned)B, 256, 0, s>>>(task, words, lists0, lists1, count);
+    k_take_parents<<<(unsigned)((B * n + 255) / 256), 256, 0, s>>>(n, B, task.root, words,
+                                                                 task.par);
+    return cudaGetLastError();
 }
 
 }  // namespace kc

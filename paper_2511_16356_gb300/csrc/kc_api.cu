@@ -382,14 +382,16 @@ bool use_solo(const kc_graph *g) {
            g->ttf_variant == KC_TTF_BIT;
 }
 
-// Whether AUTO draws the trees of a low-diameter graph by cycle popping in shared
-// memory (k4_pop.cu), which also evaluates f.
-bool use_pop(const kc_graph *g) {
-    if (g->walker != KC_WALK_WARP || !g->auto_walker || g->ttf_variant != KC_TTF_SCAN ||
-        2 * g->m >= ((int64_t)1 << 32))
-        return false;
+// Whether AUTO draws the trees of a low-diameter graph by cycle popping
+// (k4_pop.cu): in shared memory, where f is evaluated too, or in memory.
+enum : int { kPopNone = 0, kPopSmall = 1, kPopLarge = 2 };
+int use_pop(const kc_graph *g) {
+    if (g->walker != KC_WALK_WARP || !g->auto_walker || g->ttf_variant != KC_TTF_SCAN)
+        return kPopNone;
+    const int64_t twom = 2 * g->m;
     const int64_t root_deg = g->h_row_off[(size_t)g->root + 1] - g->h_row_off[(size_t)g->root];
-    return kc_host::pop_small(g->n, 2 * g->m, root_deg);
+    if (twom < ((int64_t)1 << 32) && kc_host::pop_small(g->n, twom, root_deg)) return kPopSmall;
+    return kc_host::pop_large(g->n, twom, root_deg) ? kPopLarge : kPopNone;
 }
 
 // The trees of wave w (sample ids c.sids): steps, and f unless they are only to be
@@ -661,23 +663,61 @@ bool run_wave_pipelined(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool reje
 
 // Returns whether the trees' parents are in the pool already (k4_pop.cu).
 bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = false) {
-    if (!canonical && !g->tuning && use_pop(g)) {
+    const int pop = canonical || g->tuning ? kPopNone : use_pop(g);
+    if (pop) {
+        const GraphView gv = view_of(g);
         const Carved c = carve(g, p);
         WaveView w = c.wv;
         w.B = B;
         KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
         KC_CK(g, launch_iota(c.sids, sid0, B, g->stream));
-        {
+        uint32_t err = 0;
+        if (pop == kPopSmall) {
             Phase ph(g, g->t_wilson);
-            KC_CK(g, launch_pop_small(pop_task(g, view_of(g), w, c.sids, g->root, -1, true,
+            KC_CK(g, launch_pop_small(pop_task(g, gv, w, c.sids, g->root, -1, true,
                                                pool_slot(g)),
                                       B, g->stream));
             ph.done(1);
         }
-        uint32_t err = 0;
-        KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
+        // in memory: all three steps a sub-wave at a time
+        for (int64_t sub = 0; pop == kPopLarge && sub < B && !err; sub += p.BT) {
+            WaveView sv = w;
+            sv.B = std::min<int64_t>(p.BT, B - sub);
+            sv.word = w.word + sub * g->n;
+            sv.ord = w.ord + sub * g->n;
+            sv.steps = w.steps + sub;
+            sv.f = w.f + sub;
+            int32_t *par = pool_slot(g) ? pool_slot(g) + sub * g->n : sv.ord;
+            {
+                Phase ph(g, g->t_wilson);
+                KC_CK(g, launch_pop_large(pop_task(g, gv, sv, c.sids + sub, g->root, -1, false,
+                                                   par),
+                                          sv.B, sv.word, sv.size, sv.din, sv.f, g->num_sms,
+                                          g->stream));
+                ph.done(4);
+            }
+            KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
+            if (err) break;
+            {
+                Phase ph(g, g->t_traverse);
+                int nl = 0;
+                KC_CK(g, launch_traverse_parents(gv, sv, ParTrees{par, nullptr}, true, false, -1,
+                                                 -1, false, g->stream, &nl));
+                ph.done(nl);
+            }
+            {
+                Phase ph(g, g->t_ttf);
+                KC_CK(g, launch_ttf_scan_parents(gv, sv, ParTrees{par, nullptr}, g->stream));
+                ph.done(1);
+            }
+        }
+        if (!err)
+            KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
         if (!err) return true;
-        if (!solo_retry(g, err)) throw Fail{KC_ERR_CUDA};
+        if (!solo_retry(g, err)) {
+            g->last_error = "inconsistent tree state";
+            throw Fail{KC_ERR_CUDA};
+        }
     }
     // pipelining pays when traversal and TTF take long enough to hide: several
     // sub-waves, or large graphs; short waves of small graphs run straight
@@ -1130,7 +1170,8 @@ void refresh_slots(kc_graph *g, const std::vector<int64_t> &slots) {
         if (!p.bit) {  // any valid DFN serves the tau0 scan
             const ParTrees trees{g->d_parents, ub.slots};
             int nl = 0;
-            KC_CK(g, launch_traverse_parents(gv, w, trees, false, -1, -1, false, g->stream, &nl));
+            KC_CK(g, launch_traverse_parents(gv, w, trees, false, false, -1, -1, false,
+                                             g->stream, &nl));
             KC_CK(g, launch_ttf_scan_parents(gv, w, trees, g->stream));
             KC_CK(g, launch_scatter_results(ub.slots, b, w.f, nullptr, nullptr, g->d_f,
                                             g->d_steps, g->d_sid, g->stream));
@@ -1178,16 +1219,20 @@ void resample_slots(kc_graph *g, const std::vector<int64_t> &slots, bool cond, i
         w.B = b;
         w.pos0 = cond ? 2 : 1;
         KC_CK(g, launch_iota(c.sids, g->next_sid, b, g->stream));
-        bool pop = use_pop(g);
+        int pop = use_pop(g);
         if (pop) {
+            const PopTask task = pop_task(g, gv, w, c.sids, cond ? v : g->root, cond ? u : -1,
+                                          false, w.ord);
             KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
-            KC_CK(g, launch_pop_small(pop_task(g, gv, w, c.sids, cond ? v : g->root,
-                                               cond ? u : -1, false, w.ord),
-                                      b, g->stream));
-            g->t_update.launches += 1;
+            if (pop == kPopSmall)
+                KC_CK(g, launch_pop_small(task, b, g->stream));
+            else
+                KC_CK(g, launch_pop_large(task, b, w.word, w.size, w.din, w.f, g->num_sms,
+                                          g->stream));
+            g->t_update.launches += pop == kPopSmall ? 1 : 4;
             uint32_t err = 0;
             KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
-            pop = !solo_retry(g, err);
+            if (solo_retry(g, err)) pop = kPopNone;
         }
         for (bool solo = use_solo(g); !pop; solo = false) {
             KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
@@ -1240,7 +1285,7 @@ void transform_slots(kc_graph *g, const std::vector<int64_t> &slots, bool insert
         // DFN serves; cut-link picks the k-th crossing edge in the id-ordered
         // preorder, and its trees hold the edge that the graph has lost
         int nl = 0;
-        KC_CK(g, launch_traverse_parents(gv, w, ParTrees{g->d_parents, ub.slots}, !insert,
+        KC_CK(g, launch_traverse_parents(gv, w, ParTrees{g->d_parents, ub.slots}, false, !insert,
                                          insert ? -1 : u, insert ? -1 : v, true, g->stream, &nl));
         KC_CK(g, launch_link_cut(g->d_row_off, g->d_col, w, ub.slots, g->d_parents, ub.factor,
                                  ub.cut, g->root, u, v, g->seed, (uint32_t)g->update_seq, insert,
@@ -1735,7 +1780,7 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
             std::vector<char> solo(G), pop(G);
             for (size_t k = 0; k < G; ++k) {
                 solo[k] = use_solo(gs[idx[k]]) ? 1 : 0;
-                pop[k] = use_pop(gs[idx[k]]) ? 1 : 0;
+                pop[k] = use_pop(gs[idx[k]]) == kPopSmall ? 1 : 0;
             }
             std::vector<size_t> by_work(G);
             for (size_t k = 0; k < G; ++k) by_work[k] = k;

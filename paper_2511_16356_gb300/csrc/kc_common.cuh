@@ -471,6 +471,10 @@ struct PopTask {
 };
 // n at most kc_host::kPopSmallMax, 2m < 2^32: trees and f from shared memory
 cudaError_t launch_pop_small(const PopTask &task, int64_t B, cudaStream_t s);
+// any n: trees in memory.  words [B][n] (left zeroed), two lists [B][n], found [B];
+// task.par receives the parents, task.f is not used.  B at most 65535.
+cudaError_t launch_pop_large(const PopTask &task, int64_t B, uint64_t *words, int32_t *lists0,
+                             int32_t *lists1, int64_t *found, int64_t num_sms, cudaStream_t s);
 // entries (task, tree) of a device table of tasks; max_n: their largest n
 cudaError_t launch_pop_small_multi(const PopTask *tasks, const int2 *entry, int64_t count,
                                    int64_t max_n, cudaStream_t s);
@@ -509,11 +513,12 @@ struct ParTrees {
 };
 // Order-free traversal (k2_parents.cu): w.size, w.vol and w.din (by_id: the DFN with
 // children in ascending id, else some valid one), w.aux the preorder if wanted;
-// w.word is scratch.  (eu, ev): an edge that the trees may hold and the graph does
-// not (eu < 0: none), needed with by_id.  w.B at most 65535.
-cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool by_id,
-                                    int32_t eu, int32_t ev, bool want_preorder, cudaStream_t s,
-                                    int *launches = nullptr);
+// w.word is scratch (zeroed: it is zero already).  (eu, ev): an edge that the trees
+// may hold and the graph does not (eu < 0: none), needed with by_id.  w.B at most
+// 65535.
+cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool zeroed,
+                                    bool by_id, int32_t eu, int32_t ev, bool want_preorder,
+                                    cudaStream_t s, int *launches = nullptr);
 // f by the tau0 scan of trees traversed that way
 cudaError_t launch_ttf_scan_parents(const GraphView &g, WaveView w, ParTrees trees,
                                     cudaStream_t s);

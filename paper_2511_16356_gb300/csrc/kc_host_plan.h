@@ -136,6 +136,10 @@ constexpr int64_t kPopSmallMax = 16000;
 inline bool pop_small(int64_t n, int64_t twom, int64_t root_deg) {
     return n <= kPopSmallMax && (n <= 4096 || 16 * (twom / std::max<int64_t>(root_deg, 1)) <= n);
 }
+// In memory only where the root is such a hub.
+inline bool pop_large(int64_t n, int64_t twom, int64_t root_deg) {
+    return n > kPopSmallMax && 16 * (twom / std::max<int64_t>(root_deg, 1)) <= n;
+}
 inline int pop_small_threads(int64_t n) { return n <= 1024 ? 128 : (n <= 4096 ? 256 : 1024); }
 
 }  // namespace kc_host

@@ -118,3 +118,17 @@ def test_popped_trees_at_the_step_cap():
     with kc.KemenyGraph.from_graph(g, _cfg(step_cap=5)) as G:
         st = kc.kc_sample(G.h, 3, 40, check=False)
         assert kc.STATUS[st] == "KC_ERR_STEP_LIMIT"
+
+
+@pytest.mark.parametrize("trees", [1, 40, 200])
+def test_popped_trees_in_memory_match_oracle(trees):
+    """Power-law graph with a hub as root, too large for shared memory; fewer trees
+    than SMs and more, a kept tree, and trees conditioned on an edge (BSM insertion)."""
+    g = S.chung_lu(20000, 2.1, 8.0, 5)
+    t0 = O.tau0(g)
+    with kc.KemenyGraph.from_graph(g, _cfg(keep_trees=1)) as G:
+        G.sample(43, trees)
+        _check(g, G.samples(), 43, 0, trees)
+        tr, ref = G.tree(trees - 1), O.tree(g, t0, 43, trees - 1)
+        for key in ("parent", "depth", "din", "dout", "vol"):
+            assert np.array_equal(tr[key], getattr(ref, key)), key
