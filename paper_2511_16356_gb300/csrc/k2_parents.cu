@@ -163,6 +163,17 @@ __global__ void k_par_jump(GraphView g, WaveView w, int want_pre) {
     }
 }
 
+// the jumps that add up to the depths
+__global__ void k_par_depth_init(GraphView g, WaveView w, ParTrees trees) {
+    const int64_t n = g.n;
+    const int64_t t = blockIdx.y;
+    const int32_t *__restrict__ par = parents(trees, t, n);
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+         v += (int64_t)gridDim.x * blockDim.x)
+        w.word[t * n + v] = v == g.root ? (uint64_t)(uint32_t)v
+                                        : (1ull << 32 | (uint32_t)par[v]);
+}
+
 }  // namespace
 
 cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool zeroed,
@@ -182,6 +193,14 @@ cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees tre
     }
     k_par_jump<<<grid, 256, 0, s>>>(g, w, want_preorder ? 1 : 0);
     if (launches) *launches += by_id ? 4 : 3;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_depths_parents(const GraphView &g, WaveView w, ParTrees trees,
+                                  cudaStream_t s) {
+    const dim3 grid((unsigned)std::min<int64_t>((g.n + 255) / 256, 4096), (unsigned)w.B);
+    k_par_depth_init<<<grid, 256, 0, s>>>(g, w, trees);
+    k_par_jump<<<grid, 256, 0, s>>>(g, w, 0);
     return cudaGetLastError();
 }
 

@@ -370,13 +370,14 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 }
 
 // parents of the finished maps, and the words zeroed for the traversal
-__global__ void __launch_bounds__(256) k_take_parents(int64_t n, int64_t B, int32_t root,
-                                                      uint64_t *words, int32_t *par) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= B * n) return;
-    const int32_t p = w_next(words[k]);
-    words[k] = 0;
-    par[k] = k % n == root ? -1 : p;
+__global__ void __launch_bounds__(256) k_take_parents(int64_t n, int32_t root, uint64_t *words,
+                                                      int32_t *par) {
+    const int64_t at = (int64_t)blockIdx.y * n;
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= n) return;
+    const int32_t p = w_next(words[at + v]);
+    words[at + v] = 0;
+    par[at + v] = v == root ? -1 : p;
 }
 
 template <int kThreads, bool kMulti>
@@ -427,8 +428,7 @@ cudaError_t launch_pop_large(const PopTask &task, int64_t B, uint64_t *words, in
         k_pop_rounds<1024><<<(unsigned)B, 1024, 0, s>>>(task, words, lists0, lists1, count);
     else
         k_pop_rounds<256><<<(unsigned)B, 256, 0, s>>>(task, words, lists0, lists1, count);
-    k_take_parents<<<(unsigned)((B * n + 255) / 256), 256, 0, s>>>(n, B, task.root, words,
-                                                                 task.par);
+    k_take_parents<<<dim3(rows, (unsigned)B), 256, 0, s>>>(n, task.root, words, task.par);
     return cudaGetLastError();
 }
 

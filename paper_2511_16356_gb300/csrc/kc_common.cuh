@@ -519,6 +519,9 @@ struct ParTrees {
 cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool zeroed,
                                     bool by_id, int32_t eu, int32_t ev, bool want_preorder,
                                     cudaStream_t s, int *launches = nullptr);
+// depths of the trees into w.din; w.word is scratch
+cudaError_t launch_depths_parents(const GraphView &g, WaveView w, ParTrees trees,
+                                  cudaStream_t s);
 // f by the tau0 scan of trees traversed that way
 cudaError_t launch_ttf_scan_parents(const GraphView &g, WaveView w, ParTrees trees,
                                     cudaStream_t s);
