@@ -30,6 +30,7 @@
 // first cycles 16, first arrows 5; traversal 65, tau0 scan 10); 10000 vertices in
 // shared memory, 500 trees 5.26 -> 1.27 ms.
 #include <algorithm>
+#include <atomic>
 
 #include "kc_common.cuh"
 #include "kc_host_plan.h"
@@ -73,14 +74,19 @@ __device__ __forceinline__ uint32_t led_cycle(volatile uint32_t *nx, uint32_t a)
     return 0;
 }
 
-template <int kThreads, bool kMulti>
+// kKind: kFused evaluates f; kTrees leaves the parents in task.par only (whose row
+// holds the two lists meanwhile) and needs 4 bytes a vertex; kTreesCsr does so
+// from the CSR arrays alone, and marks a tree that it cannot finish kPopRedo
+// instead of raising an error.
+enum : int { kFused = 0, kTrees = 1, kTreesCsr = 2 };
+template <int kThreads, bool kMulti, int kKind>
 __global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 12 : (kThreads <= 256 ? 6 : 1))
     k_pop_small(PopTask one, const PopTask *__restrict__ tasks, const int2 *__restrict__ entry) {
     const int64_t t = kMulti ? (int64_t)entry[blockIdx.x].y : (int64_t)blockIdx.x;
     const PopTask task = kMulti ? tasks[entry[blockIdx.x].x] : one;
     const GraphView &g = task.g;
     const uint32_t n = (uint32_t)g.n, root = (uint32_t)task.root;
-    const uint32_t sample = (uint32_t)task.sids[t];
+    const uint32_t sample = (uint32_t)(kKind == kTreesCsr ? task.first_sid + t : task.sids[t]);
     const uint32_t tid = threadIdx.x;
     const VRec *__restrict__ rec = g.rec;
 
@@ -89,12 +95,20 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 12 : (kThreads <= 
     uint32_t *acc = smem + n;  // [n] the two lists of active vertices; then reports, jumps
     uint32_t *vol = smem + 2 * n;
     uint16_t *size = reinterpret_cast<uint16_t *>(smem + 3 * n);
-    uint16_t *list = reinterpret_cast<uint16_t *>(acc), *fresh = list + n;
+    uint16_t *list = kKind == kFused ? reinterpret_cast<uint16_t *>(acc)
+                                     : reinterpret_cast<uint16_t *>(task.par + t * n);
+    uint16_t *fresh = list + n;
     __shared__ uint32_t s_count[2];
     __shared__ unsigned long long s_f;
 
     // arrow number `count` of v
     auto arrow = [&](uint32_t v, uint32_t count) {
+        if (kKind == kTreesCsr) {
+            const int64_t off = g.row_off[v];
+            const uint32_t k = bounded_draw_k(task.keys, task.seed, v, count, sample, kTagWalk,
+                                              (uint32_t)(g.row_off[v + 1] - off));
+            return (uint32_t)g.col[off + k];
+        }
         const VRec r = load_rec(rec + v);
         const uint32_t k = bounded_draw_k(task.keys, task.seed, v, count, sample, kTagWalk,
                                           (uint32_t)r.deg);
@@ -158,84 +172,84 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 12 : (kThreads <= 
     __syncthreads();
     if (end) {  // uniform
         if (tid == 0) {
-            atomicOr(task.err, (uint32_t)end);
-            task.steps[t] = -1;
+            if (kKind != kTreesCsr) atomicOr(task.err, (uint32_t)end);
+            task.steps[t] = kKind == kTreesCsr ? kPopRedo : -1;
         }
         return;
     }
     if (tid == 0) task.steps[t] = pops + (int64_t)n - task.placed;
-    if (task.par)
+    if (kKind != kFused || task.par)
         for (uint32_t v = tid; v < n; v += kThreads)
             task.par[t * n + v] = v == root ? -1 : (int32_t)(nx[v] & kTarget);
-    if (!task.f) return;
-
-    // ---- sizes, volumes and preorder.  acc of a vertex: unreported children
-    // (high half) and sizes reported (low half); the child that reports last goes
-    // on with its parent.  After its own report it holds the vertex's preorder
-    // relative to an ancestor: offset (high half) and that ancestor (low half).
-    for (uint32_t v = tid; v < n; v += kThreads) {
-        acc[v] = 0;
-        vol[v] = (uint32_t)g.deg[v];
-    }
-    __syncthreads();
-    for (uint32_t v = tid; v < n; v += kThreads)
-        if (v != root) atomicAdd(&acc[nx[v] & kTarget], 1u << 16);
-    __syncthreads();
-    for (uint32_t v = tid; v < n; v += kThreads) {
-        if (*(volatile uint32_t *)&acc[v] != 0u) continue;  // has children
-        uint32_t x = v, sx = 1;
-        while (x != root) {
-            const uint32_t p = nx[x] & kTarget;
-            size[x] = (uint16_t)sx;
-            atomicAdd(&vol[p], *(volatile uint32_t *)&vol[x]);
-            __threadfence_block();
-            const uint32_t old = atomicAdd(&acc[p], sx - (1u << 16));
-            acc[x] = (((old & 0xFFFFu) + 1u) << 16) | p;
-            if ((old >> 16) != 1u) break;  // siblings still to report
-            __threadfence_block();
-            sx = 1u + (old & 0xFFFFu) + sx;
-            x = p;
+    if constexpr (kKind == kFused) {
+        // ---- sizes, volumes and preorder.  acc of a vertex: unreported children
+        // (high half) and sizes reported (low half); the child that reports last goes
+        // on with its parent.  After its own report it holds the vertex's preorder
+        // relative to an ancestor: offset (high half) and that ancestor (low half).
+        for (uint32_t v = tid; v < n; v += kThreads) {
+            acc[v] = 0;
+            vol[v] = (uint32_t)g.deg[v];
         }
-    }
-    __syncthreads();
-    if (tid == 0) acc[root] = root;
-    __syncthreads();
-    // pointer jumping in place: a pair is read and written whole, and holds at
-    // any time
-    for (uint32_t v = tid; v < n; v += kThreads) {
-        volatile uint32_t *pairs = acc;
-        uint32_t p = pairs[v];
-        while ((p & kTarget) != root) {
-            const uint32_t q = pairs[p & kTarget];
-            p = (((p >> 16) + (q >> 16)) << 16) | (q & kTarget);
-            pairs[v] = p;
-        }
-    }
-    __syncthreads();
-
-    // ---- f: every vertex walks up tau0 (as k_ttf_scan)
-    long long contrib = 0;
-    for (uint32_t v = tid; v < n; v += kThreads) {
-        if (v == root) continue;
-        const uint32_t inv = acc[v] >> 16;
-        long long q = 0;
-        uint32_t x = v;
-        for (int it = 0; x != root && it <= g.ecc; ++it) {
-            const uint32_t p0x = (uint32_t)g.p0[x];
-            if ((nx[x] & kTarget) == p0x) {
-                if (inv - (acc[x] >> 16) < size[x]) q += g.twom - (int64_t)vol[x];
-            } else if (p0x != root && (nx[p0x] & kTarget) == x) {
-                if (inv - (acc[p0x] >> 16) < size[p0x]) q -= g.twom - (int64_t)vol[p0x];
+        __syncthreads();
+        for (uint32_t v = tid; v < n; v += kThreads)
+            if (v != root) atomicAdd(&acc[nx[v] & kTarget], 1u << 16);
+        __syncthreads();
+        for (uint32_t v = tid; v < n; v += kThreads) {
+            if (*(volatile uint32_t *)&acc[v] != 0u) continue;  // has children
+            uint32_t x = v, sx = 1;
+            while (x != root) {
+                const uint32_t p = nx[x] & kTarget;
+                size[x] = (uint16_t)sx;
+                atomicAdd(&vol[p], *(volatile uint32_t *)&vol[x]);
+                __threadfence_block();
+                const uint32_t old = atomicAdd(&acc[p], sx - (1u << 16));
+                acc[x] = (((old & 0xFFFFu) + 1u) << 16) | p;
+                if ((old >> 16) != 1u) break;  // siblings still to report
+                __threadfence_block();
+                sx = 1u + (old & 0xFFFFu) + sx;
+                x = p;
             }
-            x = p0x;
         }
-        contrib += (long long)g.deg[v] * q;
-    }
+        __syncthreads();
+        if (tid == 0) acc[root] = root;
+        __syncthreads();
+        // pointer jumping in place: a pair is read and written whole, and holds at
+        // any time
+        for (uint32_t v = tid; v < n; v += kThreads) {
+            volatile uint32_t *pairs = acc;
+            uint32_t p = pairs[v];
+            while ((p & kTarget) != root) {
+                const uint32_t q = pairs[p & kTarget];
+                p = (((p >> 16) + (q >> 16)) << 16) | (q & kTarget);
+                pairs[v] = p;
+            }
+        }
+        __syncthreads();
+
+        // ---- f: every vertex walks up tau0 (as k_ttf_scan)
+        long long contrib = 0;
+        for (uint32_t v = tid; v < n; v += kThreads) {
+            if (v == root) continue;
+            const uint32_t inv = acc[v] >> 16;
+            long long q = 0;
+            uint32_t x = v;
+            for (int it = 0; x != root && it <= g.ecc; ++it) {
+                const uint32_t p0x = (uint32_t)g.p0[x];
+                if ((nx[x] & kTarget) == p0x) {
+                    if (inv - (acc[x] >> 16) < size[x]) q += g.twom - (int64_t)vol[x];
+                } else if (p0x != root && (nx[p0x] & kTarget) == x) {
+                    if (inv - (acc[p0x] >> 16) < size[p0x]) q -= g.twom - (int64_t)vol[p0x];
+                }
+                x = p0x;
+            }
+            contrib += (long long)g.deg[v] * q;
+        }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) contrib += __shfl_down_sync(kFull, contrib, o);
-    if ((tid & 31) == 0 && contrib != 0) atomicAdd(&s_f, (unsigned long long)contrib);
-    __syncthreads();
-    if (tid == 0) task.f[t] = (int64_t)s_f;
+        for (int o = 16; o > 0; o >>= 1) contrib += __shfl_down_sync(kFull, contrib, o);
+        if ((tid & 31) == 0 && contrib != 0) atomicAdd(&s_f, (unsigned long long)contrib);
+        __syncthreads();
+        if (tid == 0) task.f[t] = (int64_t)s_f;
+    }
 }
 
 // ---- larger trees, in memory ------------------------------------------------
@@ -257,7 +271,9 @@ __global__ void __launch_bounds__(256) k_first_arrows(PopTask task, int64_t B, u
     const int64_t t0 = (int64_t)blockIdx.y * kFirstTrees;
     const int64_t t1 = t0 + kFirstTrees < B ? t0 + kFirstTrees : B;
     for (int64_t t = t0; t < t1; ++t) {
-        uint64_t x = (uint64_t)(uint32_t)task.root | (uint64_t)kSettled << 32;
+        // settled words are not followed: the root's target is its parent, -1
+        uint64_t x = (uint64_t)kSettled << 32 |
+                     (v == task.root ? 0xFFFFFFFFu : (uint32_t)task.root);
         if (v != task.root && v != task.fixed) {
             const uint32_t k = bounded_draw_k(task.keys, task.seed, (uint32_t)v, 0,
                                               (uint32_t)task.sids[t], kTagWalk, (uint32_t)r.deg);
@@ -369,49 +385,84 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
     }
 }
 
-// parents of the finished maps, and the words zeroed for the traversal
-__global__ void __launch_bounds__(256) k_take_parents(int64_t n, int32_t root, uint64_t *words,
+// parents of the finished maps (all trees of a wave in one run of `count` words), and
+// the words zeroed for the traversal
+__global__ void __launch_bounds__(256) k_take_parents(int64_t count, uint64_t *words,
                                                       int32_t *par) {
-    const int64_t at = (int64_t)blockIdx.y * n;
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= n) return;
-    const int32_t p = w_next(words[at + v]);
-    words[at + v] = 0;
-    par[at + v] = v == root ? -1 : p;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    if (reinterpret_cast<uintptr_t>(words) & 15) {  // the first word alone
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            par[0] = w_next(words[0]);
+            words[0] = 0;
+        }
+        ++words;
+        ++par;
+        --count;
+    }
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; 2 * k + 1 < count; k += step) {
+        ulonglong2 *w = reinterpret_cast<ulonglong2 *>(words) + k;
+        const ulonglong2 x = *w;
+        *w = make_ulonglong2(0, 0);
+        par[2 * k] = w_next(x.x);
+        par[2 * k + 1] = w_next(x.y);
+    }
+    if ((count & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
+        par[count - 1] = w_next(words[count - 1]);
+        words[count - 1] = 0;
+    }
 }
 
-template <int kThreads, bool kMulti>
+constexpr int kMostDynamic = 224 * 1024;  // of 227 KB a block; the static part is small
+static_assert(kc_host::pop_small_bytes(kc_host::kPopSmallMax) <= kMostDynamic &&
+                  4 * kc_host::kPopTreesMax <= kMostDynamic,
+              "the largest trees fit a block");
+
+template <int kThreads, bool kMulti, int kKind>
 cudaError_t launch_small(const PopTask &one, const PopTask *tasks, const int2 *entry,
                          int64_t blocks, int64_t max_n, cudaStream_t s) {
-    const size_t bytes = kc_host::pop_small_bytes(max_n);
-    const cudaError_t e = cudaFuncSetAttribute(k_pop_small<kThreads, kMulti>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)bytes);
+    const size_t bytes =
+        kKind == kFused ? kc_host::pop_small_bytes(max_n) : sizeof(uint32_t) * (size_t)max_n;
+    // raised once per device, on the first call (a later one may be captured)
+    static std::atomic<uint64_t> raised{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    k_pop_small<kThreads, kMulti><<<(unsigned)blocks, kThreads, bytes, s>>>(one, tasks, entry);
+    if (dev >= 64 || !((raised.load() >> dev) & 1u)) {
+        e = cudaFuncSetAttribute(k_pop_small<kThreads, kMulti, kKind>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kMostDynamic);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) raised.fetch_or((uint64_t)1 << dev);
+    }
+    k_pop_small<kThreads, kMulti, kKind><<<(unsigned)blocks, kThreads, bytes, s>>>(one, tasks,
+                                                                                   entry);
     return cudaGetLastError();
 }
 
-template <bool kMulti>
+template <bool kMulti, int kKind>
 cudaError_t launch_small_any(const PopTask &one, const PopTask *tasks, const int2 *entry,
                              int64_t blocks, int64_t max_n, cudaStream_t s) {
     if (blocks <= 0) return cudaSuccess;
     switch (kc_host::pop_small_threads(max_n)) {
-        case 128: return launch_small<128, kMulti>(one, tasks, entry, blocks, max_n, s);
-        case 256: return launch_small<256, kMulti>(one, tasks, entry, blocks, max_n, s);
-        default: return launch_small<1024, kMulti>(one, tasks, entry, blocks, max_n, s);
+        case 128: return launch_small<128, kMulti, kKind>(one, tasks, entry, blocks, max_n, s);
+        case 256: return launch_small<256, kMulti, kKind>(one, tasks, entry, blocks, max_n, s);
+        default: return launch_small<1024, kMulti, kKind>(one, tasks, entry, blocks, max_n, s);
     }
 }
 
 }  // namespace
 
 cudaError_t launch_pop_small(const PopTask &task, int64_t B, cudaStream_t s) {
-    return launch_small_any<false>(task, nullptr, nullptr, B, task.g.n, s);
+    return launch_small_any<false, kFused>(task, nullptr, nullptr, B, task.g.n, s);
+}
+
+cudaError_t launch_pop_trees(const PopTask &task, int64_t B, cudaStream_t s) {
+    return task.g.rec ? launch_small_any<false, kTrees>(task, nullptr, nullptr, B, task.g.n, s)
+                      : launch_small_any<false, kTreesCsr>(task, nullptr, nullptr, B, task.g.n, s);
 }
 
 cudaError_t launch_pop_small_multi(const PopTask *tasks, const int2 *entry, int64_t count,
                                    int64_t max_n, cudaStream_t s) {
-    return launch_small_any<true>(PopTask{}, tasks, entry, count, max_n, s);
+    return launch_small_any<true, kFused>(PopTask{}, tasks, entry, count, max_n, s);
 }
 
 cudaError_t launch_pop_large(const PopTask &task, int64_t B, uint64_t *words, int32_t *lists0,
@@ -428,7 +479,8 @@ cudaError_t launch_pop_large(const PopTask &task, int64_t B, uint64_t *words, in
         k_pop_rounds<1024><<<(unsigned)B, 1024, 0, s>>>(task, words, lists0, lists1, count);
     else
         k_pop_rounds<256><<<(unsigned)B, 256, 0, s>>>(task, words, lists0, lists1, count);
-    k_take_parents<<<dim3(rows, (unsigned)B), 256, 0, s>>>(n, task.root, words, task.par);
+    k_take_parents<<<(unsigned)std::min<int64_t>((B * n + 511) / 512, 32 * num_sms), 256, 0, s>>>(
+        B * n, words, task.par);
     return cudaGetLastError();
 }
 

@@ -408,6 +408,7 @@ PopTask pop_task(const kc_graph *g, const GraphView &gv, const WaveView &w, cons
     k.keys = host_keys(g->seed);
     k.step_cap = step_cap_of(g);
     k.sids = sids;
+    k.first_sid = 0;
     k.steps = w.steps;
     k.f = want_f ? w.f : nullptr;
     k.par = store;
@@ -1237,12 +1238,13 @@ void resample_slots(kc_graph *g, const std::vector<int64_t> &slots, bool cond, i
             const PopTask task = pop_task(g, gv, w, c.sids, cond ? v : g->root, cond ? u : -1,
                                           false, w.ord);
             KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
-            if (pop == kPopSmall)
-                KC_CK(g, launch_pop_small(task, b, g->stream));
+            const bool block = g->n <= kc_host::kPopTreesMax;
+            if (block)
+                KC_CK(g, launch_pop_trees(task, b, g->stream));
             else
                 KC_CK(g, launch_pop_large(task, b, w.word, w.size, w.din, w.f, g->num_sms,
                                           g->stream));
-            g->t_update.launches += pop == kPopSmall ? 1 : 4;
+            g->t_update.launches += block ? 1 : 4;
             uint32_t err = 0;
             KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
             if (solo_retry(g, err)) pop = kPopNone;

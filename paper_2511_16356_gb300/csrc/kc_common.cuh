@@ -464,17 +464,23 @@ struct PopTask {
     PhiloxKeys keys;          // of the seed
     int64_t step_cap;         // departures of a tree past which it fails (kErrStepLimit)
     const int64_t *sids;      // [B]
+    int64_t first_sid;        // without records: the sample ids are first_sid + t
     int64_t *steps;           // [B]
-    int64_t *f;               // [B], or null: trees only
-    int32_t *par;             // [B][n] parents (-1 at the root), or null
+    int64_t *f;               // [B] (launch_pop_small and its batched form)
+    int32_t *par;             // [B][n] parents (-1 at the root); there it may be null
     uint32_t *err;
 };
+constexpr int64_t kPopRedo = -2;  // steps of a tree that launch_pop_trees could not finish
 // n at most kc_host::kPopSmallMax, 2m < 2^32: trees and f from shared memory
 cudaError_t launch_pop_small(const PopTask &task, int64_t B, cudaStream_t s);
 // any n: trees in memory.  words [B][n] (left zeroed), two lists [B][n], found [B];
 // task.par receives the parents, task.f is not used.  B at most 65535.
 cudaError_t launch_pop_large(const PopTask &task, int64_t B, uint64_t *words, int32_t *lists0,
                              int32_t *lists1, int64_t *found, int64_t num_sms, cudaStream_t s);
+// n at most kc_host::kPopTreesMax: trees only, from shared memory.  Without records
+// (task.g.rec null) the arrows come from the CSR arrays and a tree past the step cap
+// or the pop counts gets steps = kPopRedo instead of an error.
+cudaError_t launch_pop_trees(const PopTask &task, int64_t B, cudaStream_t s);
 // entries (task, tree) of a device table of tasks; max_n: their largest n
 cudaError_t launch_pop_small_multi(const PopTask *tasks, const int2 *entry, int64_t count,
                                    int64_t max_n, cudaStream_t s);

@@ -132,3 +132,30 @@ def test_popped_trees_in_memory_match_oracle(trees):
         tr, ref = G.tree(trees - 1), O.tree(g, t0, 43, trees - 1)
         for key in ("parent", "depth", "din", "dout", "vol"):
             assert np.array_equal(tr[key], getattr(ref, key)), key
+
+
+@pytest.mark.parametrize("n,trees", [(2, 5), (1000, 40), (5000, 20), (56000, 3), (56001, 3)])
+@pytest.mark.parametrize("cap", [0, 30000])
+def test_trees_without_allocation_match_oracle(n, trees, cap):
+    """kc_wilson_noalloc at the edges of its two ways: trees, step counts and the
+    status, also where some trees pass the step cap."""
+    torch = pytest.importorskip("torch")
+    g = S.complete(2) if n == 2 else S.complete_bipartite(25, n - 25)
+    t0 = O.tau0(g)
+    ro, co = torch.from_numpy(g.row_off).cuda(), torch.from_numpy(g.col).cuda()
+    par = torch.full((trees, n), -7, dtype=torch.int32, device="cuda")
+    steps = torch.zeros(trees, dtype=torch.int64, device="cuda")
+    status = torch.full((1,), 5, dtype=torch.int32, device="cuda")
+    st = kc.load().kc_wilson_noalloc(n, ro.data_ptr(), co.data_ptr(), t0.r, 71, 4, trees, cap,
+                                     par.data_ptr(), steps.data_ptr(), status.data_ptr(),
+                                     torch.cuda.current_stream().cuda_stream)
+    assert st == kc.KC_OK
+    torch.cuda.synchronize()
+    _, want = O.sample_batch(g, t0, 71, 4, trees)
+    over = want > cap if cap else want < 0
+    got = steps.cpu().numpy()
+    assert int(status.item()) == int(over.any())
+    assert np.array_equal(got[~over], want[~over])
+    assert np.all(got[over] == cap + 1)
+    for k in np.flatnonzero(~over)[:3]:
+        assert np.array_equal(par[k].cpu().numpy(), O.tree(g, t0, 71, 4 + int(k)).parent)
