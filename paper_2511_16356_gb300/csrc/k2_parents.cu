@@ -176,13 +176,12 @@ __global__ void k_par_depth_init(GraphView g, WaveView w, ParTrees trees) {
 
 }  // namespace
 
-cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool zeroed,
-                                    bool by_id, int32_t eu, int32_t ev, bool want_preorder,
-                                    cudaStream_t s, int *launches) {
+cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool by_id,
+                                    int32_t eu, int32_t ev, bool want_preorder, cudaStream_t s,
+                                    int *launches) {
     const size_t per = (size_t)(w.B * g.n);
     cudaError_t e;
-    if (!zeroed && (e = cudaMemsetAsync(w.word, 0, sizeof(uint64_t) * per, s)) != cudaSuccess)
-        return e;
+    if ((e = cudaMemsetAsync(w.word, 0, sizeof(uint64_t) * per, s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(w.vol, 0, sizeof(int64_t) * per, s)) != cudaSuccess) return e;
     const dim3 grid((unsigned)std::min<int64_t>((g.n + 255) / 256, 4096), (unsigned)w.B);
     k_par_count<<<grid, 256, 0, s>>>(g.n, w, trees);

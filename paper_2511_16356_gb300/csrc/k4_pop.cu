@@ -18,6 +18,13 @@
 // vertices that does not hold a).  Settled paths are never followed again, so all
 // rounds together settle each vertex once.
 //
+// Once few vertices are active, the round works on the map that they form: each
+// follows the arrows to the next active vertex only, and that map is squared until
+// its images are the vertices on its cycles (contracted_round); each of those lists
+// its own piece of the cycle.  A round of some 50 active vertices then costs its
+// longest piece where the leaders' loops went around several times: 2000 trees of a
+// random graph of 2000 vertices (kc_wilson_noalloc) 2.62 -> 2.23 ms.
+//
 // k_pop_small keeps the tree in shared memory: 14 bytes a vertex.  Larger trees
 // stay in memory: the first arrows (k_first_arrows) and the cycles of the first map
 // (k_first_cycles) are passes over all vertices of all trees, the rounds after it,
@@ -41,11 +48,46 @@ namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// Vertex word in shared memory: target (16 bits), pops (14), settled, active
+// Vertex word in shared memory: target (16 bits), pops (13), on a cycle, settled,
+// active
 constexpr uint32_t kActive = 1u << 31;
 constexpr uint32_t kSettled = 1u << 30;
+constexpr uint32_t kOnCycle = 1u << 29;
 constexpr uint32_t kTarget = 0xFFFFu;
-constexpr uint32_t kSmallMostPops = 0x3FFFu;
+constexpr uint32_t kSmallMostPops = 0x1FFFu;
+
+// Squares the map `next` of the `active` vertices list[] (-1: leads to the root)
+// until every image lies on a cycle of it.  The whole block calls; each thread holds
+// up to kHold vertices.
+constexpr int kHold = 4;
+template <int kThreads, class Vertex, class Hop>
+__device__ __forceinline__ void square_map(const Vertex *list, uint32_t active, Hop *next) {
+    const Hop none = (Hop)-1;
+    volatile Hop *map = next;
+    const int rounds = 32 - __clz(active);  // 2^rounds > active
+    const bool warp = active <= 32 * kHold;  // one warp holds them all
+    const uint32_t step = warp ? 32 : kThreads;
+    if (!warp || threadIdx.x < 32) {
+        for (int r = 0; r < rounds; ++r) {
+            Hop h[kHold];
+#pragma unroll
+            for (int j = 0; j < kHold; ++j) {
+                const uint32_t i = threadIdx.x + j * step;
+                h[j] = none;
+                if (i < active) h[j] = map[list[i]];
+                if (h[j] != none) h[j] = map[h[j]];
+            }
+            if (warp) __syncwarp(); else __syncthreads();
+#pragma unroll
+            for (int j = 0; j < kHold; ++j) {
+                const uint32_t i = threadIdx.x + j * step;
+                if (i < active) map[list[i]] = h[j];
+            }
+            if (warp) __syncwarp(); else __syncthreads();
+        }
+    }
+    __syncthreads();
+}
 
 // The length of the cycle that active vertex a leads, or 0 (see above).
 __device__ __forceinline__ uint32_t led_cycle(volatile uint32_t *nx, uint32_t a) {
@@ -75,7 +117,8 @@ __device__ __forceinline__ uint32_t led_cycle(volatile uint32_t *nx, uint32_t a)
 }
 
 // kKind: kFused evaluates f; kTrees leaves the parents in task.par only (whose row
-// holds the two lists meanwhile) and needs 4 bytes a vertex; kTreesCsr does so
+// holds the two lists meanwhile) and needs 6 bytes a vertex (4, past
+// kPopContractMax, without contracted rounds); kTreesCsr does so
 // from the CSR arrays alone, and marks a tree that it cannot finish kPopRedo
 // instead of raising an error.
 enum : int { kFused = 0, kTrees = 1, kTreesCsr = 2 };
@@ -98,6 +141,8 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 12 : (kThreads <= 
     uint16_t *list = kKind == kFused ? reinterpret_cast<uint16_t *>(acc)
                                      : reinterpret_cast<uint16_t *>(task.par + t * n);
     uint16_t *fresh = list + n;
+    uint16_t *next = reinterpret_cast<uint16_t *>(kKind == kFused ? vol : smem + n);  // [n]
+    const bool contract = kKind == kFused || n <= kc_host::kPopContractMax;
     __shared__ uint32_t s_count[2];
     __shared__ unsigned long long s_f;
 
@@ -128,22 +173,65 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 12 : (kThreads <= 
     int64_t pops = 0;
     int end = 0;
     for (int round = 0;; ++round) {
-        for (uint32_t i = tid; i < active; i += kThreads) {
-            const uint32_t a = round == 0 ? i : list[i];
-            if (nx[a] & kSettled) continue;
-            const uint32_t len = led_cycle(nx, a);
-            if (len == 0) continue;
-            uint32_t x = a, at = atomicAdd(&s_count[round & 1], len);
-            do {
-                fresh[at++] = (uint16_t)x;
-                x = nx[x] & kTarget;
-            } while (x != a);
+        if (round > 0 && contract && active <= kHold * kThreads) {
+            volatile uint32_t *vx = nx;
+            uint32_t len[kHold];
+            for (int j = 0; j < kHold; ++j) {
+                const uint32_t i = tid + j * kThreads;
+                if (i >= active) break;
+                const uint32_t a = list[i];
+                uint32_t x = vx[a] & kTarget, w = vx[x], l = 1;
+                for (; w < kSettled; ++l) {
+                    x = w & kTarget;
+                    w = vx[x];
+                }
+                len[j] = l;
+                next[a] = (w & kSettled) ? (uint16_t)0xFFFFu : (uint16_t)x;
+            }
+            __syncthreads();
+            square_map<kThreads>(list, active, next);
+            for (uint32_t i = tid; i < active; i += kThreads) {
+                const uint32_t h = next[list[i]];
+                if (h != 0xFFFFu) vx[h] = vx[h] | kOnCycle;
+            }
+            __syncthreads();
+            for (int j = 0; j < kHold; ++j) {
+                const uint32_t i = tid + j * kThreads;
+                if (i >= active) break;
+                uint32_t x = list[i], w = vx[x];
+                if (w & kOnCycle) {  // its piece of the cycle
+                    uint32_t at = atomicAdd(&s_count[round & 1], len[j]);
+                    do {
+                        fresh[at++] = (uint16_t)x;
+                        x = w & kTarget;
+                        w = vx[x];
+                    } while (!(w & kActive));
+                } else if (next[x] == 0xFFFFu) {  // its piece of a path to the root
+                    do {
+                        vx[x] = w | kSettled;
+                        x = w & kTarget;
+                        w = vx[x];
+                    } while (w < kSettled);
+                }
+            }
+        } else {
+            for (uint32_t i = tid; i < active; i += kThreads) {
+                const uint32_t a = round == 0 ? i : list[i];
+                if (nx[a] & kSettled) continue;
+                const uint32_t len = led_cycle(nx, a);
+                if (len == 0) continue;
+                uint32_t x = a, at = atomicAdd(&s_count[round & 1], len);
+                do {
+                    fresh[at++] = (uint16_t)x;
+                    x = nx[x] & kTarget;
+                } while (x != a);
+            }
         }
         __syncthreads();
         const uint32_t found = s_count[round & 1];
         for (uint32_t i = tid; i < active; i += kThreads) {
             const uint32_t a = round == 0 ? i : list[i];
-            nx[a] &= ~kActive;
+            nx[a] &= ~(kActive | kOnCycle);
         }
         if (tid == 0) s_count[(round + 1) & 1] = 0;
         if (found == 0) break;
@@ -253,7 +341,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 12 : (kThreads <= 
 }
 
 // ---- larger trees, in memory ------------------------------------------------
-// Vertex word: target (low half); pops, settled (bit 30), active (bit 31).
+// Vertex word: target (low half); pops and the three flags above.
 __device__ __forceinline__ uint64_t large_arrow(const PopTask &task, uint32_t sample, uint32_t v,
                                                 uint32_t count) {
     const VRec r = load_rec(task.g.rec + v);
@@ -335,12 +423,12 @@ __global__ void __launch_bounds__(256) k_first_cycles(int64_t n, uint64_t *words
 
 template <int kThreads>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
-    k_pop_rounds(PopTask task, uint64_t *words, int32_t *lists0, int32_t *lists1,
+    k_pop_rounds(PopTask task, uint64_t *words, int32_t *lists0, int32_t *lists1, int32_t *nexts,
                  const unsigned long long *found0) {
     const int64_t t = blockIdx.x, n = task.g.n;
     const uint32_t sample = (uint32_t)task.sids[t], tid = threadIdx.x;
     uint64_t *word = words + t * n;
-    int32_t *list = lists0 + t * n, *fresh = lists1 + t * n;
+    int32_t *list = lists0 + t * n, *fresh = lists1 + t * n, *next = nexts + t * n;
     __shared__ uint32_t s_count[2];
     uint32_t active = (uint32_t)found0[t];
     int64_t pops = 0;
@@ -356,7 +444,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
         bool full = false;
         for (uint32_t i = tid; i < active; i += kThreads) {
             const int32_t v = list[i];
-            const uint32_t c = (uint32_t)(word[v] >> 32) + 1;
+            const uint32_t c = ((uint32_t)(word[v] >> 32) & (kOnCycle - 1u)) + 1;
             word[v] = large_arrow(task, sample, (uint32_t)v, c) | (uint64_t)(c | kActive) << 32;
             full = full || c >= kWalkCountMask;
         }
@@ -364,15 +452,62 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
             end = kErrCountField;
             break;
         }
-        for (uint32_t i = tid; i < active; i += kThreads) {
-            const int32_t a = list[i];
-            if ((word[a] >> 32) & kSettled) continue;
-            const int32_t len = led_cycle_large<false>(word, a);
-            if (len) list_cycle(word, fresh, atomicAdd(&s_count[round & 1], (uint32_t)len), a);
+        if (active <= kHold * kThreads) {
+            const uint64_t settled = (uint64_t)kSettled << 32;
+            uint32_t len[kHold];
+            for (int j = 0; j < kHold; ++j) {
+                const uint32_t i = tid + j * kThreads;
+                if (i >= active) break;
+                const int32_t a = list[i];
+                int32_t x = w_next(word[a]);
+                uint64_t w = word[x];
+                uint32_t l = 1;
+                for (; w < settled; ++l) {
+                    x = w_next(w);
+                    w = word[x];
+                }
+                len[j] = l;
+                next[a] = (w & settled) ? -1 : x;
+            }
+            __syncthreads();
+            square_map<kThreads>(list, active, next);
+            for (uint32_t i = tid; i < active; i += kThreads) {
+                const int32_t h = next[list[i]];
+                if (h >= 0) word[h] |= (uint64_t)kOnCycle << 32;
+            }
+            __syncthreads();
+            for (int j = 0; j < kHold; ++j) {
+                const uint32_t i = tid + j * kThreads;
+                if (i >= active) break;
+                int32_t x = list[i];
+                uint64_t w = word[x];
+                if ((w >> 32) & kOnCycle) {  // its piece of the cycle
+                    uint32_t at = atomicAdd(&s_count[round & 1], len[j]);
+                    do {
+                        fresh[at++] = x;
+                        x = w_next(w);
+                        w = word[x];
+                    } while (!((w >> 32) & kActive));
+                } else if (next[x] < 0) {  // its piece of a path to the root
+                    do {
+                        word[x] = w | settled;
+                        x = w_next(w);
+                        w = word[x];
+                    } while (w < settled);
+                }
+            }
+        } else {
+            for (uint32_t i = tid; i < active; i += kThreads) {
+                const int32_t a = list[i];
+                if ((word[a] >> 32) & kSettled) continue;
+                const int32_t len = led_cycle_large<false>(word, a);
+                if (len)
+                    list_cycle(word, fresh, atomicAdd(&s_count[round & 1], (uint32_t)len), a);
+            }
         }
         __syncthreads();
         for (uint32_t i = tid; i < active; i += kThreads)
-            word[list[i]] &= ~((uint64_t)kActive << 32);
+            word[list[i]] &= ~((uint64_t)(kActive | kOnCycle) << 32);
         active = s_count[round & 1];
         if (tid == 0) s_count[(round + 1) & 1] = 0;
         int32_t *const swap = list;
@@ -385,43 +520,27 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
     }
 }
 
-// parents of the finished maps (all trees of a wave in one run of `count` words), and
-// the words zeroed for the traversal
-__global__ void __launch_bounds__(256) k_take_parents(int64_t count, uint64_t *words,
+// Parents of the finished maps, all trees of a wave in one run of `count` words.  It
+// only reads the words: clearing them on the way for the traversal took 14 ms for
+// 768 million of them, reading and then clearing takes 1.3 and 0.9.
+__global__ void __launch_bounds__(256) k_take_parents(int64_t count, const uint64_t *words,
                                                       int32_t *par) {
-    const int64_t step = (int64_t)gridDim.x * blockDim.x;
-    if (reinterpret_cast<uintptr_t>(words) & 15) {  // the first word alone
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            par[0] = w_next(words[0]);
-            words[0] = 0;
-        }
-        ++words;
-        ++par;
-        --count;
-    }
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; 2 * k + 1 < count; k += step) {
-        ulonglong2 *w = reinterpret_cast<ulonglong2 *>(words) + k;
-        const ulonglong2 x = *w;
-        *w = make_ulonglong2(0, 0);
-        par[2 * k] = w_next(x.x);
-        par[2 * k + 1] = w_next(x.y);
-    }
-    if ((count & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
-        par[count - 1] = w_next(words[count - 1]);
-        words[count - 1] = 0;
-    }
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count;
+         k += (int64_t)gridDim.x * blockDim.x)
+        par[k] = w_next(words[k]);
 }
 
 constexpr int kMostDynamic = 224 * 1024;  // of 227 KB a block; the static part is small
 static_assert(kc_host::pop_small_bytes(kc_host::kPopSmallMax) <= kMostDynamic &&
-                  4 * kc_host::kPopTreesMax <= kMostDynamic,
+                  kc_host::pop_trees_bytes(kc_host::kPopContractMax) <= kMostDynamic &&
+                  kc_host::pop_trees_bytes(kc_host::kPopTreesMax) <= kMostDynamic,
               "the largest trees fit a block");
 
 template <int kThreads, bool kMulti, int kKind>
 cudaError_t launch_small(const PopTask &one, const PopTask *tasks, const int2 *entry,
                          int64_t blocks, int64_t max_n, cudaStream_t s) {
     const size_t bytes =
-        kKind == kFused ? kc_host::pop_small_bytes(max_n) : sizeof(uint32_t) * (size_t)max_n;
+        kKind == kFused ? kc_host::pop_small_bytes(max_n) : kc_host::pop_trees_bytes(max_n);
     // raised once per device, on the first call (a later one may be captured)
     static std::atomic<uint64_t> raised{0};
     int dev = 0;
@@ -466,7 +585,8 @@ cudaError_t launch_pop_small_multi(const PopTask *tasks, const int2 *entry, int6
 }
 
 cudaError_t launch_pop_large(const PopTask &task, int64_t B, uint64_t *words, int32_t *lists0,
-                             int32_t *lists1, int64_t *found, int64_t num_sms, cudaStream_t s) {
+                             int32_t *lists1, int32_t *nexts, int64_t *found, int64_t num_sms,
+                             cudaStream_t s) {
     const int64_t n = task.g.n;
     const cudaError_t e = cudaMemsetAsync(found, 0, sizeof(int64_t) * (size_t)B, s);
     if (e != cudaSuccess) return e;
@@ -476,10 +596,10 @@ cudaError_t launch_pop_large(const PopTask &task, int64_t B, uint64_t *words, in
         task, B, words);
     k_first_cycles<<<dim3(rows, (unsigned)B), 256, 0, s>>>(n, words, lists0, count);
     if (B <= num_sms)
-        k_pop_rounds<1024><<<(unsigned)B, 1024, 0, s>>>(task, words, lists0, lists1, count);
+        k_pop_rounds<1024><<<(unsigned)B, 1024, 0, s>>>(task, words, lists0, lists1, nexts, count);
     else
-        k_pop_rounds<256><<<(unsigned)B, 256, 0, s>>>(task, words, lists0, lists1, count);
-    k_take_parents<<<(unsigned)std::min<int64_t>((B * n + 511) / 512, 32 * num_sms), 256, 0, s>>>(
+        k_pop_rounds<256><<<(unsigned)B, 256, 0, s>>>(task, words, lists0, lists1, nexts, count);
+    k_take_parents<<<(unsigned)std::min<int64_t>((B * n + 255) / 256, 64 * num_sms), 256, 0, s>>>(
         B * n, words, task.par);
     return cudaGetLastError();
 }

@@ -693,8 +693,8 @@ bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
                 Phase ph(g, g->t_wilson);
                 KC_CK(g, launch_pop_large(pop_task(g, gv, sv, c.sids + sub, g->root, -1, false,
                                                    par),
-                                          sv.B, sv.word, sv.size, sv.din, sv.f, g->num_sms,
-                                          g->stream));
+                                          sv.B, sv.word, sv.size, sv.din, (int32_t *)sv.vol, sv.f,
+                                          g->num_sms, g->stream));
                 ph.done(4);
             }
             KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
@@ -702,8 +702,8 @@ bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
             {
                 Phase ph(g, g->t_traverse);
                 int nl = 0;
-                KC_CK(g, launch_traverse_parents(gv, sv, ParTrees{par, nullptr}, true, false, -1,
-                                                 -1, false, g->stream, &nl));
+                KC_CK(g, launch_traverse_parents(gv, sv, ParTrees{par, nullptr}, false, -1, -1,
+                                                 false, g->stream, &nl));
                 ph.done(nl);
             }
             {
@@ -992,7 +992,7 @@ void traverse_tau0(kc_graph *g, int &launches) {
     int nl = 0;
     if (g->ecc <= n / 64) {
         KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
-        KC_CK(g, launch_traverse_parents(gv, w, ParTrees{g->d_p0, nullptr}, false, true, -1, -1,
+        KC_CK(g, launch_traverse_parents(gv, w, ParTrees{g->d_p0, nullptr}, true, -1, -1,
                                          false, g->stream, &nl));
         uint32_t err = 0;
         KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
@@ -1184,7 +1184,7 @@ void refresh_slots(kc_graph *g, const std::vector<int64_t> &slots) {
         if (!p.bit) {  // any valid DFN serves the tau0 scan
             const ParTrees trees{g->d_parents, ub.slots};
             int nl = 0;
-            KC_CK(g, launch_traverse_parents(gv, w, trees, false, false, -1, -1, false,
+            KC_CK(g, launch_traverse_parents(gv, w, trees, false, -1, -1, false,
                                              g->stream, &nl));
             KC_CK(g, launch_ttf_scan_parents(gv, w, trees, g->stream));
             KC_CK(g, launch_scatter_results(ub.slots, b, w.f, nullptr, nullptr, g->d_f,
@@ -1242,8 +1242,8 @@ void resample_slots(kc_graph *g, const std::vector<int64_t> &slots, bool cond, i
             if (block)
                 KC_CK(g, launch_pop_trees(task, b, g->stream));
             else
-                KC_CK(g, launch_pop_large(task, b, w.word, w.size, w.din, w.f, g->num_sms,
-                                          g->stream));
+                KC_CK(g, launch_pop_large(task, b, w.word, w.size, w.din, (int32_t *)w.vol, w.f,
+                                          g->num_sms, g->stream));
             g->t_update.launches += block ? 1 : 4;
             uint32_t err = 0;
             KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
@@ -1300,7 +1300,7 @@ void transform_slots(kc_graph *g, const std::vector<int64_t> &slots, bool insert
         // DFN serves; cut-link picks the k-th crossing edge in the id-ordered
         // preorder, and its trees hold the edge that the graph has lost
         int nl = 0;
-        KC_CK(g, launch_traverse_parents(gv, w, ParTrees{g->d_parents, ub.slots}, false, !insert,
+        KC_CK(g, launch_traverse_parents(gv, w, ParTrees{g->d_parents, ub.slots}, !insert,
                                          insert ? -1 : u, insert ? -1 : v, true, g->stream, &nl));
         KC_CK(g, launch_link_cut(g->d_row_off, g->d_col, w, ub.slots, g->d_parents, ub.factor,
                                  ub.cut, g->root, u, v, g->seed, (uint32_t)g->update_seq, insert,
@@ -2502,7 +2502,7 @@ kc_status kc_get_tree(kc_graph *g, int64_t sample, int32_t *parent, int32_t *dep
             w.B = 1;
             const ParTrees tree{g->d_parents + sample * n, nullptr};
             KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
-            KC_CK(g, launch_traverse_parents(gv, w, tree, false, true, -1, -1, false, g->stream));
+            KC_CK(g, launch_traverse_parents(gv, w, tree, true, -1, -1, false, g->stream));
             check_err(g, "get_tree");
             std::vector<int32_t> din((size_t)n), size((size_t)n);
             KC_CK(g, copy_sync(g, din.data(), w.din, n4, cudaMemcpyDeviceToHost));

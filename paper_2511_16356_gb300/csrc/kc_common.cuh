@@ -473,10 +473,11 @@ struct PopTask {
 constexpr int64_t kPopRedo = -2;  // steps of a tree that launch_pop_trees could not finish
 // n at most kc_host::kPopSmallMax, 2m < 2^32: trees and f from shared memory
 cudaError_t launch_pop_small(const PopTask &task, int64_t B, cudaStream_t s);
-// any n: trees in memory.  words [B][n] (left zeroed), two lists [B][n], found [B];
+// any n: trees in memory.  words, two lists and a map, [B][n] each, found [B];
 // task.par receives the parents, task.f is not used.  B at most 65535.
 cudaError_t launch_pop_large(const PopTask &task, int64_t B, uint64_t *words, int32_t *lists0,
-                             int32_t *lists1, int64_t *found, int64_t num_sms, cudaStream_t s);
+                             int32_t *lists1, int32_t *nexts, int64_t *found, int64_t num_sms,
+                             cudaStream_t s);
 // n at most kc_host::kPopTreesMax: trees only, from shared memory.  Without records
 // (task.g.rec null) the arrows come from the CSR arrays and a tree past the step cap
 // or the pop counts gets steps = kPopRedo instead of an error.
@@ -519,12 +520,11 @@ struct ParTrees {
 };
 // Order-free traversal (k2_parents.cu): w.size, w.vol and w.din (by_id: the DFN with
 // children in ascending id, else some valid one), w.aux the preorder if wanted;
-// w.word is scratch (zeroed: it is zero already).  (eu, ev): an edge that the trees
-// may hold and the graph does not (eu < 0: none), needed with by_id.  w.B at most
-// 65535.
-cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool zeroed,
-                                    bool by_id, int32_t eu, int32_t ev, bool want_preorder,
-                                    cudaStream_t s, int *launches = nullptr);
+// w.word is scratch.  (eu, ev): an edge that the trees may hold and the graph does
+// not (eu < 0: none), needed with by_id.  w.B at most 65535.
+cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool by_id,
+                                    int32_t eu, int32_t ev, bool want_preorder, cudaStream_t s,
+                                    int *launches = nullptr);
 // depths of the trees into w.din; w.word is scratch
 cudaError_t launch_depths_parents(const GraphView &g, WaveView w, ParTrees trees,
                                   cudaStream_t s);

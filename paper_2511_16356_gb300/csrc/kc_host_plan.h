@@ -127,8 +127,11 @@ inline int queue_group(int64_t B, int64_t num_sms) {
 // (227 KB a block, less its static part) and the threads of a block.
 constexpr size_t pop_small_bytes(int64_t n) { return (size_t)n * 12 + ((size_t)n * 2 + 3) / 4 * 4; }
 constexpr int64_t kPopSmallMax = 16000;
-// Trees without f hold 4 bytes a vertex there.
-constexpr int64_t kPopTreesMax = 56000;
+// Trees without f hold 6 bytes a vertex there, past kPopContractMax 4.
+constexpr int64_t kPopContractMax = 38000, kPopTreesMax = 56000;
+constexpr size_t pop_trees_bytes(int64_t n) {
+    return (size_t)n * (n <= kPopContractMax ? 6 : 4);
+}
 // Whether popping pays: its rounds follow the longest loops, which are long where
 // the first walk is -- the walk to the root takes about 2m / deg(root) departures.
 // Power-law graphs (a hub as the root): 10000 vertices, 500 trees 5.26 -> 1.27 ms
