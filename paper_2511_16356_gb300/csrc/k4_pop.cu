@@ -68,20 +68,29 @@ __device__ __forceinline__ void square_map(const Vertex *list, uint32_t active, 
     const bool warp = active <= 32 * kHold;  // one warp holds them all
     const uint32_t step = warp ? 32 : kThreads;
     if (!warp || threadIdx.x < 32) {
+        Vertex a[kHold];
+        Hop h[kHold];
+#pragma unroll
+        for (int j = 0; j < kHold; ++j) {
+            const uint32_t i = threadIdx.x + j * step;
+            a[j] = 0;
+            h[j] = none;
+            if (i < active) {
+                a[j] = list[i];
+                h[j] = map[a[j]];
+            }
+        }
         for (int r = 0; r < rounds; ++r) {
-            Hop h[kHold];
 #pragma unroll
             for (int j = 0; j < kHold; ++j) {
-                const uint32_t i = threadIdx.x + j * step;
-                h[j] = none;
-                if (i < active) h[j] = map[list[i]];
+                if (j * step >= active) break;
                 if (h[j] != none) h[j] = map[h[j]];
             }
             if (warp) __syncwarp(); else __syncthreads();
 #pragma unroll
             for (int j = 0; j < kHold; ++j) {
-                const uint32_t i = threadIdx.x + j * step;
-                if (i < active) map[list[i]] = h[j];
+                if (j * step >= active) break;
+                if (threadIdx.x + j * step < active) map[a[j]] = h[j];
             }
             if (warp) __syncwarp(); else __syncthreads();
         }
@@ -123,7 +132,7 @@ __device__ __forceinline__ uint32_t led_cycle(volatile uint32_t *nx, uint32_t a)
 // instead of raising an error.
 enum : int { kFused = 0, kTrees = 1, kTreesCsr = 2 };
 template <int kThreads, bool kMulti, int kKind>
-__global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 12 : (kThreads <= 256 ? 6 : 1))
+__global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 10 : (kThreads <= 256 ? 5 : 1))
     k_pop_small(PopTask one, const PopTask *__restrict__ tasks, const int2 *__restrict__ entry) {
     const int64_t t = kMulti ? (int64_t)entry[blockIdx.x].y : (int64_t)blockIdx.x;
     const PopTask task = kMulti ? tasks[entry[blockIdx.x].x] : one;
@@ -180,10 +189,24 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 12 : (kThreads <= 
                 const uint32_t i = tid + j * kThreads;
                 if (i >= active) break;
                 const uint32_t a = list[i];
-                uint32_t x = vx[a] & kTarget, w = vx[x], l = 1;
-                for (; w < kSettled; ++l) {
-                    x = w & kTarget;
+                // three hops a test: every word's target is a vertex, so a hop
+                // past the end is only wasted, and a test between two hops would
+                // wait for the first
+                uint32_t x = vx[a] & kTarget, w, l = 1;
+                for (;; l += 3) {
                     w = vx[x];
+                    const uint32_t x1 = w & kTarget, w1 = vx[x1];
+                    const uint32_t x2 = w1 & kTarget, w2 = vx[x2];
+                    if ((w | w1 | w2) < kSettled) {
+                        x = w2 & kTarget;
+                        continue;
+                    }
+                    if (w >= kSettled) break;
+                    const bool first = w1 >= kSettled;
+                    x = first ? x1 : x2;
+                    w = first ? w1 : w2;
+                    l += first ? 1 : 2;
+                    break;
                 }
                 len[j] = l;
                 next[a] = (w & kSettled) ? (uint16_t)0xFFFFu : (uint16_t)x;
