@@ -12,13 +12,9 @@
 //        and test tau-ancestry with the DFN intervals of tau: O(n ecc) work, all
 //        vertices of all trees in parallel.  Used when the depth is small (the
 //        O(n Delta) bound of Thm 8).
-//  BIT:  Algorithm 1: a DFS over tau in preorder keeps, for the tau-ancestors of
-//        the current vertex, range adds over tau0-DFN intervals in a Fenwick
-//        array and queries the point in0(v).  O(n log n) per tree.  A warp owns a
-//        tree and handles 32 preorder positions per round: all 32 point queries
-//        are loaded first, then the 32 visits are replayed in lane order with the
-//        stack held in registers, each range add both issued to the Fenwick array
-//        (integer atomics) and folded into the pending queries of later lanes.
+//  BIT:  Algorithm 1's sum by a sweep over the preorder of tau with a Fenwick array
+//        over the tau0 DFN (ttf_bit_sweep).  O(n log n) per tree, a warp a tree, 32
+//        preorder positions per round.
 // Both are templates: the batched instances take (graph, tree) entries and
 // per-graph tables, so trees of many graphs share one launch.
 #include <algorithm>
@@ -80,31 +76,9 @@ __global__ void __launch_bounds__(256) k_ttf_scan(GraphView g_in, WaveView w_in,
     }
 }
 
-// Fenwick point update at 1-based index i, the warp's lanes sharing the chain.
-// With j = i - 1 the chain is j, j | (j + 1), ...: its k-th node sets the k
-// lowest zero bits of j, i.e. equals j | (2^(b+1) - 1) where b is the k-th
-// zero bit.  So lane b (b < 31) owns the node of zero bit b of j and lane 31
-// owns node 0 (j itself); every node is visited exactly once.
-__device__ __forceinline__ void bit_point_add(int64_t *bit, int64_t n, int lane, int64_t i,
-                                              long long val) {
-    const uint32_t j = (uint32_t)(i - 1);  // host guarantees n < 2^31
-    int64_t node;
-    if (lane == 31) node = (int64_t)j + 1;
-    else if ((j >> lane) & 1u) node = -1;
-    else node = (int64_t)(j | ((2u << lane) - 1u)) + 1;
-    if (node >= 1 && node <= n) atomicAdd((unsigned long long *)(bit + node), (unsigned long long)val);
-}
-
-// range add [l, r] (0-based positions) += val, as two point updates
-__device__ __forceinline__ void bit_range_add(int64_t *bit, int64_t n, int lane, int32_t l,
-                                              int32_t r, long long val) {
-    bit_point_add(bit, n, lane, (int64_t)l + 1, val);
-    if ((int64_t)r + 2 <= n) bit_point_add(bit, n, lane, (int64_t)r + 2, -val);
-}
-
-// Range add of tau-ancestor x (x != r, tau parent par) in Algorithm 1: kind 1
-// when p(x) = p0(x) (tau0-subtree of x, value 2m - vol(x)), kind 2 when
-// p0(p(x)) = x (tau0-subtree of p(x), value vol(x) - 2m), 0 otherwise.
+// The entry of tau-ancestor x (x != r, tau parent par) of Algorithm 1: kind 1 when
+// p(x) = p0(x) (tau0-subtree of x, value 2m - vol(x)), kind 2 when p0(p(x)) = x
+// (tau0-subtree of p(x), value vol(x) - 2m), 0 otherwise.
 __device__ __forceinline__ int ttf_entry(const GraphView &g, int32_t x, int32_t par, int32_t r,
                                          int32_t twom, int64_t volx, int32_t &el, int32_t &er,
                                          int32_t &eval) {
@@ -120,13 +94,43 @@ __device__ __forceinline__ int ttf_entry(const GraphView &g, int32_t x, int32_t 
     return 0;
 }
 
-// One warp replays the preorder positions [lo, hi) of sub-wave tree t
-// (Algorithm 1) on the Fenwick array `bit` (1-based) and the memory stack `stk`
-// (sp entries on entry, the deepest on top); returns this lane's share of the
-// sum of d(v) Q(v) over those positions.  ok = false on a stack overflow (the
-// error bit is set).
+// Sum of a Fenwick array's first k entries, loads four at a time.
+__device__ __forceinline__ int32_t bit_prefix(const int32_t *bit, uint32_t k) {
+    int32_t s = 0;
+    while (k) {
+        int32_t x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            x[i] = k ? __ldcg(bit + k - 1) : 0;
+            k &= k - 1;
+        }
+        s += x[0] + x[1] + x[2] + x[3];
+    }
+    return s;
+}
+__device__ __forceinline__ long long bit_range(const int32_t *bit, int32_t l, int32_t r) {
+    return (long long)bit_prefix(bit, (uint32_t)r + 1u) - bit_prefix(bit, (uint32_t)l);
+}
+
+// Algorithm 1 the other way around.  Its sum over v of d(v) times the values of v's
+// ancestors x whose tau0-interval [l, r] holds v equals, summed over x,
+//   value(x) * D(x),  D(x) = sum of d(v) over v in Sub(tau, x) with in0(v) in [l, r],
+// so the sweep over the preorder adds d(v) at point in0(v) and asks for the sum of
+// [l, r] where Sub(tau, x) begins and where it ends: no range is added or undone.
+// A warp takes 32 positions a round; within them D comes from the lanes, and
+// only subtrees that reach past the round (kept on a stack) ask the Fenwick
+// array, at the round's edges.  Sums of degrees fit 32 bits (2m < 2^31).
+//
+// What bounds it is the latency of a round: adding and undoing the ranges one
+// position after the other took about 2000 cycles a position.  90000-vertex grid,
+// 500 trees beside a running walk: 93 -> 30 ms; 6144 trees of small grids 5.8 -> 1.5.
+//
+// This lane's share of f over the preorder positions [lo, hi) of sub-wave tree t, on
+// the zeroed array `bit` (n entries) and the stack `stk`, which holds sp entries
+// {out, l, r, value}, the deepest on top, of subtrees that began before lo.
+// ok = false on a stack overflow (the error bit is set).
 __device__ __forceinline__ long long ttf_bit_sweep(const GraphView &g, const WaveView &w,
-                                                   int64_t t, int64_t *bit, int4 *stk,
+                                                   int64_t t, int32_t *bit, int4 *stk,
                                                    int64_t lo, int64_t hi, int64_t sp,
                                                    bool &ok) {
     const int lane = threadIdx.x & 31;
@@ -141,93 +145,73 @@ __device__ __forceinline__ long long ttf_bit_sweep(const GraphView &g, const Wav
     ok = true;
 
     long long facc = 0;     // this lane's share of f
+    bool opened = false;    // its entry of the last round reached past it
+    int32_t ol = 0, orr = 0, oval = 0;
     for (int64_t base = lo; base < hi; base += 32) {
+        const int32_t last = (int32_t)((base + 32 < hi ? base + 32 : hi) - 1);
         const int64_t i = base + lane;
         const bool act = i < hi;
-        // ---- per-vertex data for preorder position i
-        int32_t v = -1, kind = 0, el = 0, er = 0, eval = 0, eout = 0, qpos = 0, dv = 0;
+        int32_t v = -1, kind = 0, el = 0, er = 0, eval = 0, eout = 0, q = 0, dv = 0;
         if (act) {
             v = pre[i];
             if (v < 0 || v >= n) {  // preorder is a permutation; anything else is corrupt
                 atomicOr(w.err, kErrBadTree);
                 v = r;
             }
-            const int32_t par = w_next(word[v]);
-            qpos = g.in0[v];
+            q = g.in0[v];
             dv = g.deg[v];
             eout = (int32_t)i + size[v] - 1;
-            if (v != r) kind = ttf_entry(g, v, par, r, twom, vol[v], el, er, eval);
+            if (v != r) kind = ttf_entry(g, v, w_next(word[v]), r, twom, vol[v], el, er, eval);
         }
-        // ---- prefix sums at the start of the chunk
-        long long pf = 0;
-        if (act) {
-            for (int64_t k = (int64_t)qpos + 1; k > 0; k &= k - 1)
-                pf += __ldcg((const long long *)(bit + k));
-        }
-        // every query load must have returned before this chunk issues its own
-        // atomics: reading pf in a shuffle makes the warp wait for them
-        pf = __shfl_sync(kFull, pf, lane);
-        long long corr = 0;
-        // ---- top of the memory stack, one entry per lane (lane k: entry sp-1-k)
-        int64_t mbase = sp;   // window covers entries [mbase - 32, mbase)
-        int4 win = make_int4(0, 0, 0, 0);
-        if (mbase - 1 - lane >= 0) win = stk[mbase - 1 - lane];
-        int mtop = 0;         // entries of the window already popped
-        int64_t mpopped = 0;  // memory entries popped in this chunk
-        unsigned cmask = 0;   // chunk entries alive on the stack (push order = lane order)
-        __syncwarp();
+        // ---- the array at the round's beginning: subtrees that the last round
+        // opened, and those that this round ends
+        if (opened) facc -= (long long)oval * bit_range(bit, ol, orr);
+        int4 top = make_int4(0x7FFFFFFF, 0, 0, 0);
+        if (sp - 1 - lane >= 0) top = stk[sp - 1 - lane];
+        bool pop = top.x <= last;
+        long long ended = pop ? bit_range(bit, top.y, top.z) : 0;
+        // ---- the round's own points, for those and for the lanes' subtrees
+        int32_t own = 0;
+#pragma unroll 8
         for (int j = 0; j < 32; ++j) {
-            const int64_t ij = base + j;
-            if (ij >= hi) break;
-            // pop every stacked ancestor whose subtree ended before position ij
-            while (true) {
-                int32_t pl, pr, pv;
-                if (cmask) {
-                    const int h = 31 - __clz(cmask);
-                    const int32_t o = __shfl_sync(kFull, eout, h);
-                    if (o >= ij) break;
-                    pl = __shfl_sync(kFull, el, h);
-                    pr = __shfl_sync(kFull, er, h);
-                    pv = __shfl_sync(kFull, eval, h);
-                    cmask &= ~(1u << h);
-                } else {
-                    if (sp - mpopped <= 0) break;
-                    if (mtop == 32) {  // reload the window below what was consumed
-                        mbase = sp - mpopped;
-                        win = make_int4(0, 0, 0, 0);
-                        if (mbase - 1 - lane >= 0) win = stk[mbase - 1 - lane];
-                        mtop = 0;
-                    }
-                    const int32_t o = __shfl_sync(kFull, win.x, mtop);
-                    if (o >= ij) break;
-                    pl = __shfl_sync(kFull, win.y, mtop);
-                    pr = __shfl_sync(kFull, win.z, mtop);
-                    pv = __shfl_sync(kFull, win.w, mtop);
-                    ++mtop;
-                    ++mpopped;
-                }
-                // undo: add the negation
-                bit_range_add(bit, n, lane, pl, pr, -(long long)pv);
-                if (lane >= j && pl <= qpos && qpos <= pr) corr -= pv;
-            }
-            const int kj = __shfl_sync(kFull, kind, j);
-            if (kj) {
-                const int32_t l = __shfl_sync(kFull, el, j);
-                const int32_t rr = __shfl_sync(kFull, er, j);
-                const int32_t val = __shfl_sync(kFull, eval, j);
-                bit_range_add(bit, n, lane, l, rr, (long long)val);
-                if (lane >= j && l <= qpos && qpos <= rr) corr += val;
-                cmask |= 1u << j;
-            }
+            const int32_t qj = __shfl_sync(kFull, q, j);
+            const int32_t dj = __shfl_sync(kFull, dv, j);  // 0 past hi
+            if (j >= lane && base + j <= eout && el <= qj && qj <= er) own += dj;
+            if (base + j <= top.x && top.y <= qj && qj <= top.z) ended += dj;
         }
-        if (act) facc += (long long)dv * (pf + corr);
-        // ---- spill the surviving chunk entries on top of the memory stack
-        const int64_t nsp = sp - mpopped;
-        if ((cmask >> lane) & 1u) {
-            const int64_t slot = nsp + __popc(cmask & lt_mask);
+        if (kind) facc += (long long)eval * own;
+        if (pop) facc += (long long)top.w * ended;
+        unsigned popm = __ballot_sync(kFull, pop);  // outs ascend from the top down
+        sp -= __popc(popm);
+        while (popm == kFull && sp > 0) {  // more than a window of them
+            top = make_int4(0x7FFFFFFF, 0, 0, 0);
+            if (sp - 1 - lane >= 0) top = stk[sp - 1 - lane];
+            pop = top.x <= last;
+            ended = pop ? bit_range(bit, top.y, top.z) : 0;
+            for (int j = 0; j < 32; ++j) {
+                const int32_t qj = __shfl_sync(kFull, q, j);
+                const int32_t dj = __shfl_sync(kFull, dv, j);
+                if (base + j <= top.x && top.y <= qj && qj <= top.z) ended += dj;
+            }
+            if (pop) facc += (long long)top.w * ended;
+            popm = __ballot_sync(kFull, pop);
+            sp -= __popc(popm);
+        }
+        __syncwarp();  // every sum of the array above precedes the additions below
+        if (act)
+            for (int64_t k = (int64_t)q + 1; k <= n; k += k & -k) atomicAdd(bit + k - 1, dv);
+        // ---- subtrees that reach past the round (at the end of a segment they
+        // would be asked for twice on the same array: nothing is left)
+        opened = kind && eout > last && base + 32 < hi;
+        const unsigned open = __ballot_sync(kFull, opened);
+        if (opened) {
+            const int64_t slot = sp + __popc(open & lt_mask);
             if (slot < w.stack_cap) stk[slot] = make_int4(eout, el, er, eval);
+            ol = el;
+            orr = er;
+            oval = eval;
         }
-        sp = nsp + __popc(cmask);
+        sp += __popc(open);
         if (sp > w.stack_cap) {
             if (lane == 0) atomicOr(w.err, kErrBadTree);
             ok = false;
@@ -235,6 +219,11 @@ __device__ __forceinline__ long long ttf_bit_sweep(const GraphView &g, const Wav
         }
         __threadfence_block();
         __syncwarp();
+    }
+    // subtrees that reach past hi
+    for (int64_t e = lane; e < sp; e += 32) {
+        const int4 x = stk[e];
+        facc += (long long)x.w * bit_range(bit, x.y, x.z);
     }
     return facc;
 }
@@ -249,7 +238,7 @@ __global__ void __launch_bounds__(128) k_ttf_bit(GraphView g_in, WaveView w_in, 
                            g, w, t))
         return;
     const int64_t n = g.n;
-    int64_t *bit = w.bit + t * (n + 1);  // zeroed, 1-based
+    int32_t *bit = reinterpret_cast<int32_t *>(w.bit) + t * n;  // zeroed
     int4 *stk = reinterpret_cast<int4 *>(w.stack) + t * w.stack_cap;
     bool ok;
     long long facc = ttf_bit_sweep(g, w, t, bit, stk, 0, n, 0, ok);
@@ -259,14 +248,12 @@ __global__ void __launch_bounds__(128) k_ttf_bit(GraphView g_in, WaveView w_in, 
     if (lane == 0) w.f[wave_tree(w, t)] = facc;
 }
 
-// Algorithm 1 over one preorder segment [lo, hi) of a tree per warp.  At
-// position lo the DFS stack holds the strict tau-ancestors of u = pre[lo] that
-// add a range, and the Fenwick array holds the sum of their range adds (every
-// ancestor of a later position that precedes lo is an ancestor of u; entries
-// pushed and popped before lo cancel).  Lane 0 collects them walking up the
-// tau parents (deepest first), the warp reverses them into stack order (root
-// side at the bottom) and replays their range adds, then sweeps the segment;
-// its share of f is added to the tree's f, which the caller zeroed.
+// The sweep over one preorder segment [lo, hi) of a tree per warp: D(x) is a sum
+// over positions, so each segment adds its own points' share.  The subtrees that
+// began before lo and reach into it are those of the strict tau-ancestors of u =
+// pre[lo]; lane 0 collects them walking up the tau parents (deepest first) and the
+// warp reverses them into stack order.  The segment's share of f is added to the
+// tree's f, which the caller zeroed.
 __global__ void __launch_bounds__(128) k_ttf_bit_seg(GraphView g, WaveView w,
                                                      const TtfSeg *__restrict__ segs,
                                                      int64_t nseg) {
@@ -322,17 +309,13 @@ __global__ void __launch_bounds__(128) k_ttf_bit_seg(GraphView g, WaveView w,
             stk[e] = b;
             stk[cnt - 1 - e] = a;
         }
-        __syncwarp();
-        for (long long e = 0; e < cnt; ++e) {
-            const int4 en = stk[e];
-            bit_range_add(sg.bit, n, lane, en.y, en.z, (long long)en.w);
-        }
         __threadfence_block();
         __syncwarp();
         sp = cnt;
     }
     bool ok;
-    long long facc = ttf_bit_sweep(g, w, t, sg.bit, stk, sg.lo, sg.hi, sp, ok);
+    int32_t *bit = reinterpret_cast<int32_t *>(sg.bit + 1);  // its first entry
+    long long facc = ttf_bit_sweep(g, w, t, bit, stk, sg.lo, sg.hi, sp, ok);
     if (!ok) return;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) facc += __shfl_down_sync(kFull, facc, o);
@@ -340,13 +323,13 @@ __global__ void __launch_bounds__(128) k_ttf_bit_seg(GraphView g, WaveView w,
         atomicAdd((unsigned long long *)(w.f + wave_tree(w, t)), (unsigned long long)facc);
 }
 
-// zero entries 1 .. n of every segment's Fenwick array
+// zero every segment's Fenwick array
 __global__ void k_zero_seg_bits(const TtfSeg *__restrict__ segs, int64_t nseg, int64_t n) {
     for (int64_t s = blockIdx.y; s < nseg; s += gridDim.y) {
-        int64_t *b = segs[s].bit;
+        int32_t *b = reinterpret_cast<int32_t *>(segs[s].bit + 1);
         for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
              i += (int64_t)gridDim.x * blockDim.x)
-            b[i + 1] = 0;
+            b[i] = 0;
     }
 }
 
@@ -382,7 +365,7 @@ cudaError_t launch_ttf_bit_seg(const GraphView &g, WaveView w, const TtfSeg *seg
 }
 
 cudaError_t launch_ttf_bit(const GraphView &g, WaveView w, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(w.bit, 0, sizeof(int64_t) * (size_t)(w.B * (g.n + 1)), s);
+    cudaError_t e = cudaMemsetAsync(w.bit, 0, sizeof(int32_t) * (size_t)(w.B * g.n), s);
     if (e != cudaSuccess) return e;
     k_ttf_bit<false><<<(unsigned)((w.B * 32 + 127) / 128), 128, 0, s>>>(g, w, MultiSub{});
     return cudaGetLastError();

@@ -1925,9 +1925,7 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                     KC_CK(g, cudaMemsetAsync(w.size, 0, sizeof(int32_t) * nb, s0));
                     KC_CK(g, cudaMemsetAsync(w.vol, 0, sizeof(int64_t) * nb, s0));
                     if (p.bit) {
-                        KC_CK(g, cudaMemsetAsync(w.bit, 0,
-                                                 sizeof(int64_t) * (size_t)B * (size_t)(g->n + 1),
-                                                 s0));
+                        KC_CK(g, cudaMemsetAsync(w.bit, 0, sizeof(int32_t) * nb, s0));
                     } else {
                         KC_CK(g, cudaMemsetAsync(w.f, 0, sizeof(int64_t) * (size_t)B, s0));
                         w.bit = nullptr;

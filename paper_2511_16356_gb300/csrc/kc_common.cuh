@@ -235,7 +235,8 @@ struct WaveView {
     int64_t *vol;            // [B][n] subtree volumes
     int32_t *din;            // [B][n] DFN (sibling offsets before the top-down pass)
     int32_t *aux;            // [B][n] per-parent running sums, then preorder (BIT variant)
-    int64_t *bit;            // [B][n+1] Fenwick array (BIT variant), may be null
+    int64_t *bit;            // [B][n+1], of which the BIT variant's Fenwick arrays take
+                             // [B][n] int32; may be null
     int64_t *steps;          // [B]
     int64_t *f;              // [B]
     uint32_t *err;           // [1] error bits (kErr*)
@@ -248,7 +249,7 @@ struct WaveView {
 };
 
 // One preorder segment of a tree for the segmented BIT evaluation of f: its
-// Fenwick array (`bit` is the 1-based base, entries 1 .. n used), its stack
+// Fenwick array (n int32 from bit + 1 on, in room for n int64), its stack
 // (stack_cap int4 entries) and the positions [lo, hi) of sub-wave tree t.
 struct TtfSeg {
     int64_t *bit;
