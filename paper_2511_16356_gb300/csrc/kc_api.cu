@@ -382,16 +382,16 @@ bool use_solo(const kc_graph *g) {
            g->ttf_variant == KC_TTF_BIT;
 }
 
-// Whether AUTO draws the trees of a low-diameter graph by cycle popping
-// (k4_pop.cu): in shared memory, where f is evaluated too, or in memory.
-enum : int { kPopNone = 0, kPopSmall = 1, kPopLarge = 2 };
+// Whether and how AUTO draws the trees of a low-diameter graph by cycle popping
+// (k4_pop.cu, kc_host_plan.h).
+using kc_host::kPopLarge;
+using kc_host::kPopNone;
+using kc_host::kPopSmall;
 int use_pop(const kc_graph *g) {
     if (g->walker != KC_WALK_WARP || !g->auto_walker || g->ttf_variant != KC_TTF_SCAN)
         return kPopNone;
-    const int64_t twom = 2 * g->m;
-    const int64_t root_deg = g->h_row_off[(size_t)g->root + 1] - g->h_row_off[(size_t)g->root];
-    if (twom < ((int64_t)1 << 32) && kc_host::pop_small(g->n, twom, root_deg)) return kPopSmall;
-    return kc_host::pop_large(g->n, twom, root_deg) ? kPopLarge : kPopNone;
+    return kc_host::pop_kind(
+        g->n, 2 * g->m, g->h_row_off[(size_t)g->root + 1] - g->h_row_off[(size_t)g->root]);
 }
 
 // The trees of wave w (sample ids c.sids): steps, and f unless they are only to be
@@ -416,9 +416,25 @@ PopTask pop_task(const kc_graph *g, const GraphView &gv, const WaveView &w, cons
     return k;
 }
 
-// Where the parents of the next B trees of the pool go when trees are kept.
+// Where the parents of the pool's next trees go when trees are kept; pop_par: or else.
 int32_t *pool_slot(const kc_graph *g) {
     return g->cfg.keep_trees ? g->d_parents + g->pool * g->n : nullptr;
+}
+
+int32_t *pop_par(const kc_graph *g, const WaveView &w) {
+    return pool_slot(g) ? pool_slot(g) : w.ord;
+}
+
+// The trees of a task (their parents), in memory or in shared memory; w.B trees, w's
+// sub-wave arrays are scratch.  Returns the kernels launched.
+int pop_trees(kc_graph *g, const PopTask &task, const WaveView &w, bool in_memory) {
+    if (!in_memory) {
+        KC_CK(g, launch_pop_trees(task, w.B, g->stream));
+        return 1;
+    }
+    KC_CK(g, launch_pop_large(task, w.B, w.word, w.size, w.din, (int32_t *)w.vol, w.f, g->num_sms,
+                              g->stream));
+    return 4;
 }
 
 // Words of k1_solo.cu with the arrow queues of `root`'s trees (-1: no vertex in
@@ -680,8 +696,8 @@ bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
                                       B, g->stream));
             ph.done(1);
         }
-        // in memory: all three steps a sub-wave at a time
-        for (int64_t sub = 0; pop == kPopLarge && sub < B && !err; sub += p.BT) {
+        // otherwise trees, traversal and f apart, a sub-wave at a time
+        for (int64_t sub = 0; pop != kPopSmall && sub < B && !err; sub += p.BT) {
             WaveView sv = w;
             sv.B = std::min<int64_t>(p.BT, B - sub);
             sv.word = w.word + sub * g->n;
@@ -691,11 +707,8 @@ bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
             int32_t *par = pool_slot(g) ? pool_slot(g) + sub * g->n : sv.ord;
             {
                 Phase ph(g, g->t_wilson);
-                KC_CK(g, launch_pop_large(pop_task(g, gv, sv, c.sids + sub, g->root, -1, false,
-                                                   par),
-                                          sv.B, sv.word, sv.size, sv.din, (int32_t *)sv.vol, sv.f,
-                                          g->num_sms, g->stream));
-                ph.done(4);
+                ph.done(pop_trees(g, pop_task(g, gv, sv, c.sids + sub, g->root, -1, false, par),
+                                  sv, pop == kPopLarge));
             }
             KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
             if (err) break;
@@ -1238,13 +1251,7 @@ void resample_slots(kc_graph *g, const std::vector<int64_t> &slots, bool cond, i
             const PopTask task = pop_task(g, gv, w, c.sids, cond ? v : g->root, cond ? u : -1,
                                           false, w.ord);
             KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
-            const bool block = g->n <= kc_host::kPopTreesMax;
-            if (block)
-                KC_CK(g, launch_pop_trees(task, b, g->stream));
-            else
-                KC_CK(g, launch_pop_large(task, b, w.word, w.size, w.din, (int32_t *)w.vol, w.f,
-                                          g->num_sms, g->stream));
-            g->t_update.launches += block ? 1 : 4;
+            g->t_update.launches += pop_trees(g, task, w, g->n > kc_host::kPopTreesMax);
             uint32_t err = 0;
             KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
             if (solo_retry(g, err)) pop = kPopNone;
@@ -1788,14 +1795,16 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
             }
             if (idx.empty()) break;
             const size_t G = idx.size();
-            // graphs whose trees a block each pops (k4_pop.cu, a launch for each block
-            // size), graphs that run one walker per tree (k1_solo.cu) and graphs that
-            // run 32, a launch each: longest trees first, so that none starts last, the
-            // last kind's interleaved, so that a launch mixes sizes
+            // graphs whose trees and f a block each pops (k4_pop.cu, a launch for each
+            // block size), graphs that run one walker per tree (k1_solo.cu) and graphs
+            // that run 32, a launch each: longest trees first, so that none starts last,
+            // the last kind's interleaved, so that a launch mixes sizes.  Larger popped
+            // trees have launches of their own.
             std::vector<char> solo(G), pop(G);
             for (size_t k = 0; k < G; ++k) {
                 solo[k] = use_solo(gs[idx[k]]) ? 1 : 0;
-                pop[k] = use_pop(gs[idx[k]]) == kPopSmall ? 1 : 0;
+                pop[k] = (char)use_pop(gs[idx[k]]);
+                if (pop[k] != kPopSmall && bs[k] > plans[(size_t)idx[k]].BT) pop[k] = kPopNone;
             }
             std::vector<size_t> by_work(G);
             for (size_t k = 0; k < G; ++k) by_work[k] = k;
@@ -1819,7 +1828,7 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                 entry.clear();
                 for (size_t k : by_work) {  // largest first: classes are contiguous
                     kc_graph *g = gs[idx[k]];
-                    if (!pop[k]) continue;
+                    if (pop[k] != kPopSmall) continue;
                     tasks[k] = pop_task(g, gv[k], wv[k], sids[k], g->root, -1, true,
                                         pool_slot(g));
                     if (classes.empty() || kc_host::pop_small_threads(classes.back().max_n) !=
@@ -1841,8 +1850,12 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                 for (size_t k = 0; k < G; ++k) {
                     kc_graph *g = gs[idx[k]];
                     KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), s0));
-                    if (pop[k]) continue;
-                    if (solo[k]) init_queues(g, gv[k], wv[k], sids[k], g->root, s0);
+                    if (pop[k] == kPopSmall) continue;
+                    if (pop[k])
+                        pop_trees(g, pop_task(g, gv[k], wv[k], sids[k], g->root, -1, false,
+                                              pop_par(g, wv[k])),
+                                  wv[k], pop[k] == kPopLarge);
+                    else if (solo[k]) init_queues(g, gv[k], wv[k], sids[k], g->root, s0);
                     else KC_CK(g, launch_wave_init(gv[k], wv[k], s0));
                 }
                 const size_t bytes = (sizeof(GraphView) + sizeof(WaveView) + sizeof(PopTask)) * G +
@@ -1916,7 +1929,17 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                 if (hdr[0]) throw Fail{KC_ERR_CUDA};
                 if (p.bit) ensure_stack(g, p, hdr[1]);
                 cv[k] = carve(g, p);
-                if (pop[k]) continue;  // f is there
+                if (pop[k] == kPopSmall) continue;  // f is there
+                if (pop[k]) {
+                    const ParTrees trees{pop_par(g, wv[k]), nullptr};
+                    int nl = 0;
+                    KC_CK(g, launch_traverse_parents(gv[k], wv[k], trees, false, -1, -1, false, s0,
+                                                     &nl));
+                    KC_CK(g, launch_ttf_scan_parents(gv[k], wv[k], trees, s0));
+                    g->t_traverse.launches += nl;
+                    g->t_ttf.launches += 1;
+                    continue;
+                }
                 WaveView w = cv[k].wv;
                 w.B = B;
                 const GraphView v = view_of(g);

@@ -132,18 +132,20 @@ constexpr int64_t kPopContractMax = 38000, kPopTreesMax = 56000;
 constexpr size_t pop_trees_bytes(int64_t n) {
     return (size_t)n * (n <= kPopContractMax ? 6 : 4);
 }
-// Whether popping pays: its rounds follow the longest loops, which are long where
-// the first walk is -- the walk to the root takes about 2m / deg(root) departures.
-// Power-law graphs (a hub as the root): 10000 vertices, 500 trees 5.26 -> 1.27 ms
-// against 32 walkers and their traversal.  Sparse random graphs: 2000 vertices,
-// 2000 trees 3.9 -> 3.5 ms, even at 15000 vertices (24.0 / 23.8 ms) and behind when
-// blocks of many sizes share a call.
-inline bool pop_small(int64_t n, int64_t twom, int64_t root_deg) {
-    return n <= kPopSmallMax && (n <= 4096 || 16 * (twom / std::max<int64_t>(root_deg, 1)) <= n);
-}
-// In memory only where the root is such a hub.
-inline bool pop_large(int64_t n, int64_t twom, int64_t root_deg) {
-    return n > kPopSmallMax && 16 * (twom / std::max<int64_t>(root_deg, 1)) <= n;
+// How AUTO draws the trees of a low-diameter graph (against 32 walkers a tree and
+// their traversal; GB300, ms):
+//   up to kPopSmallMax vertices in shared memory, f included (random graph of 8000
+//   vertices, 1000 trees 13.6 -> 6.3; of 15000 24.0 -> 12.4; power-law graph of 10000,
+//   500 trees 5.3 -> 0.9);
+//   past it in memory where the root is a hub, so that the walk to it, of about
+//   2m / deg(root) departures, is short and the rounds touch few vertices (2 million
+//   vertices, 384 trees 830 -> 140);
+//   otherwise trees in shared memory while a block holds them.
+enum : int { kPopNone = 0, kPopSmall = 1, kPopLarge = 2, kPopTrees = 3 };
+inline int pop_kind(int64_t n, int64_t twom, int64_t root_deg) {
+    if (n <= kPopSmallMax && twom < ((int64_t)1 << 32)) return kPopSmall;
+    if (16 * (twom / std::max<int64_t>(root_deg, 1)) <= n) return kPopLarge;
+    return n <= kPopContractMax ? kPopTrees : kPopNone;
 }
 inline int pop_small_threads(int64_t n) { return n <= 1024 ? 128 : (n <= 4096 ? 256 : 1024); }
 

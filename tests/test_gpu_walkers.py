@@ -120,6 +120,15 @@ def test_popped_trees_at_the_step_cap():
         assert kc.STATUS[st] == "KC_ERR_STEP_LIMIT"
 
 
+@pytest.mark.parametrize("n", [16500, 38000, 38400])
+def test_popped_trees_of_random_graphs_match_oracle(n):
+    """No hub: trees in shared memory up to 38000 vertices, walkers past them."""
+    g = S.er_lcc(n, 8.0 / n, 9)
+    with kc.KemenyGraph.from_graph(g, _cfg(keep_trees=1)) as G:
+        G.sample(47, 20)
+        _check(g, G.samples(), 47, 0, 20)
+
+
 @pytest.mark.parametrize("trees", [1, 40, 200])
 def test_popped_trees_in_memory_match_oracle(trees):
     """Power-law graph with a hub as root, too large for shared memory; fewer trees

@@ -18,7 +18,11 @@ extern "C" int hq_group(int64_t B, int64_t sms) { return kc_host::queue_group(B,
 extern "C" int hq_max_bits() { return kc_host::kMaxQueueBits; }
 extern "C" uint64_t hq_pop_bytes(int64_t n) { return kc_host::pop_small_bytes(n); }
 extern "C" int hq_pop_threads(int64_t n) { return kc_host::pop_small_threads(n); }
-extern "C" int hq_pop(int64_t n, int64_t twom, int64_t d) { return kc_host::pop_small(n, twom, d); }
+extern "C" int hq_pop(int64_t n, int64_t twom, int64_t d) { return kc_host::pop_kind(n, twom, d); }
+extern "C" uint64_t hq_trees_bytes(int64_t n) { return kc_host::pop_trees_bytes(n); }
+extern "C" int64_t hq_trees_max(int contract) {
+    return contract ? kc_host::kPopContractMax : kc_host::kPopTreesMax;
+}
 extern "C" int64_t hq_pop_max() { return kc_host::kPopSmallMax; }
 extern "C" int hq_width() { return kc_host::kQueueWidth; }
 """
@@ -38,7 +42,9 @@ def queue(tmp_path_factory):
     lib.hq_group.argtypes = [ctypes.c_int64, ctypes.c_int64]
     lib.hq_pop_bytes.restype = ctypes.c_uint64
     lib.hq_pop_max.restype = ctypes.c_int64
-    for f in (lib.hq_pop_bytes, lib.hq_pop_threads):
+    lib.hq_trees_bytes.restype = ctypes.c_uint64
+    lib.hq_trees_max.restype = ctypes.c_int64
+    for f in (lib.hq_pop_bytes, lib.hq_pop_threads, lib.hq_trees_bytes):
         f.argtypes = [ctypes.c_int64]
     lib.hq_pop.argtypes = [ctypes.c_int64] * 3
     return lib
@@ -68,6 +74,16 @@ def test_popped_trees_fit_a_block(queue):
     for n in (2, 3, 1024, 1025, 4096, 4097, top):
         assert 14 * n <= queue.hq_pop_bytes(n) <= 14 * n + 2
         assert queue.hq_pop_threads(n) in (128, 256, 1024)
-        assert queue.hq_pop(n, 10 * n, n - 1)
-    assert not queue.hq_pop(top + 1, 10 * top, top)
-    assert not queue.hq_pop(8000, 64000, 20) and queue.hq_pop(4000, 32000, 20)
+        assert queue.hq_pop(n, 10 * n, 1) == 1
+    for contract, each in ((1, 6), (0, 4)):
+        n = queue.hq_trees_max(contract)
+        assert queue.hq_trees_bytes(n) == each * n <= 227 * 1024 - 64
+
+
+def test_popping_follows_size_and_root(queue):
+    small, trees = queue.hq_pop_max(), queue.hq_trees_max(1)
+    assert queue.hq_pop(small + 1, 10 * small, small) == 2  # a hub: in memory
+    assert queue.hq_pop(small + 1, 10 * small, 20) == 3     # else in a block
+    assert queue.hq_pop(trees + 1, 10 * trees, 20) == 0     # until it does not fit
+    assert queue.hq_pop(4000000, 68000000, 8000) == 2
+    assert queue.hq_pop(9000, 1 << 32, 8999) == 3           # 32-bit volumes do not hold 2m
