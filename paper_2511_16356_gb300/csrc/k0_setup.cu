@@ -7,7 +7,7 @@ namespace kc {
 
 namespace {
 
-__global__ void k_build_records(GraphView g, VRec *rec, int32_t *deg) {
+__global__ void k_build_records(GraphView g, VRec *rec, int4 *rec4, int32_t *deg) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= g.n) return;
     const int64_t off = g.row_off[v];
@@ -19,6 +19,7 @@ __global__ void k_build_records(GraphView g, VRec *rec, int32_t *deg) {
 #pragma unroll
     for (int k = 0; k < kInline; ++k) r.nbr[k] = k < d ? g.col[off + k] : -1;
     rec[v] = r;
+    if (rec4) rec4[v] = make_int4(r.nbr[0], r.nbr[1], r.nbr[2], r.nbr[3]);
     deg[v] = d;
 }
 
@@ -262,8 +263,9 @@ cudaError_t launch_central_pick(int64_t n, const int32_t *deg, int32_t dmax, con
     return cudaGetLastError();
 }
 
-cudaError_t launch_build_records(const GraphView &g, VRec *rec, int32_t *deg, cudaStream_t s) {
-    k_build_records<<<blocks_for(g.n, 256), 256, 0, s>>>(g, rec, deg);
+cudaError_t launch_build_records(const GraphView &g, VRec *rec, int4 *rec4, int32_t *deg,
+                                 cudaStream_t s) {
+    k_build_records<<<blocks_for(g.n, 256), 256, 0, s>>>(g, rec, rec4, deg);
     return cudaGetLastError();
 }
 

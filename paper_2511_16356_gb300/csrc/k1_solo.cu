@@ -5,22 +5,19 @@
 //
 // What bounds a sequential walker is the chain of one departure: load the word
 // of the vertex, ten dependent Philox rounds, select the neighbour, load its
-// word.  Here the word of a vertex outside the tree holds the target of its next
-// departure and a queue of the arrows after it as neighbour indices, so the walk
-// is a pointer chase: the next word is requested at once, and behind the walker
-// the vertex left gets its new target (a bit field and a select) while that load
-// is in flight.  An empty queue is refilled by the warp, one arrow per lane.  The
-// first queue of every vertex comes from a parallel initialisation
-// (k_queue_init), which replaces the clearing of the words.
+// word.  Here the word of a vertex outside the tree holds a queue of its next
+// arrows as neighbour indices, so a departure is a load, a select and a shift; an
+// empty queue is refilled by the warp, one arrow per lane.  The first queue of
+// every vertex comes from a parallel initialisation (k_queue_init), which replaces
+// the clearing of the words.
 //
 // Word of a vertex outside the tree, b = bits of a neighbour index (kc_host_plan.h):
-//   low half   target of the next departure
-//   high half  bits [0, 17): the last arrow taken, the next arrow, those after it
-//              (b bits each), then a single 1 that marks the end of the queue;
-//              bits [17, 31): departures so far; bit 31 clear
+//   low half   the last arrow taken, the next arrow, those after it (b bits each),
+//              then a single 1 that marks the end of the queue
+//   high half  departures so far (bit 31 clear)
 // In-tree words are the common ones (parent, depth, bit 63).  A departure count
-// that its field may not hold sets kErrCountField and the host repeats the wave
-// with the walkers of k1_wilson.cu.
+// near its limit sets kErrCountField and the host repeats the wave with the
+// walkers of k1_wilson.cu.
 #include <algorithm>
 
 #include "kc_common.cuh"
@@ -31,12 +28,29 @@ namespace kc {
 namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
-constexpr uint32_t kQueue = (1u << kc_host::kQueueWidth) - 1u;
-constexpr uint32_t kOneMore = 1u << kc_host::kQueueWidth;  // one departure in the high half
-constexpr uint32_t kMostDepartures = (1u << (31 - kc_host::kQueueWidth)) - 1u;
+
+// Neighbours of a vertex.  kDeg4 (every degree at most 4): the 16-byte record, so
+// that a departure loads one piece of it.
+template <bool kDeg4>
+struct Nbrs {
+    VRec r;
+    __device__ __forceinline__ void load(const GraphView &g, int32_t v) { r = load_rec(g.rec + v); }
+    __device__ __forceinline__ int32_t pick(uint32_t k, const GraphView &g) const {
+        return nbr_of<false>(r, k, g.col);
+    }
+};
+template <>
+struct Nbrs<true> {
+    int4 r;
+    __device__ __forceinline__ void load(const GraphView &g, int32_t v) { r = __ldg(g.rec4 + v); }
+    __device__ __forceinline__ int32_t pick(uint32_t k, const GraphView &) const {
+        const int32_t lo = (k & 1u) ? r.y : r.x, hi = (k & 1u) ? r.w : r.z;
+        return (k & 2u) ? hi : lo;
+    }
+};
 
 // Words of every tree of the wave: the first `slots` arrows of each vertex, the
-// root (if any) in the tree.  A thread keeps one vertex's record for kInitTrees
+// root (if any) in the tree.  A thread keeps one vertex's degree for kInitTrees
 // trees.
 constexpr int kInitTrees = 8;
 __global__ void __launch_bounds__(256) k_queue_init(GraphView g, WaveView w, PhiloxKeys keys,
@@ -46,7 +60,7 @@ __global__ void __launch_bounds__(256) k_queue_init(GraphView g, WaveView w, Phi
     const int64_t n = g.n;
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n) return;
-    const VRec r = load_rec(g.rec + v);
+    const uint32_t deg = (uint32_t)g.deg[v];
     for (int64_t t0 = (int64_t)blockIdx.y * kInitTrees; t0 < w.B;
          t0 += (int64_t)gridDim.y * kInitTrees) {
         const int64_t t1 = t0 + kInitTrees < w.B ? t0 + kInitTrees : w.B;
@@ -57,14 +71,12 @@ __global__ void __launch_bounds__(256) k_queue_init(GraphView g, WaveView w, Phi
                 w.ord[t * n] = root;
             } else {
                 const uint32_t sample = (uint32_t)sids[t];
-                uint32_t q = 1u << (b * (slots + 1)), first = 0;
-                for (int j = 0; j < slots; ++j) {
-                    const uint32_t d = bounded_draw_k(keys, seed, (uint32_t)v, (uint32_t)j,
-                                                      sample, kTagWalk, (uint32_t)r.deg);
-                    q |= d << (b * (j + 1));
-                    first = j == 0 ? d : first;
-                }
-                x = (uint64_t)(uint32_t)nbr_of<false>(r, first, g.col) | ((uint64_t)q << 32);
+                uint32_t q = 1u << (b * (slots + 1));
+                for (int j = 0; j < slots; ++j)
+                    q |= bounded_draw_k(keys, seed, (uint32_t)v, (uint32_t)j, sample, kTagWalk,
+                                        deg)
+                         << (b * (j + 1));
+                x = q;
             }
             w.word[t * n + v] = x;
         }
@@ -95,17 +107,16 @@ __device__ __forceinline__ void finish_tree(const WaveView &w, int64_t t, int en
 // it is longer than the vertices left (corrupt state).
 template <int kGroup, bool kDeg4>
 __device__ __forceinline__ int32_t commit_path(unsigned gm, uint64_t *word, int32_t *ord,
-                                               const VRec *__restrict__ rec,
-                                               const int32_t *__restrict__ col, int32_t n,
-                                               uint32_t kmask, int32_t s, int32_t h, int32_t dh,
-                                               int32_t pos) {
+                                               const GraphView &g, int32_t n, uint32_t kmask,
+                                               int32_t s, int32_t h, int32_t dh, int32_t pos) {
     constexpr int32_t kIn = kGroup - 1;
     const int lane = threadIdx.x & kIn;
     int32_t len = 0, mine = 0, par = 0, x = s;
+    Nbrs<kDeg4> r;
     while (x != h) {
-        const uint32_t hi = (uint32_t)(word[x] >> 32);
-        const VRec r = load_rec(rec + x);
-        const int32_t px = nbr_of<kDeg4>(r, hi & kmask, col);
+        const uint32_t lo = (uint32_t)word[x];
+        r.load(g, x);
+        const int32_t px = r.pick(lo & kmask, g);
         if (lane == (len & kIn)) {
             mine = x;
             par = px;
@@ -129,8 +140,8 @@ __device__ __forceinline__ int32_t commit_path(unsigned gm, uint64_t *word, int3
     for (j -= kGroup; j >= lane; j -= kGroup) {
         __syncwarp(gm);
         const int32_t y = ord[n - 1 - j];
-        const int32_t py =
-            nbr_of<kDeg4>(load_rec(rec + y), (uint32_t)(word[y] >> 32) & kmask, col);
+        r.load(g, y);
+        const int32_t py = r.pick((uint32_t)word[y] & kmask, g);
         __syncwarp(gm);
         word[y] = w_make(py, (uint32_t)(dh + len - j), true);
         ord[pos + len - 1 - j] = y;
@@ -139,119 +150,95 @@ __device__ __forceinline__ int32_t commit_path(unsigned gm, uint64_t *word, int3
     return len;
 }
 
-// One tree per group of kGroup lanes, 32 / kGroup trees per warp.
-//
-// Measured (GB300, perturbed grids, ncu): about 52 warp instructions and 250
-// cycles a departure with one tree per warp on an otherwise idle SM, of which 60
-// wait for L1; 32 concurrent walkers of one tree (k_wilson_warp) take about 650.
-// 1000 trees of the 350x350 grid: 1330 -> 661 ms; 4522 trees of it under a cap of
-// 13 n departures: 1640 (k_wilson, one tree per lane) -> 508 ms.  With 28 trees
-// an SM the schedulers issue in 0.7 of their slots, so the rest is instructions.
-//  The lanes of a
+// One tree per group of kGroup lanes, 32 / kGroup trees per warp.  The lanes of a
 // group follow their walk together (one address, one transaction) and share the
 // work around it: starts are looked up and paths committed kGroup vertices at a
 // time, and a refill draws an arrow per lane.  All walks of a warp depart in
 // lockstep until one of them meets the tree; when one queue is empty, every
 // walk's vertex is refilled, which costs the warp the same.
-// kMulti (with kGroup 32): block j takes tree mw.entry[j].y of graph
-// mw.entry[j].x.
-struct QueueShape {
-    int b, slots;
-};
-template <int kGroup, bool kDeg4, bool kMulti, bool kReject>
-__global__ void __launch_bounds__(32, kGroup == 32 ? 28 : (kGroup == 16 ? 20 : 24)) k_wilson_queue(
-    GraphView g_in, WaveView w_in, PhiloxKeys keys_in, uint64_t seed_in,
-    const int64_t *__restrict__ sids_in, QueueShape shape_in, int64_t step_cap_in,
-    volatile int32_t *done_flag, MultiWalk mw) {
-    constexpr int kTrees = 32 / kGroup;
+//
+// Measured (GB300, perturbed grids, ncu): 32 warp instructions and 187 cycles a
+// departure with one tree per warp on an otherwise idle SM, of which 40 wait for
+// memory (L1 serves 95%); the 32 lockstep walkers of one tree (k_wilson_warp) take
+// about 650 cycles, a walker per lane (k_wilson) about 1100.  Walk of 500 trees of a
+// 40000-vertex grid: 348 (k_wilson_warp) -> 140 ms; of 4522 trees of the 350x350 grid
+// under a cap of 13 n departures: 1640 (k_wilson) -> 345 ms.  The word that held the
+// next target itself, with the queue behind it, made the load chain shorter and the
+// kernel slower: 52 instructions, 250 cycles.
+template <int kGroup, bool kDeg4, bool kReject>
+__device__ __forceinline__ void walk_trees(const GraphView &g, const WaveView &w,
+                                           const PhiloxKeys &keys, uint64_t seed, uint32_t sample,
+                                           int64_t t, bool on, int bits, int slots,
+                                           int64_t step_cap, volatile int32_t *done_flag) {
+    constexpr bool kOne = kGroup == 32;
     constexpr unsigned kIn = kGroup - 1;
     const unsigned lane = threadIdx.x & kIn;
     const unsigned gshift = threadIdx.x & ~kIn;
-    const unsigned gm = kGroup == 32 ? kFull : ((1u << (kGroup & 31)) - 1u) << gshift;
-    const int e = kMulti ? mw.entry[blockIdx.x].x : 0;
-    const int64_t t = kMulti ? (int64_t)mw.entry[blockIdx.x].y
-                             : (int64_t)blockIdx.x * kTrees + gshift / kGroup;
-    const uint64_t seed = kMulti ? mw.seeds[e] : seed_in;
-    const PhiloxKeys keys = kMulti ? philox_keys(seed) : keys_in;
-    const int64_t step_cap = kMulti ? mw.step_caps[e] : step_cap_in;
-    const int64_t n64 = kMulti ? mw.graphs[e].n : g_in.n;
-    const VRec *__restrict__ rec = kMulti ? mw.graphs[e].rec : g_in.rec;
-    const int32_t *__restrict__ col = kMulti ? mw.graphs[e].col : g_in.col;
-    const WaveView w = kMulti ? mw.waves[e] : w_in;
-    const int b = kMulti ? mw.queue_bits[e] : shape_in.b;
-    const int slots = kMulti ? kc_host::queue_slots(b) : shape_in.slots;
-    const int32_t n = (int32_t)n64;
+    const unsigned gm = kOne ? kFull : ((1u << (kGroup & 31)) - 1u) << gshift;
+    const int32_t n = (int32_t)g.n;
+    const int b = kDeg4 ? 2 : bits;
     const uint32_t kmask = (1u << b) - 1u;
-    // what follows is the same in every lane of a group
-    bool on = kTrees == 1 || t < w.B;  // the tree is still being walked
+    const uint32_t last = 2u << (2 * b);  // a queue below this holds one more arrow
+    // what follows is the same in every lane of a group; on: its tree is being walked
     const int64_t tt = on ? t : 0;
-    uint64_t *word = w.word + tt * n64;
-    int32_t *ord = w.ord + tt * n64;
-    const uint32_t sample = (uint32_t)(kMulti ? mw.sids[e][tt] : sids_in[tt]);
-    int64_t steps = 0;           // departures before the last refill or path
-    uint32_t more = 0;           // and since
+    uint64_t *word = w.word + tt * g.n;
+    int32_t *ord = w.ord + tt * g.n;
+    int64_t steps = 0;  // departures before the last refill or path
+    uint32_t more = 0;  // and since
     int32_t pos = w.pos0, maxd = 0;
     int32_t s = 0, base = -kGroup;  // start of the walk; chunk of starts looked up
     unsigned todo = 0;              // its vertices that were outside the tree
-    int32_t u = 0, lo = 0;          // the walk's vertex, its word and record
-    uint32_t hi = 0;
-    VRec ra, rb;
-    ra.deg = rb.deg = 1;
+    int32_t u = 0;                  // the walk's vertex, its word and neighbours
+    uint32_t lo = 0, hi = 0;
+    Nbrs<kDeg4> ra{}, rb{};
     int end = kEndOk;
     bool start = on, hit = false;
 
-    // One departure of every walk, from the vertex of record rc to that of rn;
+    // One departure of every walk, from the vertex of neighbours rc to that of rn;
     // whether some walk has to leave the lockstep.
-    auto depart = [&](const VRec &rc, VRec &rn) -> bool {
+    auto depart = [&](const Nbrs<kDeg4> &rc, Nbrs<kDeg4> &rn) -> bool {
         int32_t v = 0;
         uint64_t x = 0;
-        uint32_t left = 0, next = 0, count = 0;
-        if (kTrees == 1 || on) {
-            v = lo;
+        if (kOne || on) {
+            v = rc.pick((lo >> b) & kmask, g);
             x = word[v];
-            rn = load_rec(rec + v);
-            const uint32_t queue = hi & kQueue;
-            left = queue >> b;  // the arrow taken, then the rest
-            next = left >> b;
-            count = (hi ^ queue) + kOneMore;
+            rn.load(g, v);
         }
-        uint32_t k = next & kmask;
-        const bool empty = (kTrees == 1 || on) && next == 1u;  // only the end mark
-        if (kTrees == 1 ? empty : __any_sync(kFull, empty)) {
+        const bool empty = (kOne || on) && lo < last;
+        lo >>= b;
+        ++hi;
+        if (kOne ? empty : __any_sync(kFull, empty)) {
             // lane j draws the arrow after the next j
-            const uint32_t c = count >> kc_host::kQueueWidth;
             uint32_t d = 0;
             if (lane < (unsigned)slots)
-                d = bounded_draw_k(keys, seed, (uint32_t)u, c + lane, sample, kTagWalk,
-                                   (uint32_t)rc.deg)
+                d = bounded_draw_k(keys, seed, (uint32_t)u, hi + lane, sample, kTagWalk,
+                                   (uint32_t)g.deg[u])
                     << (b * (lane + 1));
-            if (kGroup == 32) {
+            if (kOne) {
                 d = __reduce_or_sync(kFull, d);
             } else {
 #pragma unroll
                 for (int o = kGroup / 2; o > 0; o >>= 1) d |= __shfl_xor_sync(kFull, d, o);
             }
-            left = (left & kmask) | d | (1u << (b * (slots + 1)));
-            k = (d >> b) & kmask;
+            lo = (lo & kmask) | d | (1u << (b * (slots + 1)));
             steps += more + 1;
             more = (uint32_t)-1;
-            if (c + slots > kMostDepartures) end = kEndField;
+            if (hi + slots >= kWalkCountMask) end = kEndField;
             if (steps > step_cap) end = kEndSteps;
             if (!on) end = kEndOk;
-        } else if (kTrees == 1) {
+        } else if (kOne) {
             __syncwarp();  // every lane has read the words of the last departure
         }
-        if (kTrees == 1 || on) {
-            const int32_t target = nbr_of<kDeg4>(rc, k, col);
-            word[u] = (uint64_t)(uint32_t)target | ((uint64_t)(count + left) << 32);
+        if (kOne || on) {
+            word[u] = (uint64_t)lo | ((uint64_t)hi << 32);
             ++more;
             u = v;
-            lo = w_next(x);
+            lo = (uint32_t)x;
             hi = (uint32_t)(x >> 32);
             hit = (int32_t)hi < 0;
         }
         const bool leave = hit || end != kEndOk;
-        return kTrees == 1 ? leave : __any_sync(kFull, leave);
+        return kOne ? leave : __any_sync(kFull, leave);
     };
 
     for (;;) {
@@ -277,13 +264,13 @@ __global__ void __launch_bounds__(32, kGroup == 32 ? 28 : (kGroup == 16 ? 20 : 2
                 const uint64_t x = word[s];
                 if (w_in_tree(x)) continue;  // an earlier path of this chunk took it
                 u = s;
-                lo = w_next(x);
+                lo = (uint32_t)x;
                 hi = (uint32_t)(x >> 32);
-                ra = load_rec(rec + s);
+                ra.load(g, s);
                 break;
             }
         }
-        if (kTrees == 1 ? !on : !__any_sync(kFull, on)) break;
+        if (kOne ? !on : !__any_sync(kFull, on)) break;
         // ---- departures
         for (;;) {
             if (depart(ra, rb)) {
@@ -302,8 +289,8 @@ __global__ void __launch_bounds__(32, kGroup == 32 ? 28 : (kGroup == 16 ? 20 : 2
                 hit = false;
                 start = true;
                 hi &= 0x7FFFFFFFu;
-                len = commit_path<kGroup, kDeg4>(gm, word, ord, rec, col, n, kmask, s, u,
-                                                 (int32_t)hi, pos);
+                len = commit_path<kGroup, kDeg4>(gm, word, ord, g, n, kmask, s, u, (int32_t)hi,
+                                                 pos);
                 if (len < 0) end = kEndField;
             }
             if (end != kEndOk) {
@@ -317,6 +304,36 @@ __global__ void __launch_bounds__(32, kGroup == 32 ? 28 : (kGroup == 16 ? 20 : 2
         }
         __syncwarp();
     }
+}
+
+template <int kGroup, bool kDeg4, bool kReject>
+__global__ void __launch_bounds__(32, kGroup == 32 ? 32 : 24)
+    k_wilson_queue(GraphView g, WaveView w, PhiloxKeys keys, uint64_t seed,
+                   const int64_t *__restrict__ sids, int bits, int slots, int64_t step_cap,
+                   volatile int32_t *done_flag) {
+    const int64_t t = (int64_t)blockIdx.x * (32 / kGroup) + threadIdx.x / kGroup;
+    const bool on = t < w.B;
+    walk_trees<kGroup, kDeg4, kReject>(g, w, keys, seed, (uint32_t)sids[on ? t : 0], t, on, bits,
+                                       slots, step_cap, done_flag);
+}
+
+// block j takes tree mw.entry[j].y of graph mw.entry[j].x
+__global__ void __launch_bounds__(32, 32) k_wilson_queue_multi(MultiWalk mw) {
+    const int e = mw.entry[blockIdx.x].x;
+    const int64_t t = mw.entry[blockIdx.x].y;
+    const GraphView g = mw.graphs[e];
+    const WaveView w = mw.waves[e];
+    const uint64_t seed = mw.seeds[e];
+    const PhiloxKeys keys = philox_keys(seed);
+    const uint32_t sample = (uint32_t)mw.sids[e][t];
+    const int bits = mw.queue_bits[e];
+    const int slots = kc_host::queue_slots(bits);
+    if (g.rec4)
+        walk_trees<32, true, false>(g, w, keys, seed, sample, t, true, bits, slots,
+                                    mw.step_caps[e], nullptr);
+    else
+        walk_trees<32, false, false>(g, w, keys, seed, sample, t, true, bits, slots,
+                                     mw.step_caps[e], nullptr);
 }
 
 }  // namespace
@@ -335,14 +352,14 @@ template <int kGroup, bool kDeg4>
 void launch_group(const GraphView &g, const WaveView &w, uint64_t seed, const int64_t *sids,
                   int bits, int64_t step_cap, bool reject, cudaStream_t s, int32_t *done_flag) {
     const PhiloxKeys K = host_keys(seed);
-    const QueueShape q{bits, std::min(kc_host::queue_slots(bits), kGroup)};
+    const int slots = std::min(kc_host::queue_slots(bits), kGroup);
     const unsigned blocks = (unsigned)((w.B * kGroup + 31) / 32);
     if (reject)
-        k_wilson_queue<kGroup, kDeg4, false, true><<<blocks, 32, 0, s>>>(
-            g, w, K, seed, sids, q, step_cap, done_flag, MultiWalk{});
+        k_wilson_queue<kGroup, kDeg4, true><<<blocks, 32, 0, s>>>(g, w, K, seed, sids, bits, slots,
+                                                                  step_cap, done_flag);
     else
-        k_wilson_queue<kGroup, kDeg4, false, false><<<blocks, 32, 0, s>>>(
-            g, w, K, seed, sids, q, step_cap, done_flag, MultiWalk{});
+        k_wilson_queue<kGroup, kDeg4, false><<<blocks, 32, 0, s>>>(g, w, K, seed, sids, bits,
+                                                                   slots, step_cap, done_flag);
 }
 }  // namespace
 
@@ -350,18 +367,16 @@ cudaError_t launch_wilson_queue(const GraphView &g, WaveView w, uint64_t seed,
                                 const int64_t *sids, int bits, int64_t step_cap, bool reject,
                                 int64_t num_sms, cudaStream_t s, int32_t *done_flag) {
     const int group = kc_host::queue_group(w.B, num_sms);
-    const bool deg4 = bits <= 2;
+    const bool deg4 = g.rec4 != nullptr;
     auto *launch = group == 32 ? (deg4 ? launch_group<32, true> : launch_group<32, false>)
-                 : group == 16 ? (deg4 ? launch_group<16, true> : launch_group<16, false>)
-                               : (deg4 ? launch_group<8, true> : launch_group<8, false>);
+                               : (deg4 ? launch_group<16, true> : launch_group<16, false>);
     launch(g, w, seed, sids, bits, step_cap, reject, s, done_flag);
     return cudaGetLastError();
 }
 
 cudaError_t launch_wilson_queue_multi(const MultiWalk &mw, cudaStream_t s) {
     if (mw.count <= 0) return cudaSuccess;
-    k_wilson_queue<32, false, true, false><<<(unsigned)mw.count, 32, 0, s>>>(
-        GraphView{}, WaveView{}, PhiloxKeys{}, 0, nullptr, QueueShape{1, 1}, 0, nullptr, mw);
+    k_wilson_queue_multi<<<(unsigned)mw.count, 32, 0, s>>>(mw);
     return cudaGetLastError();
 }
 

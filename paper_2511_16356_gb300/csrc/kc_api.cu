@@ -90,6 +90,7 @@ GraphView view_of(const kc_graph *g) {
     v.col = g->d_col;
     v.deg = g->d_deg;
     v.rec = g->d_rec;
+    v.rec4 = g->max_deg <= 4 ? g->d_rec4 : nullptr;
     v.root = g->root;
     v.ecc = g->ecc;
     v.p0 = g->d_p0;
@@ -443,7 +444,7 @@ int pop_trees(kc_graph *g, const PopTask &task, const WaveView &w, bool in_memor
 void init_queues(kc_graph *g, const GraphView &gv, const WaveView &w, const int64_t *sids,
                  int32_t root, cudaStream_t s) {
     KC_CK(g, launch_queue_init(gv, w, g->seed, sids, root, kc_host::queue_bits(g->max_deg),
-                               g->ttf_variant == KC_TTF_BIT ? 32 : 2, s));
+                               g->ttf_variant == KC_TTF_BIT ? 10 : 2, s));
 }
 
 // Words and order of a wave before its walk, rooted at g->root.
@@ -1108,7 +1109,8 @@ void edit_graph(kc_graph *g, int32_t u, int32_t v, bool insert) {
     g->m += insert ? 1 : -1;
     g->max_deg += insert ? 1 : 0;
     g->host_csr_stale = true;
-    KC_CK(g, launch_build_records(view_of(g), g->d_rec, g->d_deg, g->stream));
+    KC_CK(g, launch_build_records(view_of(g), g->d_rec, g->max_deg <= 4 ? g->d_rec4 : nullptr,
+                                  g->d_deg, g->stream));
     g->t_update.launches += 4;
 }
 
@@ -2101,6 +2103,7 @@ kc_status kc_graph_destroy(kc_graph *g) {
     dfree(g->d_col);
     dfree(g->d_deg);
     dfree(g->d_rec);
+    dfree(g->d_rec4);
     dfree(g->d_p0);
     dfree(g->d_level0);
     dfree(g->d_in0);
@@ -2204,6 +2207,7 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
         g->col_cap = (size_t)twom;
         dalloc(g, &g->d_deg, n);
         dalloc(g, &g->d_rec, n);
+        if (g->max_deg <= 4) dalloc(g, &g->d_rec4, n);
         dalloc(g, &g->d_p0, n);
         dalloc(g, &g->d_level0, n);
         dalloc(g, &g->d_in0, n);
@@ -2219,7 +2223,7 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
         Phase ph(g, g->t_setup);
         int launches = 0;
         GraphView gv = view_of(g);
-        KC_CK(g, launch_build_records(gv, g->d_rec, g->d_deg, g->stream));
+        KC_CK(g, launch_build_records(gv, g->d_rec, g->d_rec4, g->d_deg, g->stream));
         ++launches;
         uint32_t *d_flags = g->d_err;
         KC_CK(g, cudaMemsetAsync(d_flags, 0, 4 * sizeof(uint32_t), g->stream));

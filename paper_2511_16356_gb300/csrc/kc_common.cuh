@@ -216,6 +216,7 @@ struct GraphView {
     const int32_t *col;      // [2m]
     const int32_t *deg;      // [n]
     const VRec *rec;         // [n]
+    const int4 *rec4;        // [n] the neighbours where every degree is at most 4, else null
     int32_t root;
     int32_t ecc;
     const int32_t *p0;       // [n] tau0 parent, -1 at the root
@@ -292,6 +293,7 @@ struct kc_graph {
     int32_t *d_col = nullptr;
     int32_t *d_deg = nullptr;
     kc::VRec *d_rec = nullptr;
+    int4 *d_rec4 = nullptr;  // used while max_deg <= 4
     int32_t root = -1, ecc = 0;
     int32_t *d_p0 = nullptr, *d_level0 = nullptr, *d_in0 = nullptr, *d_out0 = nullptr;
     int32_t ttf_variant = KC_TTF_SCAN;
@@ -367,7 +369,9 @@ struct kc_graph {
 namespace kc {
 
 // Launch helpers implemented in the .cu files.  Each returns cudaGetLastError().
-cudaError_t launch_build_records(const GraphView &g, VRec *rec, int32_t *deg, cudaStream_t s);
+// rec4: [n] or null (some degree exceeds 4)
+cudaError_t launch_build_records(const GraphView &g, VRec *rec, int4 *rec4, int32_t *deg,
+                                 cudaStream_t s);
 cudaError_t launch_validate(const GraphView &g, uint32_t *flags, cudaStream_t s);
 cudaError_t launch_root(const GraphView &g, unsigned long long *best, cudaStream_t s);
 cudaError_t launch_bfs_init(int64_t n, int32_t r, int32_t *level, cudaStream_t s);

@@ -99,27 +99,26 @@ inline int64_t reject_wave_size(int64_t need, int64_t drawn, int64_t accepted, d
 }
 
 // Arrow queues of the one-walker kernels (k1_solo.cu): bits of a neighbour index
-// in a graph of largest degree max_deg, and how many arrows a queue of
-// kQueueWidth bits holds behind the last one taken and before its end mark.  At
-// most kMaxQueueBits bits leave room for one.
-constexpr int kQueueWidth = 17;
-constexpr int kMaxQueueBits = (kQueueWidth - 1) / 2;
+// in a graph of largest degree max_deg (at least 2), and how many arrows a queue of
+// 32 bits holds behind the last one taken and before its end mark.  At most
+// kMaxQueueBits bits leave room for one.
+constexpr int kMaxQueueBits = 15;
 constexpr int queue_bits(int64_t max_deg) {
-    int b = 1;
+    int b = 2;
     while (b < 63 && ((int64_t)1 << b) < max_deg) ++b;
     return b;
 }
-constexpr int queue_slots(int bits) { return (kQueueWidth - 1 - bits) / bits; }
+constexpr int queue_slots(int bits) { return (31 - bits) / bits; }
 
-// Lanes per tree of those kernels for a wave of B trees (32, 16 or 8): one tree
-// per warp while all are resident (28 an SM), as it has the shortest chain per
-// departure; then as many trees per warp as make them resident (40 and 96 an
-// SM).  350x350 grid under a cap of 13 n departures, walk in ms for 32 / 16 / 8
-// lanes: 3044 trees 347 / 469 / 645, 4522 trees 549 / 508 / 666, 8929 trees
-// 904 / 975 / 726, 17672 trees 1579 / 1551 / 1423.
+// Lanes per tree of those kernels for a wave of B trees: one tree per warp, which
+// has the shortest chain per departure, unless the wave is a little too large for
+// all of them to be resident (32 an SM) and two trees per warp make them so (48).
+// 350x350 grid under a cap of 13 n departures, walk in ms for 32 / 16 / 8 lanes: 3044
+// trees 260 / 362 / 523, 4522 trees 345 / 397 / 546, 5991 trees 482 / 430 / 575, 8929
+// trees 628 / 742 / 620, 17672 trees 1133 / 1174 / 1204.
 inline int queue_group(int64_t B, int64_t num_sms) {
     const int64_t per_sm = (B + std::max<int64_t>(num_sms, 1) - 1) / std::max<int64_t>(num_sms, 1);
-    return per_sm <= 28 ? 32 : (per_sm <= 40 ? 16 : 8);
+    return per_sm > 32 && per_sm <= 48 ? 16 : 32;
 }
 
 // Cycle popping in shared memory (k_pop_small): its bytes for n vertices (two

@@ -67,16 +67,17 @@ SMALL = {
 
 @pytest.mark.parametrize("name,trees", [(k, 40) for k in SMALL] +
                          [("K3", 100000), ("star40", 3000), ("er300", 5000),
+                          ("grid17x13", 6000), ("er300", 7200),
                           ("grid17x13", 9800), ("er300", 20000), ("grid17x13", 40000)])
 def test_arrows_drawn_ahead_match_oracle(name, trees):
-    """One walker per tree, one to 32 trees per warp (40 trees up to 40000)."""
+    """One walker per tree, one and two trees per warp (5000 and 6000 trees)."""
     g = SMALL[name]()
     with kc.KemenyGraph.from_graph(g, _cfg(walker=kc.KC_WALK_LANE)) as G:
         G.sample(17, trees)
         _check(g, G.samples(), 17, 0, trees)
 
 
-@pytest.mark.parametrize("name,trees", [("cycle500", 64), ("grid17x13", 4000)])
+@pytest.mark.parametrize("name,trees", [("cycle500", 64), ("grid17x13", 3600)])
 def test_arrows_drawn_ahead_reject_match_oracle(name, trees):
     """Rejection by walk length, one tree and several trees per warp."""
     g = SMALL[name]()
