@@ -32,13 +32,20 @@ namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-__device__ __forceinline__ const int32_t *parents(const ParTrees &p, int64_t t, int64_t n) {
-    return p.par + (p.slot ? p.slot[t] : t) * n;
+// the parents of tree t
+struct Parents {
+    const int32_t *par;
+    int stride;
+    __device__ __forceinline__ int32_t operator[](int64_t v) const { return par[v * stride]; }
+};
+__device__ __forceinline__ Parents parents(const ParTrees &p, int64_t t, int64_t n) {
+    const int64_t row = p.slot ? p.slot[t] : (p.map ? (int64_t)p.map[t] : t);
+    return Parents{p.par + row * n * p.stride, p.stride};
 }
 
 __global__ void k_par_count(int64_t n, WaveView w, ParTrees trees) {
     const int64_t t = blockIdx.y;
-    const int32_t *__restrict__ par = parents(trees, t, n);
+    const Parents par = parents(trees, t, n);
     uint64_t *word = w.word + t * n;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
@@ -51,7 +58,7 @@ __global__ void k_par_count(int64_t n, WaveView w, ParTrees trees) {
 __global__ void k_par_up(GraphView g, WaveView w, ParTrees trees) {
     const int64_t n = g.n;
     const int64_t t = blockIdx.y;
-    const int32_t *__restrict__ par = parents(trees, t, n);
+    const Parents par = parents(trees, t, n);
     uint64_t *word = w.word + t * n;
     int32_t *size = w.size + t * n;
     int64_t *vol = w.vol + t * n;
@@ -94,7 +101,7 @@ __global__ void __launch_bounds__(256) k_par_sibling_rows(GraphView g, WaveView 
     const int lane = threadIdx.x & 31;
     const int64_t n = g.n;
     const int64_t t = blockIdx.y;
-    const int32_t *__restrict__ par = parents(trees, t, n);
+    const Parents par = parents(trees, t, n);
     const int32_t *__restrict__ size = w.size + t * n;
     uint64_t *word = w.word + t * n;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -167,7 +174,7 @@ __global__ void k_par_jump(GraphView g, WaveView w, int want_pre) {
 __global__ void k_par_depth_init(GraphView g, WaveView w, ParTrees trees) {
     const int64_t n = g.n;
     const int64_t t = blockIdx.y;
-    const int32_t *__restrict__ par = parents(trees, t, n);
+    const Parents par = parents(trees, t, n);
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x)
         w.word[t * n + v] = v == g.root ? (uint64_t)(uint32_t)v
@@ -178,7 +185,8 @@ __global__ void k_par_depth_init(GraphView g, WaveView w, ParTrees trees) {
 
 cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool by_id,
                                     int32_t eu, int32_t ev, bool want_preorder, cudaStream_t s,
-                                    int *launches) {
+                                    int *launches, uint64_t *scratch) {
+    if (scratch) w.word = scratch;  // the kernels' word
     const size_t per = (size_t)(w.B * g.n);
     cudaError_t e;
     if ((e = cudaMemsetAsync(w.word, 0, sizeof(uint64_t) * per, s)) != cudaSuccess) return e;

@@ -132,7 +132,8 @@ __device__ __forceinline__ uint32_t led_cycle(volatile uint32_t *nx, uint32_t a)
 // instead of raising an error.
 enum : int { kFused = 0, kTrees = 1, kTreesCsr = 2 };
 template <int kThreads, bool kMulti, int kKind>
-__global__ void __launch_bounds__(kThreads, kThreads <= 128 ? 10 : (kThreads <= 256 ? 5 : 1))
+__global__ void __launch_bounds__(kThreads,
+                                  kThreads <= 128 ? 10 : (kThreads <= 256 ? 5 : 1024 / kThreads))
     k_pop_small(PopTask one, const PopTask *__restrict__ tasks, const int2 *__restrict__ entry) {
     const int64_t t = kMulti ? (int64_t)entry[blockIdx.x].y : (int64_t)blockIdx.x;
     const PopTask task = kMulti ? tasks[entry[blockIdx.x].x] : one;
@@ -587,6 +588,7 @@ cudaError_t launch_small_any(const PopTask &one, const PopTask *tasks, const int
     switch (kc_host::pop_small_threads(max_n)) {
         case 128: return launch_small<128, kMulti, kKind>(one, tasks, entry, blocks, max_n, s);
         case 256: return launch_small<256, kMulti, kKind>(one, tasks, entry, blocks, max_n, s);
+        case 512: return launch_small<512, kMulti, kKind>(one, tasks, entry, blocks, max_n, s);
         default: return launch_small<1024, kMulti, kKind>(one, tasks, entry, blocks, max_n, s);
     }
 }

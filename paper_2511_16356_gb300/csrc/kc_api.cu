@@ -354,6 +354,38 @@ int eval_ttf_bit(kc_graph *g, const GraphView &gv, const Plan &p, const WaveView
     return 1;
 }
 
+// Start order of the concurrent walkers: a fixed pseudo-random permutation
+// (vertices sorted by a 32-bit mix of their id, which is a bijection), so that the
+// 32 walkers of a tree start far apart and rarely block each other.  Any order
+// gives the same trees; starting walkers next to each other (for example in BFS
+// order around the root) makes them collide constantly.  Built when a handle is
+// created whose waves use it, and otherwise when the 32-walker kernel takes a wave
+// over (300000 vertices: about 20 ms of a host core).
+const int32_t *start_order(kc_graph *g) {
+    if (g->d_sorder) return g->d_sorder;
+    const int64_t n = g->n;
+    std::vector<uint64_t> key((size_t)n);
+    for (int64_t v = 0; v < n; ++v) {
+        uint32_t h = (uint32_t)v * 0x9E3779B1u;
+        h ^= h >> 15;
+        h *= 0x85EBCA77u;
+        h ^= h >> 13;
+        h *= 0xC2B2AE3Du;
+        h ^= h >> 16;
+        key[(size_t)v] = ((uint64_t)h << 32) | (uint64_t)(uint32_t)v;
+    }
+    std::sort(key.begin(), key.end());
+    std::vector<int32_t> order((size_t)n);
+    for (int64_t v = 0; v < n; ++v) order[(size_t)v] = (int32_t)(uint32_t)key[(size_t)v];
+    int32_t *d = nullptr;
+    dalloc(g, &d, (size_t)n);
+    const cudaError_t e =
+        copy_sync(g, d, order.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) dfree(d);
+    KC_CK(g, e);
+    return g->d_sorder = d;
+}
+
 // Cap on Wilson departures (per tree for the one-walker kernel, per walker for
 // the 32-walker kernel): the configured value, or max(2^22, 1024 n) (about 60
 // times the mean step count of a road-shaped graph, far above that of
@@ -370,14 +402,36 @@ int fast_traversal(const kc_graph *g) {
     return (g->ttf_variant == KC_TTF_SCAN && g->n >= (1 << 16)) ? kTravLeafUp : kTravChunked;
 }
 
+// Traversal of a sub-wave's walked trees for f; depth bounds the trees' depths.
+// Trees of the BIT variant go through the order-free passes, which take a dependent
+// step (about 1.2 us) per level where the passes over the parent-first order take
+// two per 32 vertices (4.7 us together): the latter serve small graphs and trees
+// deeper than n / 8.
+void traverse_for_f(kc_graph *g, const GraphView &gv, const WaveView &w, bool bit, int64_t depth,
+                    cudaStream_t s, int *launches) {
+    if (bit && g->n >= 8192 && depth <= g->n / 8) {
+        ParTrees trees;
+        trees.par = reinterpret_cast<const int32_t *>(w.word);  // low halves
+        trees.map = w.tmap;
+        trees.stride = 2;
+        KC_CK(g, launch_traverse_parents(gv, w, trees, false, -1, -1, true, s, launches,
+                                         reinterpret_cast<uint64_t *>(w.bit)));
+        return;
+    }
+    KC_CK(g, launch_traverse(gv, w, bit, s, launches, fast_traversal(g)));
+}
+
 // Whether waves run the one-walker kernels with arrows drawn ahead (k1_solo.cu)
 // in place of the handle's walker: always for LANE, and under AUTO on
 // long-diameter graphs, where 32 walkers of a tree mostly wait for one another
 // (40000-vertex grid, walk in ms with 32 walkers / one: 64 trees 192 / 114, 500
 // trees 348 / 184, 4000 trees 590 / 316).  On graphs of low diameter the 32
 // walkers spread and stay faster (20000-vertex random graph: 24 / 28 ms).
+bool fits_queues(const kc_graph *g) {
+    return kc_host::queue_bits(g->max_deg) <= kc_host::kMaxQueueBits;
+}
 bool use_solo(const kc_graph *g) {
-    if (kc_host::queue_bits(g->max_deg) > kc_host::kMaxQueueBits) return false;
+    if (!fits_queues(g)) return false;
     if (g->walker == KC_WALK_LANE) return true;
     return g->walker == KC_WALK_WARP && g->auto_walker &&
            g->ttf_variant == KC_TTF_BIT;
@@ -473,7 +527,7 @@ void run_wilson(kc_graph *g, const GraphView &gv, const WaveView &w, const Carve
     } else if (g->walker == KC_WALK_LANE) {
         KC_CK(g, launch_wilson(gv, w, g->seed, c.sids, cap, g->stream));
     } else if (g->walker == KC_WALK_WARP) {
-        KC_CK(g, launch_wilson_warp(gv, w, g->seed, c.sids, g->d_sorder, cap, g->stream));
+        KC_CK(g, launch_wilson_warp(gv, w, g->seed, c.sids, start_order(g), cap, g->stream));
     } else {
         // lane walkers take the first starts of the hashed order (the long
         // early walks, where concurrent walkers would mostly wait on each
@@ -484,9 +538,9 @@ void run_wilson(kc_graph *g, const GraphView &gv, const WaveView &w, const Carve
         const int64_t q_stop = pm >= 1000 ? g->n : (g->n * pm) / 1000;
         const int64_t stop_at = tm >= 1000 ? 0 : std::max<int64_t>(1, (w.B * tm + 999) / 1000);
         KC_CK(g, cudaMemsetAsync(c.done, 0, sizeof(unsigned int), g->stream));
-        KC_CK(g, launch_wilson(gv, w, g->seed, c.sids, cap, g->stream, g->d_sorder, c.rs_q,
+        KC_CK(g, launch_wilson(gv, w, g->seed, c.sids, cap, g->stream, start_order(g), c.rs_q,
                                c.rs_pos, c.done, q_stop, stop_at));
-        KC_CK(g, launch_wilson_warp(gv, w, g->seed, c.sids, g->d_sorder, cap, g->stream, c.rs_q,
+        KC_CK(g, launch_wilson_warp(gv, w, g->seed, c.sids, start_order(g), cap, g->stream, c.rs_q,
                                     c.rs_pos));
     }
 }
@@ -570,10 +624,10 @@ bool run_wave_pipelined(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool reje
             KC_CK(g, launch_wilson(gv, w, g->seed, c.sids, step_cap_of(g), s1, nullptr, nullptr,
                                    nullptr, nullptr, 0, 0, g->d_done));
     } else if (reject) {
-        KC_CK(g, launch_wilson_warp_reject(gv, w, g->seed, c.sids, g->d_sorder,
+        KC_CK(g, launch_wilson_warp_reject(gv, w, g->seed, c.sids, start_order(g),
                                            g->cfg.reject_steps, s1, g->d_done));
     } else {
-        KC_CK(g, launch_wilson_warp(gv, w, g->seed, c.sids, g->d_sorder, step_cap_of(g), s1,
+        KC_CK(g, launch_wilson_warp(gv, w, g->seed, c.sids, start_order(g), step_cap_of(g), s1,
                                     nullptr, nullptr, g->d_done));
     }
     KC_CK(g, cudaEventRecord(ev_w1, s1));
@@ -625,7 +679,7 @@ bool run_wave_pipelined(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool reje
             std::array<cudaEvent_t, 3> e3 = {event(), event(), event()};
             KC_CK(g, cudaEventRecord(e3[0], s2));
             int nl = 0;
-            KC_CK(g, launch_traverse(gv, sv, p.bit, s2, &nl, fast_traversal(g)));
+            traverse_for_f(g, gv, sv, p.bit, md, s2, &nl);
             g->t_traverse.launches += nl;
             KC_CK(g, cudaEventRecord(e3[1], s2));
             if (p.bit) g->t_ttf.launches += eval_ttf_bit(g, gv, p, sv, wdone, spare, s2);
@@ -757,7 +811,7 @@ bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
     KC_CK(g, launch_iota(c.sids, sid0, B, g->stream));
     reset_segtab(g, B);
     uint32_t hdr[2] = {0, 0};
-    for (bool solo = use_solo(g);; solo = false) {
+    for (bool solo = use_solo(g) || (canonical && use_pop(g) && fits_queues(g));; solo = false) {
         KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
         {
             Phase ph(g, g->t_init);
@@ -797,8 +851,10 @@ bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
         {
             Phase ph(g, g->t_traverse);
             int nl = 0;
-            KC_CK(g, launch_traverse(gv, s, p.bit, g->stream, &nl,
-                                     canonical ? kTravCanonical : fast_traversal(g)));
+            if (canonical)
+                KC_CK(g, launch_traverse(gv, s, p.bit, g->stream, &nl, kTravCanonical));
+            else
+                traverse_for_f(g, gv, s, p.bit, (int64_t)hdr[1], g->stream, &nl);
             ph.done(nl);
         }
         {
@@ -963,7 +1019,7 @@ void build_tau0_wilson(kc_graph *g, int &launches) {
     KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
     KC_CK(g, launch_iota(c.sids, 0, 1, g->stream));
     KC_CK(g, launch_wave_init(gv, w, g->stream));
-    KC_CK(g, launch_wilson_warp(gv, w, g->cfg.tau0_seed, c.sids, g->d_sorder, step_cap_of(g),
+    KC_CK(g, launch_wilson_warp(gv, w, g->cfg.tau0_seed, c.sids, start_order(g), step_cap_of(g),
                                 g->stream));
     int32_t *d_cnt = (int32_t *)g->d_scratch;  // [0] deepest, [1] outside the tree
     KC_CK(g, cudaMemsetAsync(d_cnt, 0, 2 * sizeof(int32_t), g->stream));
@@ -1539,7 +1595,7 @@ void run_wave_reject(kc_graph *g, Plan &p, int64_t B, int64_t sid0) {
                 KC_CK(g, launch_wilson_reject(gv, w, g->seed, c.sids, nullptr,
                                               g->cfg.reject_steps, g->stream));
             else
-                KC_CK(g, launch_wilson_warp_reject(gv, w, g->seed, c.sids, g->d_sorder,
+                KC_CK(g, launch_wilson_warp_reject(gv, w, g->seed, c.sids, start_order(g),
                                                    g->cfg.reject_steps, g->stream));
             ph.done(1);
         }
@@ -1582,7 +1638,7 @@ void run_wave_reject(kc_graph *g, Plan &p, int64_t B, int64_t sid0) {
         {
             Phase ph(g, g->t_traverse);
             int nl = 0;
-            KC_CK(g, launch_traverse(gv, sv, p.bit, g->stream, &nl, fast_traversal(g)));
+            traverse_for_f(g, gv, sv, p.bit, (int64_t)hdr[1], g->stream, &nl);
             ph.done(nl);
         }
         {
@@ -1789,7 +1845,7 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                 wv.push_back(w);
                 seeds.push_back(g->seed);
                 sids.push_back(c.sids);
-                sorders.push_back(g->d_sorder);
+                sorders.push_back(nullptr);  // set below for the 32-walker launch
                 caps.push_back(step_cap_of(g));
                 qbits.push_back(kc_host::queue_bits(g->max_deg));
                 idx.push_back(i);
@@ -1858,7 +1914,10 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                                               pop_par(g, wv[k])),
                                   wv[k], pop[k] == kPopLarge);
                     else if (solo[k]) init_queues(g, gv[k], wv[k], sids[k], g->root, s0);
-                    else KC_CK(g, launch_wave_init(gv[k], wv[k], s0));
+                    else {
+                        sorders[k] = start_order(g);
+                        KC_CK(g, launch_wave_init(gv[k], wv[k], s0));
+                    }
                 }
                 const size_t bytes = (sizeof(GraphView) + sizeof(WaveView) + sizeof(PopTask)) * G +
                                      8 * G * 5 + sizeof(int2) * entry.size() + 256 * 9;
@@ -1976,7 +2035,7 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                     sw.steps = w.steps + sub;
                     sw.f = w.f + sub;
                     int nl = 0;
-                    KC_CK(g, launch_traverse(v, sw, p.bit, s0, &nl, fast_traversal(g)));
+                    traverse_for_f(g, v, sw, p.bit, (int64_t)hdr[1], s0, &nl);
                     if (p.bit) KC_CK(g, launch_ttf_bit(v, sw, s0));
                     else KC_CK(g, launch_ttf_scan(v, sw, s0));
                     g->t_traverse.launches += nl;
@@ -2172,14 +2231,16 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
     try {
         clear_stale_error();
         KC_CK(g, cudaGetDevice(&g->device));
-        cudaDeviceProp prop;
-        KC_CK(g, cudaGetDeviceProperties(&prop, g->device));
-        if (prop.major != 10 || prop.minor != 3) {
+        int major = 0, minor = 0, sms = 0;
+        KC_CK(g, cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, g->device));
+        KC_CK(g, cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, g->device));
+        KC_CK(g, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device));
+        if (major != 10 || minor != 3) {
             g->last_error = "the library is built for sm_103a only";
             throw Fail{KC_ERR_NO_DEVICE};
         }
-        g->resident_trees = (int64_t)prop.multiProcessorCount * wilson_warp_blocks_per_sm();
-        g->num_sms = prop.multiProcessorCount;
+        g->resident_trees = (int64_t)sms * wilson_warp_blocks_per_sm();
+        g->num_sms = sms;
         KC_CK(g, cudaEventCreate(&g->ev0));
         KC_CK(g, cudaEventCreate(&g->ev1));
         g->n = n;
@@ -2187,9 +2248,15 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
             throw Fail{KC_ERR_INVALID_ARG};
         g->next_sid = cfg.sample_id_base;
         // host copy of the CSR (validated layout, kept for updates)
-        g->h_row_off.resize((size_t)n + 1);
-        const cudaMemcpyKind kind = cfg.inputs_on_device ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost;
-        KC_CK(g, copy_sync(g, g->h_row_off.data(), row_off, sizeof(int64_t) * (n + 1), kind));
+        auto take = [&](auto &dst, const auto *src, size_t count) {
+            if (!cfg.inputs_on_device) {
+                dst.assign(src, src + count);
+                return;
+            }
+            dst.resize(count);
+            KC_CK(g, copy_sync(g, dst.data(), src, sizeof(*src) * count, cudaMemcpyDeviceToHost));
+        };
+        take(g->h_row_off, row_off, (size_t)n + 1);
         if (g->h_row_off[0] != 0) throw Fail{KC_ERR_INVALID_ARG};
         for (int64_t v = 0; v < n; ++v) {
             const int64_t d = g->h_row_off[v + 1] - g->h_row_off[v];
@@ -2199,8 +2266,7 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
         const int64_t twom = g->h_row_off[n];
         if (twom % 2 != 0 || twom == 0) throw Fail{twom == 0 ? KC_ERR_DISCONNECTED : KC_ERR_NOT_SYMMETRIC};
         g->m = twom / 2;
-        g->h_col.resize((size_t)twom);
-        KC_CK(g, copy_sync(g, g->h_col.data(), col, sizeof(int32_t) * twom, kind));
+        take(g->h_col, col, (size_t)twom);
 
         dalloc(g, &g->d_row_off, n + 1);
         dalloc(g, &g->d_col, twom);
@@ -2254,32 +2320,6 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
             if (cfg.root == -1) g->root = central_root(g, g->root, launches);
         }
         gv.root = g->root;
-        // Start order of the concurrent walkers: a fixed pseudo-random
-        // permutation (vertices sorted by a 32-bit mix of their id), so that the
-        // 32 walkers of a tree start far apart and rarely block each other.  Any
-        // order gives the same trees; starting walkers next to each other (for
-        // example in BFS order around the root) makes them collide constantly.
-        {
-            std::vector<uint64_t> key((size_t)n);
-            for (int64_t v = 0; v < n; ++v) {
-                uint32_t h = (uint32_t)v * 0x9E3779B1u;
-                h ^= h >> 15;
-                h *= 0x85EBCA77u;
-                h ^= h >> 13;
-                h *= 0xC2B2AE3Du;
-                h ^= h >> 16;
-                key[(size_t)v] = ((uint64_t)h << 32) | (uint64_t)(uint32_t)v;
-            }
-            std::vector<int32_t> order((size_t)n);
-            for (int64_t v = 0; v < n; ++v) order[(size_t)v] = (int32_t)v;
-            std::sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
-                return key[(size_t)a] < key[(size_t)b] || (key[(size_t)a] == key[(size_t)b] && a < b);
-            });
-            dalloc(g, &g->d_sorder, n);
-            KC_CK(g, cudaMemcpyAsync(g->d_sorder, order.data(), sizeof(int32_t) * n,
-                                     cudaMemcpyHostToDevice, g->stream));
-            KC_CK(g, cudaStreamSynchronize(g->stream));
-        }
         build_tau0(g, launches);
         gv.ecc = g->ecc;
 
@@ -2308,6 +2348,7 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
                          ? KC_WALK_LANE : KC_WALK_WARP;
         g->walker = walker;
         g->auto_walker = cfg.walker == KC_WALK_AUTO && !cfg.autotune;
+        if (!use_solo(g) && !use_pop(g)) start_order(g);
     } catch (Fail &f) {
         kc_graph_destroy(g);
         return f.st;

@@ -146,6 +146,10 @@ inline int pop_kind(int64_t n, int64_t twom, int64_t root_deg) {
     if (16 * (twom / std::max<int64_t>(root_deg, 1)) <= n) return kPopLarge;
     return n <= kPopContractMax ? kPopTrees : kPopNone;
 }
-inline int pop_small_threads(int64_t n) { return n <= 1024 ? 128 : (n <= 4096 ? 256 : 1024); }
+// Threads of a block: most of a tree's time is a few long chains, so blocks stay small
+// enough that an SM holds as many as its shared memory does.
+inline int pop_small_threads(int64_t n) {
+    return n <= 1024 ? 128 : (n <= 4096 ? 256 : (n <= 8192 ? 512 : 1024));
+}
 
 }  // namespace kc_host

@@ -94,7 +94,7 @@ def test_arrows_drawn_ahead_reject_match_oracle(name, trees):
     assert np.array_equal(got["f"], f_ref)
 
 
-@pytest.mark.parametrize("n", [2, 3, 31, 33, 1024, 1025, 4096, 4097, 16000, 16001])
+@pytest.mark.parametrize("n", [2, 3, 31, 33, 1024, 1025, 4096, 4097, 8192, 8193, 16000, 16001])
 def test_popped_trees_match_oracle(n):
     """Cycle popping in shared memory (up to 16000 vertices; past them the walkers),
     at the edges of its block sizes: f, step counts and a kept tree."""

@@ -73,7 +73,7 @@ def test_popped_trees_fit_a_block(queue):
     assert top < 1 << 16 and queue.hq_pop_bytes(top) + 64 <= 227 * 1024
     for n in (2, 3, 1024, 1025, 4096, 4097, top):
         assert 14 * n <= queue.hq_pop_bytes(n) <= 14 * n + 2
-        assert queue.hq_pop_threads(n) in (128, 256, 1024)
+        assert queue.hq_pop_threads(n) in (128, 256, 512, 1024)
         assert queue.hq_pop(n, 10 * n, 1) == 1
     for contract, each in ((1, 6), (0, 4)):
         n = queue.hq_trees_max(contract)
