@@ -10,6 +10,11 @@
 // vertex's own word then holds its preorder relative to its parent, and all
 // vertices jump to the root along those words at once (k_par_jump).
 //
+// Deep trees (grids) stay with the passes over the order: a report and the last
+// child's wait for it cost a chain of atomics per level, and beside a running walk
+// those took 89 ms for the 4500 trees of a 350x350 grid where the ordered passes
+// take 53, and slowed the walk by a tenth.
+//
 // Word of a vertex: until it reports, unreported children (high half) and sizes
 // reported (low half); then preorder offset (high half) and the ancestor it is
 // relative to (low half).  The second pair is read and written whole and holds at
@@ -32,20 +37,13 @@ namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// the parents of tree t
-struct Parents {
-    const int32_t *par;
-    int stride;
-    __device__ __forceinline__ int32_t operator[](int64_t v) const { return par[v * stride]; }
-};
-__device__ __forceinline__ Parents parents(const ParTrees &p, int64_t t, int64_t n) {
-    const int64_t row = p.slot ? p.slot[t] : (p.map ? (int64_t)p.map[t] : t);
-    return Parents{p.par + row * n * p.stride, p.stride};
+__device__ __forceinline__ const int32_t *parents(const ParTrees &p, int64_t t, int64_t n) {
+    return p.par + (p.slot ? p.slot[t] : t) * n;
 }
 
 __global__ void k_par_count(int64_t n, WaveView w, ParTrees trees) {
     const int64_t t = blockIdx.y;
-    const Parents par = parents(trees, t, n);
+    const int32_t *__restrict__ par = parents(trees, t, n);
     uint64_t *word = w.word + t * n;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
@@ -58,7 +56,7 @@ __global__ void k_par_count(int64_t n, WaveView w, ParTrees trees) {
 __global__ void k_par_up(GraphView g, WaveView w, ParTrees trees) {
     const int64_t n = g.n;
     const int64_t t = blockIdx.y;
-    const Parents par = parents(trees, t, n);
+    const int32_t *__restrict__ par = parents(trees, t, n);
     uint64_t *word = w.word + t * n;
     int32_t *size = w.size + t * n;
     int64_t *vol = w.vol + t * n;
@@ -101,7 +99,7 @@ __global__ void __launch_bounds__(256) k_par_sibling_rows(GraphView g, WaveView 
     const int lane = threadIdx.x & 31;
     const int64_t n = g.n;
     const int64_t t = blockIdx.y;
-    const Parents par = parents(trees, t, n);
+    const int32_t *__restrict__ par = parents(trees, t, n);
     const int32_t *__restrict__ size = w.size + t * n;
     uint64_t *word = w.word + t * n;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -174,7 +172,7 @@ __global__ void k_par_jump(GraphView g, WaveView w, int want_pre) {
 __global__ void k_par_depth_init(GraphView g, WaveView w, ParTrees trees) {
     const int64_t n = g.n;
     const int64_t t = blockIdx.y;
-    const Parents par = parents(trees, t, n);
+    const int32_t *__restrict__ par = parents(trees, t, n);
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x)
         w.word[t * n + v] = v == g.root ? (uint64_t)(uint32_t)v
@@ -185,8 +183,7 @@ __global__ void k_par_depth_init(GraphView g, WaveView w, ParTrees trees) {
 
 cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool by_id,
                                     int32_t eu, int32_t ev, bool want_preorder, cudaStream_t s,
-                                    int *launches, uint64_t *scratch) {
-    if (scratch) w.word = scratch;  // the kernels' word
+                                    int *launches) {
     const size_t per = (size_t)(w.B * g.n);
     cudaError_t e;
     if ((e = cudaMemsetAsync(w.word, 0, sizeof(uint64_t) * per, s)) != cudaSuccess) return e;

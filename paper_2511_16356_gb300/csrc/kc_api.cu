@@ -402,25 +402,6 @@ int fast_traversal(const kc_graph *g) {
     return (g->ttf_variant == KC_TTF_SCAN && g->n >= (1 << 16)) ? kTravLeafUp : kTravChunked;
 }
 
-// Traversal of a sub-wave's walked trees for f; depth bounds the trees' depths.
-// Trees of the BIT variant go through the order-free passes, which take a dependent
-// step (about 1.2 us) per level where the passes over the parent-first order take
-// two per 32 vertices (4.7 us together): the latter serve small graphs and trees
-// deeper than n / 8.
-void traverse_for_f(kc_graph *g, const GraphView &gv, const WaveView &w, bool bit, int64_t depth,
-                    cudaStream_t s, int *launches) {
-    if (bit && g->n >= 8192 && depth <= g->n / 8) {
-        ParTrees trees;
-        trees.par = reinterpret_cast<const int32_t *>(w.word);  // low halves
-        trees.map = w.tmap;
-        trees.stride = 2;
-        KC_CK(g, launch_traverse_parents(gv, w, trees, false, -1, -1, true, s, launches,
-                                         reinterpret_cast<uint64_t *>(w.bit)));
-        return;
-    }
-    KC_CK(g, launch_traverse(gv, w, bit, s, launches, fast_traversal(g)));
-}
-
 // Whether waves run the one-walker kernels with arrows drawn ahead (k1_solo.cu)
 // in place of the handle's walker: always for LANE, and under AUTO on
 // long-diameter graphs, where 32 walkers of a tree mostly wait for one another
@@ -679,7 +660,7 @@ bool run_wave_pipelined(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool reje
             std::array<cudaEvent_t, 3> e3 = {event(), event(), event()};
             KC_CK(g, cudaEventRecord(e3[0], s2));
             int nl = 0;
-            traverse_for_f(g, gv, sv, p.bit, md, s2, &nl);
+            KC_CK(g, launch_traverse(gv, sv, p.bit, s2, &nl, fast_traversal(g)));
             g->t_traverse.launches += nl;
             KC_CK(g, cudaEventRecord(e3[1], s2));
             if (p.bit) g->t_ttf.launches += eval_ttf_bit(g, gv, p, sv, wdone, spare, s2);
@@ -851,10 +832,8 @@ bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
         {
             Phase ph(g, g->t_traverse);
             int nl = 0;
-            if (canonical)
-                KC_CK(g, launch_traverse(gv, s, p.bit, g->stream, &nl, kTravCanonical));
-            else
-                traverse_for_f(g, gv, s, p.bit, (int64_t)hdr[1], g->stream, &nl);
+            KC_CK(g, launch_traverse(gv, s, p.bit, g->stream, &nl,
+                                     canonical ? kTravCanonical : fast_traversal(g)));
             ph.done(nl);
         }
         {
@@ -1638,7 +1617,7 @@ void run_wave_reject(kc_graph *g, Plan &p, int64_t B, int64_t sid0) {
         {
             Phase ph(g, g->t_traverse);
             int nl = 0;
-            traverse_for_f(g, gv, sv, p.bit, (int64_t)hdr[1], g->stream, &nl);
+            KC_CK(g, launch_traverse(gv, sv, p.bit, g->stream, &nl, fast_traversal(g)));
             ph.done(nl);
         }
         {
@@ -2035,7 +2014,7 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
                     sw.steps = w.steps + sub;
                     sw.f = w.f + sub;
                     int nl = 0;
-                    traverse_for_f(g, v, sw, p.bit, (int64_t)hdr[1], s0, &nl);
+                    KC_CK(g, launch_traverse(v, sw, p.bit, s0, &nl, fast_traversal(g)));
                     if (p.bit) KC_CK(g, launch_ttf_bit(v, sw, s0));
                     else KC_CK(g, launch_ttf_scan(v, sw, s0));
                     g->t_traverse.launches += nl;

@@ -518,21 +518,18 @@ cudaError_t launch_wilson_warp_reject(const GraphView &g, WaveView w, uint64_t s
 enum : int { kTravCanonical = 0, kTravChunked = 1, kTravLeafUp = 2 };
 cudaError_t launch_traverse(const GraphView &g, WaveView w, bool want_preorder, cudaStream_t s,
                             int *launches = nullptr, int mode = kTravCanonical);
-// Trees by their parent arrays: parent of v in tree t is par[(row n + v) stride], row =
-// slot[t], map[t] or t.
+// Trees by their parent arrays: parent of v in tree t is par[(slot ? slot[t] : t) n + v].
 struct ParTrees {
     const int32_t *par = nullptr;
     const int64_t *slot = nullptr;
-    const int32_t *map = nullptr;
-    int stride = 1;
 };
 // Order-free traversal (k2_parents.cu): w.size, w.vol and w.din (by_id: the DFN with
 // children in ascending id, else some valid one), w.aux the preorder if wanted;
-// scratch: [B][n] words (w.word if null).  (eu, ev): an edge that the trees may hold
-// and the graph does not (eu < 0: none), needed with by_id.  w.B at most 65535.
+// w.word is scratch.  (eu, ev): an edge that the trees may hold and the graph does
+// not (eu < 0: none), needed with by_id.  w.B at most 65535.
 cudaError_t launch_traverse_parents(const GraphView &g, WaveView w, ParTrees trees, bool by_id,
                                     int32_t eu, int32_t ev, bool want_preorder, cudaStream_t s,
-                                    int *launches = nullptr, uint64_t *scratch = nullptr);
+                                    int *launches = nullptr);
 // depths of the trees into w.din; w.word is scratch
 cudaError_t launch_depths_parents(const GraphView &g, WaveView w, ParTrees trees,
                                   cudaStream_t s);
