@@ -222,20 +222,19 @@ __global__ void __launch_bounds__(kThreads,
             for (int j = 0; j < kHold; ++j) {
                 const uint32_t i = tid + j * kThreads;
                 if (i >= active) break;
-                uint32_t x = list[i], w = vx[x];
-                if (w & kOnCycle) {  // its piece of the cycle
-                    uint32_t at = atomicAdd(&s_count[round & 1], len[j]);
-                    do {
-                        fresh[at++] = (uint16_t)x;
-                        x = w & kTarget;
-                        w = vx[x];
-                    } while (!(w & kActive));
+                uint32_t x = list[i];
+                if (vx[x] & kOnCycle) {  // its piece of the cycle
+                    const uint32_t at = atomicAdd(&s_count[round & 1], len[j]);
+                    for (uint32_t k = 0; k < len[j]; ++k) {
+                        fresh[at + k] = (uint16_t)x;
+                        x = vx[x] & kTarget;
+                    }
                 } else if (next[x] == 0xFFFFu) {  // its piece of a path to the root
-                    do {
+                    for (uint32_t k = 0; k < len[j]; ++k) {
+                        const uint32_t w = vx[x];
                         vx[x] = w | kSettled;
                         x = w & kTarget;
-                        w = vx[x];
-                    } while (w < kSettled);
+                    }
                 }
             }
         } else {
