@@ -38,6 +38,7 @@ struct Nbrs {
     __device__ __forceinline__ int32_t pick(uint32_t k, const GraphView &g) const {
         return nbr_of<false>(r, k, g.col);
     }
+    __device__ __forceinline__ uint32_t degree() const { return (uint32_t)r.deg; }
 };
 template <>
 struct Nbrs<true> {
@@ -46,6 +47,9 @@ struct Nbrs<true> {
     __device__ __forceinline__ int32_t pick(uint32_t k, const GraphView &) const {
         const int32_t lo = (k & 1u) ? r.y : r.x, hi = (k & 1u) ? r.w : r.z;
         return (k & 2u) ? hi : lo;
+    }
+    __device__ __forceinline__ uint32_t degree() const {  // -1 past the last neighbour
+        return 1u + (r.y >= 0) + (r.z >= 0) + (r.w >= 0);
     }
 };
 
@@ -212,7 +216,7 @@ __device__ __forceinline__ void walk_trees(const GraphView &g, const WaveView &w
             uint32_t d = 0;
             if (lane < (unsigned)slots)
                 d = bounded_draw_k(keys, seed, (uint32_t)u, hi + lane, sample, kTagWalk,
-                                   (uint32_t)g.deg[u])
+                                   rc.degree())
                     << (b * (lane + 1));
             if (kOne) {
                 d = __reduce_or_sync(kFull, d);

@@ -474,12 +474,13 @@ int pop_trees(kc_graph *g, const PopTask &task, const WaveView &w, bool in_memor
 }
 
 // Words of k1_solo.cu with the arrow queues of `root`'s trees (-1: no vertex in
-// the tree).  A long-diameter graph departs a dozen times from a vertex, the
-// others once or twice: their first queues stay short.
+// the tree).  A long-diameter graph departs a dozen times from a vertex, so its
+// first queues are full (350x350 grid, 4522 trees, first queues of 4 / 8 / 14
+// arrows: initialisation and walk 376 / 362 / 350 ms); the others once or twice.
 void init_queues(kc_graph *g, const GraphView &gv, const WaveView &w, const int64_t *sids,
                  int32_t root, cudaStream_t s) {
     KC_CK(g, launch_queue_init(gv, w, g->seed, sids, root, kc_host::queue_bits(g->max_deg),
-                               g->ttf_variant == KC_TTF_BIT ? 10 : 2, s));
+                               g->ttf_variant == KC_TTF_BIT ? 32 : 2, s));
 }
 
 // Words and order of a wave before its walk, rooted at g->root.
