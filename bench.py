@@ -284,8 +284,19 @@ def timed_sampling(G, T: int, steps: int, seed: int, stream, flush) -> list:
     return step_ms
 
 
+def walk_kernel(kc, st: dict, auto: bool) -> str:
+    """The kernel that draws the trees (auto: the library chose it by the graph)."""
+    bit = st["ttf_variant"] == kc.KC_TTF_BIT
+    if st["walker"] == kc.KC_WALK_LANE or (auto and bit):
+        return "k_wilson_queue"
+    if auto:  # popped where a block's shared memory holds the tree or the root is a hub
+        return "k_pop_small" if st["n"] <= 38000 else "k_pop_rounds"
+    return {kc.KC_WALK_WARP: "k_wilson_warp",
+            kc.KC_WALK_HYBRID: "k_wilson+k_wilson_warp"}[st["walker"]]
+
+
 def phase_roofline(kc, st: dict, n: int, trees: int, steps_total: int, tot_ms: float,
-                   walker_traffic=None) -> tuple:
+                   walker_traffic=None, auto=True) -> tuple:
     """The dominant phase of the timed steps (kc_stats' CUDA-event phase timers)
     and its roofline object: algorithmic bytes per launch over the mean launch
     time, against the measured HBM copy peak; plus the whole path's fraction."""
@@ -302,8 +313,7 @@ def phase_roofline(kc, st: dict, n: int, trees: int, steps_total: int, tot_ms: f
     per_launch_bytes = alg / max(1, dom_launches)
     per_launch_s = max(dom_ms, 1e-9) / 1000.0 / max(1, dom_launches)
     achieved = per_launch_bytes / per_launch_s / 1e9
-    kernel_name = {"wilson": {kc.KC_WALK_LANE: "k_wilson", kc.KC_WALK_WARP: "k_wilson_warp",
-                              kc.KC_WALK_HYBRID: "k_wilson+k_wilson_warp"}[st["walker"]],
+    kernel_name = {"wilson": walk_kernel(kc, st, auto),
                    "traverse": "traversal passes",
                    "ttf_bit": "k_ttf_bit", "ttf_scan": "k_ttf_scan"}[dom]
     traffic = None
@@ -369,7 +379,6 @@ def other_workload_leg(args, kc, stream, flush, name: str, T: int, steps: int, w
     g = S.workload(name)
     cfg = kc.kc_config_default()
     cfg.keep_trees = 0
-    cfg.autotune = 1  # the first warm-up call times both walkers and keeps the faster
     G = kc.KemenyGraph.from_graph(g, cfg, stream=stream.cuda_stream)
     G.reserve(T * (warmup + steps))
     for _ in range(warmup):
@@ -390,10 +399,7 @@ def other_workload_leg(args, kc, stream, flush, name: str, T: int, steps: int, w
            "ms_per_step": tot_ms / steps, "roofline": roof, "phase_ms": phase_ms,
            "steps_per_tree": steps_total / (T * steps),
            "ttf": "BIT" if st["ttf_variant"] == kc.KC_TTF_BIT else "SCAN",
-           "walker": WALKER_NAMES[st["walker"]], "autotune_ms": st["tune_ms"]}
-    # time to eps with the walker the autotuner chose (no tuning inside the timing)
-    cfg.autotune = 0
-    cfg.walker = st["walker"]
+           "walker": walk_kernel(kc, st, True)}
     out["time_to_eps"] = time_to_eps(kc, g, cfg, args.eps, delta, 1024, stream, name)
     return out
 
@@ -718,11 +724,10 @@ def serve_leg(args, kc):
 
 # DRAM bytes per Wilson departure of the walkers on road-shaped grids, from ncu
 # captures (dram__bytes_read.sum + dram__bytes_write.sum) on the 300x300
-# perturbed grid with 1000 trees in flight (profiles/); a full-size launch runs
-# for seconds, too long to capture, so its traffic is this figure times its
-# departures.  k_wilson_warp: 10.213 GB, k_wilson: 4.648 GB, each for the
-# same 1,133,364,358 departures.
-WALKER_GRID_DRAM_BYTES_PER_STEP = {"warp": 10.213e9 / 1133364358, "lane": 4.648e9 / 1133364358}
+# perturbed grid with 1000 trees in flight (profiles/); a full-size launch is too
+# long to capture, so its traffic is this figure times its departures.
+# k_wilson_warp: 10.213 GB for 1,133,364,358 departures.
+WALKER_GRID_DRAM_BYTES_PER_STEP = {"k_wilson_warp": 10.213e9 / 1133364358}
 
 
 def main():
@@ -819,7 +824,7 @@ def main():
         pcfg = kc.kc_config_default()
         for f, _ in kc.kc_config._fields_:
             setattr(pcfg, f, getattr(cfg, f))
-        pcfg.walker = kc.KC_WALK_WARP  # a few hundred trees: 32 walkers each finish sooner
+        pcfg.walker = kc.KC_WALK_AUTO
         P = kc.KemenyGraph.from_graph(g, pcfg, stream=stream.cuda_stream)
         P.sample(args.seed, args.reject_probe)
         probe_steps = P.samples()["steps"]
@@ -860,10 +865,11 @@ def main():
     samples = G.samples(pool0, st["pool_trees"] - pool0)
     steps_total = int(samples["steps"].sum())
     trees_timed = T * args.steps
-    traffic_per_step = (WALKER_GRID_DRAM_BYTES_PER_STEP.get(WALKER_NAMES[st["walker"]])
+    auto = args.walker == "auto"
+    traffic_per_step = (WALKER_GRID_DRAM_BYTES_PER_STEP.get(walk_kernel(kc, st, auto))
                         if args.workload.startswith("grid") else None)
     dom, roof, phase_ms = phase_roofline(kc, st, n, trees_timed, steps_total, tot_ms,
-                                         traffic_per_step)
+                                         traffic_per_step, auto)
     roof["traffic_basis"] = (None if roof["traffic"] is None else
                              "ncu dram bytes per departure on grid300x300 (1000 trees) x "
                              "departures")
@@ -881,6 +887,7 @@ def main():
                          f"{st['workspace_bytes'] / 1e9:.1f} GB",
                    "ttf": "BIT" if st["ttf_variant"] == kc.KC_TTF_BIT else "SCAN",
                    "walker": WALKER_NAMES[st["walker"]],
+                   "walk_kernel": walk_kernel(kc, st, auto),
                    "trees_in_flight": st["trees_in_flight"]},
         "roofline": roof,
         "phase_ms": phase_ms,

@@ -84,8 +84,13 @@ enum { KC_UPDATE_BSM = 0,      /* Algorithm 2 */
        KC_UPDATE_ISM = 1 };    /* Algorithm 3 */
 
 /* Wilson walkers per tree.  All give identical trees and step counts. */
-enum { KC_WALK_AUTO = 0,       /* WARP; LANE under rejection by walk length on a graph
-                                  whose TTF variant is BIT (long diameter)                */
+enum { KC_WALK_AUTO = 0,       /* by the graph.  Long diameter (the TTF variant is BIT): one
+                                  walker per tree with its arrows drawn ahead.  SCAN:
+                                  cycle popping, a block per tree in shared memory up to
+                                  38000 vertices, or in device memory where the root is a
+                                  hub (16 x 2m / deg(root) <= n); else 32 walkers.
+                                  Reported as WARP, or LANE under rejection by walk
+                                  length on a BIT graph                                */
        KC_WALK_LANE = 1,       /* one sequential walker per tree (one lane)              */
        KC_WALK_WARP = 2,       /* 32 concurrent walkers per tree popping cycles in any order */
        KC_WALK_HYBRID = 3 };   /* LANE for a prefix of the start order, then WARP for the
@@ -134,7 +139,9 @@ typedef struct {
     int64_t step_cap;           /* cap on Wilson departures (0: max(2^22, 1024 n)), per
                                    tree for the one-walker kernel and per walker for
                                    the 32-walker kernel (a tree may then take up to
-                                   32 x step_cap); exceeding it is KC_ERR_STEP_LIMIT */
+                                   32 x step_cap); exceeding it is KC_ERR_STEP_LIMIT.
+                                   Under AUTO a wave past the cap is drawn again by
+                                   the 32-walker kernel, whose cap then decides     */
     double mem_fraction;        /* share of free device memory for workspaces (0: 0.8) */
     int64_t sample_id_base;     /* first sample id of the pool (0); ranks of a
                                    multi-GPU run use disjoint bases, ids < 2^32   */
@@ -163,8 +170,8 @@ typedef struct {
                                    accepts enough trees in one go; later waves use the
                                    share seen so far.  0: 8/9                       */
     int32_t ttf_segments;       /* BIT evaluation of f (Algorithm 1) split into preorder
-                                   segments, each replayed by its own warp from the
-                                   DFS state rebuilt at its first position (same f,
+                                   segments, each swept by its own warp with its own
+                                   Fenwick array and joined by interval sums (same f,
                                    exactly).  0: automatic -- the chunks evaluated
                                    after their wave's walk has ended, up to 16
                                    segments a tree and about 32 segment warps an SM,
@@ -241,8 +248,8 @@ kc_status kc_reserve(kc_graph *g, int64_t n_trees);
 /*
  * Batched multi-graph sampling (no counterpart in the paper): the same result
  * as kc_sample(graphs[i], seeds[i], n_trees[i]) for every i, but the walks of
- * all graphs run in one 32-walker launch per round (one warp per tree, graphs
- * of uneven size mixed), which fills the GPU when each graph alone has too few
+ * all graphs that use one kernel run in one launch of it per round (graphs of
+ * uneven size mixed), which fills the GPU when each graph alone has too few
  * trees.  All work runs on graphs[0]'s stream.  The handles must be distinct
  * and on one device.  Errors: as kc_sample; on error no pool changes.
  */
@@ -409,7 +416,9 @@ kc_status kc_estimate_from_sums(const kc_pool_sums *sums, int64_t twom, int32_t 
  * afford the driver allocator's unbounded latency and implicit
  * synchronisation.  This call allocates nothing.  Its only working memory is a
  * fixed array of 8 Mi walker words (64 MiB) compiled into the library, which
- * every GPU that loads the library holds until the process exits.
+ * every GPU that loads the library holds until the process exits, and d_parent
+ * itself: trees of up to 56000 vertices are drawn in shared memory with their rows
+ * of d_parent as scratch.
  *
  * It draws n_trees uniform spanning trees rooted at `root` with sample ids
  * first_sample_id .. first_sample_id + n_trees - 1 under `seed`, using the

@@ -36,7 +36,7 @@ struct Nbrs {
     VRec r;
     __device__ __forceinline__ void load(const GraphView &g, int32_t v) { r = load_rec(g.rec + v); }
     __device__ __forceinline__ int32_t pick(uint32_t k, const GraphView &g) const {
-        return nbr_of<false>(r, k, g.col);
+        return nbr_of(r, k, g.col);
     }
     __device__ __forceinline__ uint32_t degree() const { return (uint32_t)r.deg; }
 };
@@ -166,7 +166,7 @@ __device__ __forceinline__ int32_t commit_path(unsigned gm, uint64_t *word, int3
 // memory (L1 serves 95%); the 32 lockstep walkers of one tree (k_wilson_warp) take
 // about 650 cycles, a walker per lane (k_wilson) about 1100.  Walk of 500 trees of a
 // 40000-vertex grid: 348 (k_wilson_warp) -> 140 ms; of 4522 trees of the 350x350 grid
-// under a cap of 13 n departures: 1640 (k_wilson) -> 345 ms.  The word that held the
+// under a cap of 13 n departures: 1640 (k_wilson) -> 350 ms.  The word that held the
 // next target itself, with the queue behind it, made the load chain shorter and the
 // kernel slower: 52 instructions, 250 cycles.
 template <int kGroup, bool kDeg4, bool kReject>

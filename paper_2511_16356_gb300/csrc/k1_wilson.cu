@@ -1,7 +1,9 @@
 // Wilson's loop-erased-walk sampler (Sec. 2.2; Algorithm 1, "wilson(G, r)").
 //
-// Two walkers.  k_wilson_warp (the default) runs 32 concurrent walkers of one
-// tree per warp (described below).  k_wilson runs one tree per lane as a flat
+// Two walkers, for the trees that k1_solo.cu and k4_pop.cu do not take: large graphs of
+// low diameter without a hub, the explicit WARP and HYBRID choices, neighbour indices
+// too wide for a queue, and waves past a limit of those kernels.  k_wilson_warp runs
+// 32 concurrent walkers of one tree per warp (described below).  k_wilson runs one tree per lane as a flat
 // state machine (SEEK a start vertex outside the tree, WALK, count the
 // loop-erased path, commit it); every iteration does its phase's arithmetic,
 // then one gather, then the phase's resolution, so lanes in different phases

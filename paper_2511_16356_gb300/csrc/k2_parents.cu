@@ -22,9 +22,10 @@
 // is the rate of random 32-byte sectors.
 //
 // Measured (GB300, 100000-vertex power-law graph, 20 neighbours a vertex, pool of
-// 1000 trees, 4 ISM operations of about 165 trees each): 743 -> 115 ms with
-// the cut counts of k6_update.cu; the warp-per-tree passes it replaces took 360 of
-// them (breadth-first order 176, child scan 25, top-down 56, sizes 80, siblings 21).
+// 1000 trees, 4 ISM operations of about 165 trees each): 743 -> 115 ms with the cut
+// counts of k6_update.cu (about 60 with the later steps elsewhere); the warp-per-tree
+// passes it replaces took 360 of the 743 (breadth-first order 176, child scan 25,
+// top-down 56, sizes 80, siblings 21).
 #include <algorithm>
 
 #include <cuda/atomic>

@@ -23,7 +23,7 @@
 // its images are the vertices on its cycles (contracted_round); each of those lists
 // its own piece of the cycle.  A round of some 50 active vertices then costs its
 // longest piece where the leaders' loops went around several times: 2000 trees of a
-// random graph of 2000 vertices (kc_wilson_noalloc) 2.62 -> 2.23 ms.
+// random graph of 2000 vertices (kc_wilson_noalloc) 2.62 -> 2.23 ms, 1.4 by now.
 //
 // k_pop_small keeps the tree in shared memory: 14 bytes a vertex.  Larger trees
 // stay in memory: the first arrows (k_first_arrows) and the cycles of the first map
@@ -33,9 +33,10 @@
 // rate of random sectors, about ten a vertex with the traversal.
 //
 // Measured (GB300, power-law graphs of mean degree 17, against 32 walkers a tree
-// and their traversal): 2 million vertices, 384 trees 830 -> 160 ms (rounds 43,
+// and their traversal): 2 million vertices, 384 trees 830 -> 140 ms (rounds 43,
 // first cycles 16, first arrows 5; traversal 65, tau0 scan 10); 10000 vertices in
-// shared memory, 500 trees 5.26 -> 1.27 ms.
+// shared memory, 500 trees 5.3 -> 0.9 ms.  Random graph of 2000 vertices, 2000 trees:
+// 3.8 -> 1.4 ms.
 #include <algorithm>
 #include <atomic>
 
@@ -167,7 +168,7 @@ __global__ void __launch_bounds__(kThreads,
         const VRec r = load_rec(rec + v);
         const uint32_t k = bounded_draw_k(task.keys, task.seed, v, count, sample, kTagWalk,
                                           (uint32_t)r.deg);
-        return (uint32_t)nbr_of<false>(r, k, g.col);
+        return (uint32_t)nbr_of(r, k, g.col);
     };
     for (uint32_t v = tid; v < n; v += kThreads) {
         uint32_t x = root | kSettled;
@@ -370,7 +371,7 @@ __device__ __forceinline__ uint64_t large_arrow(const PopTask &task, uint32_t sa
     const VRec r = load_rec(task.g.rec + v);
     const uint32_t k = bounded_draw_k(task.keys, task.seed, v, count, sample, kTagWalk,
                                       (uint32_t)r.deg);
-    return (uint32_t)nbr_of<false>(r, k, task.g.col);
+    return (uint32_t)nbr_of(r, k, task.g.col);
 }
 
 constexpr int kFirstTrees = 4;  // trees for which a thread keeps a vertex's record
@@ -388,7 +389,7 @@ __global__ void __launch_bounds__(256) k_first_arrows(PopTask task, int64_t B, u
         if (v != task.root && v != task.fixed) {
             const uint32_t k = bounded_draw_k(task.keys, task.seed, (uint32_t)v, 0,
                                               (uint32_t)task.sids[t], kTagWalk, (uint32_t)r.deg);
-            x = (uint32_t)nbr_of<false>(r, k, task.g.col);
+            x = (uint32_t)nbr_of(r, k, task.g.col);
         }
         words[t * n + v] = x;
     }

@@ -39,7 +39,7 @@ std::mutex g_scratch_mu;
 // Trees of up to kPopTreesMax vertices are popped in shared memory (k4_pop.cu), a
 // block each; this kernel walks the larger ones, and (redo) those that the pops
 // left: past the step cap, where the outputs are the walk's, or past their count
-// fields.  2000 trees of a sparse random graph of 2000 vertices: 12.3 -> 2.4 ms.
+// fields.  2000 trees of a sparse random graph of 2000 vertices: 12.5 -> 1.4 ms.
 //
 // One lane per tree, straight from the CSR (no walk records): the same
 // arrows (vertex u leaves along neighbour bounded(seed, u, k, sample, WALK,

@@ -164,19 +164,17 @@ __device__ __forceinline__ VRec load_rec(const VRec *p) {
     return r;
 }
 
-// neighbour number k of a record by a select, the column array from the inlined
-// ones on; kDeg4: the graph's degrees are at most 4
-template <bool kDeg4>
+// neighbour number k of a record by a select, the column array past the inlined ones
 __device__ __forceinline__ int32_t nbr_of(const VRec &r, uint32_t k,
                                           const int32_t *__restrict__ col) {
-    if (!kDeg4 && k >= (uint32_t)kInline) {
+    if (k >= (uint32_t)kInline) {
         const uint64_t off = (uint64_t)r.off_lo | ((uint64_t)r.off_hi << 32);
         return col[off + k];
     }
     const int32_t lo = (k & 1u) ? r.nbr[1] : r.nbr[0];
     const int32_t hi = (k & 1u) ? r.nbr[3] : r.nbr[2];
     const int32_t x = (k & 2u) ? hi : lo;
-    return !kDeg4 && (k & 4u) ? r.nbr[4] : x;
+    return (k & 4u) ? r.nbr[4] : x;
 }
 
 // ---------------------------------------------------------------------------
@@ -538,8 +536,8 @@ cudaError_t launch_ttf_scan_parents(const GraphView &g, WaveView w, ParTrees tre
                                     cudaStream_t s);
 cudaError_t launch_ttf_scan(const GraphView &g, WaveView w, cudaStream_t s);
 cudaError_t launch_ttf_bit(const GraphView &g, WaveView w, cudaStream_t s);
-// f of the sub-wave's trees from segments that each start from the DFS state
-// rebuilt at their first position; zeroes the segments' Fenwick arrays first and
+// f of the sub-wave's trees from segments, each with its own points and with the
+// subtrees that reach into it; zeroes the segments' Fenwick arrays first and
 // adds into w.f (zeroed by the caller).  segs: device table of nseg entries.
 cudaError_t launch_ttf_bit_seg(const GraphView &g, WaveView w, const TtfSeg *segs, int64_t nseg,
                                cudaStream_t s);
