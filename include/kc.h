@@ -433,7 +433,7 @@ kc_status kc_estimate_from_sums(const kc_pool_sums *sums, int64_t twom, int32_t 
  *  stream            cudaStream_t to run on (NULL: legacy default stream)
  * Work is enqueued on `stream`; the call returns without synchronising.
  * Requires n * n_trees <= 8 Mi, else KC_ERR_SCRATCH_LIMIT.  The first call on
- * a device looks up the array's device address (cudaGetSymbolAddress) with
+ * a device looks up the array's device address and sets up the kernels with
  * that device current; make that first call before any stream capture.
  * Every call reuses the same array and clears the part it needs; calls that
  * overlap on the GPU (several streams or host threads) race on it and must be

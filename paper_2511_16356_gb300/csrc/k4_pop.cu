@@ -560,12 +560,9 @@ static_assert(kc_host::pop_small_bytes(kc_host::kPopSmallMax) <= kMostDynamic &&
                   kc_host::pop_trees_bytes(kc_host::kPopTreesMax) <= kMostDynamic,
               "the largest trees fit a block");
 
+// The kernel's shared memory is raised once per device, on its first call there.
 template <int kThreads, bool kMulti, int kKind>
-cudaError_t launch_small(const PopTask &one, const PopTask *tasks, const int2 *entry,
-                         int64_t blocks, int64_t max_n, cudaStream_t s) {
-    const size_t bytes =
-        kKind == kFused ? kc_host::pop_small_bytes(max_n) : kc_host::pop_trees_bytes(max_n);
-    // raised once per device, on the first call (a later one may be captured)
+cudaError_t raise_shared() {
     static std::atomic<uint64_t> raised{0};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -576,6 +573,16 @@ cudaError_t launch_small(const PopTask &one, const PopTask *tasks, const int2 *e
         if (e != cudaSuccess) return e;
         if (dev < 64) raised.fetch_or((uint64_t)1 << dev);
     }
+    return cudaSuccess;
+}
+
+template <int kThreads, bool kMulti, int kKind>
+cudaError_t launch_small(const PopTask &one, const PopTask *tasks, const int2 *entry,
+                         int64_t blocks, int64_t max_n, cudaStream_t s) {
+    const size_t bytes =
+        kKind == kFused ? kc_host::pop_small_bytes(max_n) : kc_host::pop_trees_bytes(max_n);
+    const cudaError_t e = raise_shared<kThreads, kMulti, kKind>();
+    if (e != cudaSuccess) return e;
     k_pop_small<kThreads, kMulti, kKind><<<(unsigned)blocks, kThreads, bytes, s>>>(one, tasks,
                                                                                    entry);
     return cudaGetLastError();
@@ -602,6 +609,14 @@ cudaError_t launch_pop_small(const PopTask &task, int64_t B, cudaStream_t s) {
 cudaError_t launch_pop_trees(const PopTask &task, int64_t B, cudaStream_t s) {
     return task.g.rec ? launch_small_any<false, kTrees>(task, nullptr, nullptr, B, task.g.n, s)
                       : launch_small_any<false, kTreesCsr>(task, nullptr, nullptr, B, task.g.n, s);
+}
+
+cudaError_t prepare_pop_trees_csr() {
+    cudaError_t e = raise_shared<128, false, kTreesCsr>();
+    if (e == cudaSuccess) e = raise_shared<256, false, kTreesCsr>();
+    if (e == cudaSuccess) e = raise_shared<512, false, kTreesCsr>();
+    if (e == cudaSuccess) e = raise_shared<1024, false, kTreesCsr>();
+    return e;
 }
 
 cudaError_t launch_pop_small_multi(const PopTask *tasks, const int2 *entry, int64_t count,

@@ -123,7 +123,8 @@ extern "C" kc_status kc_wilson_noalloc(int64_t n, const int64_t *d_row_off, cons
         std::lock_guard<std::mutex> lock(g_scratch_mu);
         if (!g_scratch_addr[dev]) {
             void *p = nullptr;
-            const cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_words);
+            cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_words);
+            if (e == cudaSuccess) e = prepare_pop_trees_csr();
             if (e != cudaSuccess || !p) {
                 (void)cudaGetLastError();
                 return KC_ERR_CUDA;

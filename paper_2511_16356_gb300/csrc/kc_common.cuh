@@ -485,6 +485,9 @@ cudaError_t launch_pop_large(const PopTask &task, int64_t B, uint64_t *words, in
 // (task.g.rec null) the arrows come from the CSR arrays and a tree past the step cap
 // or the pop counts gets steps = kPopRedo instead of an error.
 cudaError_t launch_pop_trees(const PopTask &task, int64_t B, cudaStream_t s);
+// sets up those kernels without records on the current device, so that a later call
+// of any size can be captured
+cudaError_t prepare_pop_trees_csr();
 // entries (task, tree) of a device table of tasks; max_n: their largest n
 cudaError_t launch_pop_small_multi(const PopTask *tasks, const int2 *entry, int64_t count,
                                    int64_t max_n, cudaStream_t s);

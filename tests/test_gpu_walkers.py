@@ -169,3 +169,37 @@ def test_trees_without_allocation_match_oracle(n, trees, cap):
     assert np.all(got[over] == cap + 1)
     for k in np.flatnonzero(~over)[:3]:
         assert np.array_equal(par[k].cpu().numpy(), O.tree(g, t0, 71, 4 + int(k)).parent)
+
+
+@pytest.mark.parametrize("n", [60, 3000, 6000, 12000])
+def test_noalloc_is_captured_after_a_first_call_of_another_size(n):
+    """A call of any size can be captured once one call was made on the device: the
+    replay gives the trees that a plain call gives."""
+    torch = pytest.importorskip("torch")
+    trees = 6
+
+    def buffers(g):
+        return (torch.from_numpy(g.row_off).cuda(), torch.from_numpy(g.col).cuda(),
+                torch.zeros((trees, g.n), dtype=torch.int32, device="cuda"),
+                torch.zeros(trees, dtype=torch.int64, device="cuda"),
+                torch.zeros(1, dtype=torch.int32, device="cuda"))
+
+    def call(g, b, stream):
+        assert kc.load().kc_wilson_noalloc(g.n, b[0].data_ptr(), b[1].data_ptr(), 0, 5, 9, trees,
+                                           0, b[2].data_ptr(), b[3].data_ptr(), b[4].data_ptr(),
+                                           stream.cuda_stream) == kc.KC_OK
+
+    first = S.complete(5)
+    call(first, buffers(first), torch.cuda.current_stream())
+    g = S.complete_bipartite(25, n - 25)
+    b, plain = buffers(g), buffers(g)
+    torch.cuda.synchronize()
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=side):
+        call(g, b, side)
+    graph.replay()
+    torch.cuda.synchronize()
+    call(g, plain, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(b[2:], plain[2:]))
+    assert int(b[3].min()) >= n - 1
