@@ -27,12 +27,6 @@ __global__ void k_pool_parents(const uint64_t *word, int64_t B, int64_t n, int32
     if (k < B * n) dst[k] = w_next(word[k]);
 }
 
-__global__ void k_words_from_parents(int64_t n, int64_t B, const int32_t *parents,
-                                     uint64_t *word) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < B * n) word[k] = w_make(parents[k], 0, false);
-}
-
 struct I128 {
     long long hi;
     unsigned long long lo;
@@ -124,13 +118,6 @@ cudaError_t launch_pool_reduce(const int64_t *f, const double *w, int64_t count,
                                void *scratch, cudaStream_t s) {
     k_pool_reduce<<<1, 1024, 0, s>>>(f, w, count, 1.0 / (double)twom,
                                      reinterpret_cast<PoolSums *>(scratch));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_words_from_parents(int64_t n, int64_t B, const int32_t *parents,
-                                      uint64_t *word, cudaStream_t s) {
-    const int64_t tot = B * n;
-    k_words_from_parents<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(n, B, parents, word);
     return cudaGetLastError();
 }
 

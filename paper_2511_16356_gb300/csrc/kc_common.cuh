@@ -549,8 +549,6 @@ cudaError_t launch_pool_append(WaveView w, int64_t first, int64_t *pool_f, doubl
                                int32_t *pool_parents, int64_t n, cudaStream_t s);
 cudaError_t launch_pool_reduce(const int64_t *f, const double *w, int64_t count, int64_t twom,
                                void *scratch, cudaStream_t s);
-cudaError_t launch_words_from_parents(int64_t n, int64_t B, const int32_t *parents,
-                                      uint64_t *word, cudaStream_t s);
 
 // Sample maintenance (k6_update.cu) and effective resistance (k8_resistance.cu).
 // the edge (u, v) in the tree of every word array, u -> v; cleared: the other words
