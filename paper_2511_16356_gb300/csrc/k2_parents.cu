@@ -15,10 +15,10 @@
 // those took 89 ms for the 4500 trees of a 350x350 grid where the ordered passes
 // take 53, and slowed the walk by a tenth.
 //
-// Word of a vertex: until it reports, unreported children (high half) and sizes
-// reported (low half); then preorder offset (high half) and the ancestor it is
-// relative to (low half).  The second pair is read and written whole and holds at
-// any time, so jumps need no rounds and no second buffer.  What bounds the passes
+// Word of a vertex (kc_host_par.h): until it reports, unreported children and sizes
+// reported; then preorder offset and the ancestor it is relative to.  The second pair
+// is read and written whole and holds at any time, so jumps need no rounds and no
+// second buffer.  What bounds the passes
 // is the rate of random 32-byte sectors.
 //
 // Measured (GB300, 100000-vertex power-law graph, 20 neighbours a vertex, pool of
@@ -31,6 +31,7 @@
 #include <cuda/atomic>
 
 #include "kc_common.cuh"
+#include "kc_host_par.h"
 
 namespace kc {
 
@@ -53,7 +54,8 @@ __global__ void k_par_count(int64_t n, WaveView w, ParTrees trees) {
     }
 }
 
-// A vertex with children never has a zero word, so only leaves start threads.
+// Only leaves start threads; a vertex's thread may come to it at any time, also after
+// its tree is finished.
 __global__ void k_par_up(GraphView g, WaveView w, ParTrees trees) {
     const int64_t n = g.n;
     const int64_t t = blockIdx.y;
@@ -63,7 +65,7 @@ __global__ void k_par_up(GraphView g, WaveView w, ParTrees trees) {
     int64_t *vol = w.vol + t * n;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
-        if (*(volatile unsigned long long *)(word + v) != 0ull) continue;  // has children
+        if (!kc_host::par_is_leaf(*(volatile unsigned long long *)(word + v), v, g.root)) continue;
         int32_t x = (int32_t)v, sx = 1;
         int64_t vx = (int64_t)g.deg[v];
         for (int64_t hop = 0;; ++hop) {
@@ -71,7 +73,7 @@ __global__ void k_par_up(GraphView g, WaveView w, ParTrees trees) {
             size[x] = sx;
             vol[x] = vx;
             if (p < 0 || p >= n || hop > n) {
-                word[x] = (uint64_t)(uint32_t)x;
+                word[x] = kc_host::par_at(0, x);
                 if (p >= n || hop > n || sx != n) atomicOr(w.err, kErrBadTree);
                 break;
             }
@@ -79,12 +81,11 @@ __global__ void k_par_up(GraphView g, WaveView w, ParTrees trees) {
             cuda::atomic_ref<unsigned long long, cuda::thread_scope_device> acc(
                 *reinterpret_cast<unsigned long long *>(word + p));
             const unsigned long long old =
-                acc.fetch_add((unsigned long long)(uint32_t)sx - (1ull << 32),
-                              cuda::memory_order_release);
-            word[x] = ((old & 0xFFFFFFFFull) + 1ull) << 32 | (uint32_t)p;
-            if ((old >> 32) != 1ull) break;  // siblings still to report
+                acc.fetch_add(kc_host::par_report(sx), cuda::memory_order_release);
+            word[x] = kc_host::par_at((uint32_t)kc_host::par_sizes(old) + 1u, p);
+            if (!kc_host::par_was_last(old)) break;  // siblings still to report
             cuda::atomic_thread_fence(cuda::memory_order_acquire, cuda::thread_scope_device);
-            sx = 1 + (int32_t)(uint32_t)old + sx;
+            sx = 1 + kc_host::par_sizes(old) + sx;
             vx = (int64_t)g.deg[p] + *(volatile long long *)(vol + p);
             x = p;
         }

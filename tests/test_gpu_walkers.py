@@ -203,3 +203,30 @@ def test_noalloc_is_captured_after_a_first_call_of_another_size(n):
     torch.cuda.synchronize()
     assert all(torch.equal(x, y) for x, y in zip(b[2:], plain[2:]))
     assert int(b[3].min()) >= n - 1
+
+
+def _hubs_first(n):
+    """Vertex 0 joined to the next ones (up to 63), the others spread under those: a root 0
+    whose neighbours in id are internal."""
+    hubs = max(1, min(63, (n - 1) // 2))
+    u = np.arange(1, n)
+    return S.csr_from_edges(n, u, np.where(u <= hubs, 0, 1 + (u - 1 - hubs) % hubs))
+
+
+@pytest.mark.parametrize("n", [2, 3, 128, 129, 3000, 20000])
+def test_root_zero_is_never_taken_for_a_leaf(n):
+    """The path tree, popped trees and single-tree reads of a graph rooted at vertex 0."""
+    g = _hubs_first(n)
+    t0 = O.tau0(g, 0)
+    cfg = _cfg(keep_trees=1, root=0)
+    with kc.KemenyGraph.from_graph(g, cfg) as G:
+        tau = G.tau0()
+        assert np.array_equal(tau["in0"], t0.in0) and np.array_equal(tau["out0"], t0.out0)
+        G.sample(29, 40)
+        f_ref, st_ref = O.sample_batch(g, t0, 29, 0, 40)
+        got = G.samples()
+        assert np.array_equal(got["f"], f_ref) and np.array_equal(got["steps"], st_ref)
+        for k in range(0, 40, 13):
+            tr, ref = G.tree(k), O.tree(g, t0, 29, k)
+            for key in ("parent", "depth", "din", "dout", "vol"):
+                assert np.array_equal(tr[key], getattr(ref, key)), key
