@@ -258,12 +258,12 @@ __global__ void __launch_bounds__(kThreads,
             nx[a] &= ~(kActive | kOnCycle);
         }
         if (tid == 0) s_count[(round + 1) & 1] = 0;
-        if (found == 0) break;
         pops += found;
-        if (pops + (int64_t)n - task.placed > task.step_cap) {
+        if (pops + (int64_t)n - task.placed > task.step_cap) {  // also of a first map that is a tree
             end = kErrStepLimit;
             break;
         }
+        if (found == 0) break;
         __syncthreads();
         bool full = false;
         for (uint32_t i = tid; i < found; i += kThreads) {
@@ -458,12 +458,13 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
     int64_t pops = 0;
     int end = 0;
     if (tid < 2) s_count[tid] = 0;
-    for (int round = 0; active > 0; ++round) {
+    for (int round = 0;; ++round) {
         pops += active;
-        if (pops + n - task.placed > task.step_cap) {
+        if (pops + n - task.placed > task.step_cap) {  // also of a first map that is a tree
             end = kErrStepLimit;
             break;
         }
+        if (active == 0) break;
         __syncthreads();
         bool full = false;
         for (uint32_t i = tid; i < active; i += kThreads) {

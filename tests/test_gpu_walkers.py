@@ -230,3 +230,31 @@ def test_root_zero_is_never_taken_for_a_leaf(n):
             tr, ref = G.tree(k), O.tree(g, t0, 29, k)
             for key in ("parent", "depth", "din", "dout", "vol"):
                 assert np.array_equal(tr[key], getattr(ref, key)), key
+
+
+@pytest.mark.parametrize("n", [40, 4000, 16001])
+@pytest.mark.parametrize("cap", [5, -1, 0])
+def test_step_cap_holds_for_trees_without_a_cycle(n, cap):
+    """A star rooted at its centre pops nothing: a tree still departs n - 1 times, and
+    a cap below that (cap <= 0: n - 1 + cap) ends it."""
+    torch = pytest.importorskip("torch")
+    g, trees = S.star(n), 40
+    cap = cap if cap > 0 else n - 1 + cap
+    root = int(np.argmax(np.diff(g.row_off)))
+    ro, co = torch.from_numpy(g.row_off).cuda(), torch.from_numpy(g.col).cuda()
+    par = torch.zeros((trees, n), dtype=torch.int32, device="cuda")
+    steps = torch.zeros(trees, dtype=torch.int64, device="cuda")
+    status = torch.full((1,), 5, dtype=torch.int32, device="cuda")
+    assert kc.load().kc_wilson_noalloc(n, ro.data_ptr(), co.data_ptr(), root, 5, 0, trees, cap,
+                                       par.data_ptr(), steps.data_ptr(), status.data_ptr(),
+                                       torch.cuda.current_stream().cuda_stream) == kc.KC_OK
+    torch.cuda.synchronize()
+    assert int(status.item()) == int(cap < n - 1)
+    assert np.all(steps.cpu().numpy() == min(n - 1, cap + 1))
+    # AUTO: the 32-walker kernel decides, whose cap is per walker
+    said = []
+    for walker in (kc.KC_WALK_AUTO, kc.KC_WALK_WARP):
+        with kc.KemenyGraph.from_graph(g, _cfg(walker=walker, step_cap=cap)) as G:
+            said.append(kc.STATUS[kc.kc_sample(G.h, 3, trees, check=False)])
+    assert said[0] == said[1]
+    assert cap < n - 1 or said[0] == "KC_OK"
