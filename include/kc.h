@@ -418,7 +418,7 @@ kc_status kc_estimate_from_sums(const kc_pool_sums *sums, int64_t twom, int32_t 
  * fixed array of 8 Mi walker words (64 MiB) compiled into the library, which
  * every GPU that loads the library holds until the process exits, and d_parent
  * itself: trees of up to 56000 vertices are drawn in shared memory with their rows
- * of d_parent as scratch.
+ * of d_parent as scratch, unless there are more than 128 n of them.
  *
  * It draws n_trees uniform spanning trees rooted at `root` with sample ids
  * first_sample_id .. first_sample_id + n_trees - 1 under `seed`, using the

@@ -37,9 +37,10 @@ uint64_t *g_scratch_addr[kMaxDevices] = {};
 std::mutex g_scratch_mu;
 
 // Trees of up to kPopTreesMax vertices are popped in shared memory (k4_pop.cu), a
-// block each; this kernel walks the larger ones, and (redo) those that the pops
-// left: past the step cap, where the outputs are the walk's, or past their count
-// fields.  2000 trees of a sparse random graph of 2000 vertices: 12.5 -> 1.4 ms.
+// block each, unless a call has very many for their size (kc_host::pop_noalloc); this
+// kernel walks the others, and (redo) those that the pops left: past the step cap,
+// where the outputs are the walk's, or past their count fields.  2000 trees of a
+// sparse random graph of 2000 vertices: 12.5 -> 1.4 ms.
 //
 // One lane per tree, straight from the CSR (no walk records): the same
 // arrows (vertex u leaves along neighbour bounded(seed, u, k, sample, WALK,
@@ -139,7 +140,7 @@ extern "C" kc_status kc_wilson_noalloc(int64_t n, const int64_t *d_row_off, cons
         return KC_ERR_CUDA;
     }
     const int64_t cap = step_cap > 0 ? step_cap : std::max<int64_t>((int64_t)1 << 22, 1024 * n);
-    const bool pop = n <= kc_host::kPopTreesMax;
+    const bool pop = kc_host::pop_noalloc(n, n_trees);
     cudaError_t e;
     if (pop) {
         PopTask k{};

@@ -131,6 +131,15 @@ constexpr int64_t kPopContractMax = 38000, kPopTreesMax = 56000;
 constexpr size_t pop_trees_bytes(int64_t n) {
     return (size_t)n * (n <= kPopContractMax ? 6 : 4);
 }
+// Whether kc_wilson_noalloc pops its trees, a block each: while a block holds a tree and
+// there are at most 128 of them a vertex.  Past that a lane per tree, of few
+// departures each, fills the GPU better (GB300, ms of a lane per tree / popped, grid
+// 6x6: 14600 trees 0.41 / 0.74, 233000 trees 1.2 / 8.6; random graph of 100 vertices:
+// 10500 trees 0.34 / 0.29, 84000 trees 0.64 / 1.47; of 300: 28000 trees 1.7 / 1.2).
+constexpr int64_t kPopTreesPerVertex = 128;
+constexpr bool pop_noalloc(int64_t n, int64_t n_trees) {
+    return n <= kPopTreesMax && n_trees <= kPopTreesPerVertex * n;
+}
 // How AUTO draws the trees of a low-diameter graph (against 32 walkers a tree and
 // their traversal; GB300, ms):
 //   up to kPopSmallMax vertices in shared memory, f included (random graph of 8000

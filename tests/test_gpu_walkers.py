@@ -258,3 +258,30 @@ def test_step_cap_holds_for_trees_without_a_cycle(n, cap):
             said.append(kc.STATUS[kc.kc_sample(G.h, 3, trees, check=False)])
     assert said[0] == said[1]
     assert cap < n - 1 or said[0] == "KC_OK"
+
+
+@pytest.mark.parametrize("trees", [128 * 60, 128 * 60 + 1, 140000])
+@pytest.mark.parametrize("cap", [0, 100])
+def test_many_small_trees_without_allocation_match_oracle(trees, cap):
+    """Either side of the line between a block per tree and a lane per tree, and the largest
+    call that the scratch array takes: step counts, parents and the status."""
+    torch = pytest.importorskip("torch")
+    g = S.complete_bipartite(7, 53)
+    n, t0 = g.n, O.tau0(g)
+    if trees > (8 << 20) // n:
+        trees = (8 << 20) // n
+    ro, co = torch.from_numpy(g.row_off).cuda(), torch.from_numpy(g.col).cuda()
+    par = torch.full((trees, n), -7, dtype=torch.int32, device="cuda")
+    steps = torch.zeros(trees, dtype=torch.int64, device="cuda")
+    status = torch.full((1,), 5, dtype=torch.int32, device="cuda")
+    assert kc.load().kc_wilson_noalloc(n, ro.data_ptr(), co.data_ptr(), t0.r, 73, 2, trees, cap,
+                                       par.data_ptr(), steps.data_ptr(), status.data_ptr(),
+                                       torch.cuda.current_stream().cuda_stream) == kc.KC_OK
+    torch.cuda.synchronize()
+    _, want = O.sample_batch(g, t0, 73, 2, trees)
+    over = want > cap if cap else want < 0
+    assert int(status.item()) == int(over.any())
+    got = steps.cpu().numpy()
+    assert np.array_equal(got[~over], want[~over]) and np.all(got[over] == cap + 1)
+    for k in [*np.flatnonzero(~over)[:2], *np.flatnonzero(~over)[-2:]]:
+        assert np.array_equal(par[k].cpu().numpy(), O.tree(g, t0, 73, 2 + int(k)).parent)

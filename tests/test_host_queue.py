@@ -23,6 +23,7 @@ extern "C" uint64_t hq_trees_bytes(int64_t n) { return kc_host::pop_trees_bytes(
 extern "C" int64_t hq_trees_max(int contract) {
     return contract ? kc_host::kPopContractMax : kc_host::kPopTreesMax;
 }
+extern "C" int hq_pop_noalloc(int64_t n, int64_t t) { return kc_host::pop_noalloc(n, t); }
 extern "C" int64_t hq_pop_max() { return kc_host::kPopSmallMax; }
 """
 
@@ -46,6 +47,7 @@ def queue(tmp_path_factory):
     for f in (lib.hq_pop_bytes, lib.hq_pop_threads, lib.hq_trees_bytes):
         f.argtypes = [ctypes.c_int64]
     lib.hq_pop.argtypes = [ctypes.c_int64] * 3
+    lib.hq_pop_noalloc.argtypes = [ctypes.c_int64] * 2
     return lib
 
 
@@ -87,3 +89,13 @@ def test_popping_follows_size_and_root(queue):
     assert queue.hq_pop(trees + 1, 10 * trees, 20) == 0     # until it does not fit
     assert queue.hq_pop(4000000, 68000000, 8000) == 2
     assert queue.hq_pop(9000, 1 << 32, 8999) == 3           # 32-bit volumes do not hold 2m
+
+
+def test_many_trees_of_few_vertices_are_walked(queue):
+    """Past 128 trees a vertex; from 256 vertices on the scratch limit (n x trees at most
+    8 Mi) lets no call get there."""
+    for n in (2, 3, 40, 100, 255):
+        assert queue.hq_pop_noalloc(n, 128 * n) and not queue.hq_pop_noalloc(n, 128 * n + 1)
+    for n in (256, 2000, queue.hq_trees_max(0)):
+        assert queue.hq_pop_noalloc(n, (8 << 20) // n)
+    assert not queue.hq_pop_noalloc(queue.hq_trees_max(0) + 1, 1)
