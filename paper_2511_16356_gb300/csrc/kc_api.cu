@@ -402,8 +402,9 @@ int fast_traversal(const kc_graph *g) {
     return (g->ttf_variant == KC_TTF_SCAN && g->n >= (1 << 16)) ? kTravLeafUp : kTravChunked;
 }
 
-// Whether waves run the one-walker kernels with arrows drawn ahead (k1_solo.cu)
-// in place of the handle's walker: always for LANE, and under AUTO on
+// Whether a wave of B trees (reject: under rejection by walk length) runs the one-walker
+// kernels with arrows drawn ahead (k1_solo.cu) in place of the handle's walker: for LANE
+// while they are faster than a lane per tree (kc_host::queue_serves), and under AUTO on
 // long-diameter graphs, where 32 walkers of a tree mostly wait for one another
 // (40000-vertex grid, walk in ms with 32 walkers / one: 64 trees 192 / 114, 500
 // trees 348 / 184, 4000 trees 590 / 316).  On graphs of low diameter the 32
@@ -411,11 +412,11 @@ int fast_traversal(const kc_graph *g) {
 bool fits_queues(const kc_graph *g) {
     return kc_host::queue_bits(g->max_deg) <= kc_host::kMaxQueueBits;
 }
-bool use_solo(const kc_graph *g) {
+bool use_solo(const kc_graph *g, int64_t B, bool reject = false) {
     if (!fits_queues(g)) return false;
-    if (g->walker == KC_WALK_LANE) return true;
-    return g->walker == KC_WALK_WARP && g->auto_walker &&
-           g->ttf_variant == KC_TTF_BIT;
+    const bool bit = g->ttf_variant == KC_TTF_BIT;
+    if (g->walker == KC_WALK_LANE) return kc_host::queue_serves(B, g->num_sms, bit, reject);
+    return g->walker == KC_WALK_WARP && g->auto_walker && bit;
 }
 
 // Whether and how AUTO draws the trees of a low-diameter graph by cycle popping
@@ -776,7 +777,7 @@ bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
         B > 1 &&
         (B > p.BT || g->n >= (1 << 16))) {
         try {
-            if (!run_wave_pipelined(g, p, B, sid0, false, use_solo(g)))
+            if (!run_wave_pipelined(g, p, B, sid0, false, use_solo(g, B)))
                 run_wave_pipelined(g, p, B, sid0, false, false);
         } catch (Fail &) {
             // let both streams drain before the workspace is reused
@@ -793,7 +794,7 @@ bool run_wave(kc_graph *g, Plan &p, int64_t B, int64_t sid0, bool canonical = fa
     KC_CK(g, launch_iota(c.sids, sid0, B, g->stream));
     reset_segtab(g, B);
     uint32_t hdr[2] = {0, 0};
-    for (bool solo = use_solo(g) || (canonical && use_pop(g) && fits_queues(g));; solo = false) {
+    for (bool solo = use_solo(g, B) || (canonical && use_pop(g) && fits_queues(g));; solo = false) {
         KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
         {
             Phase ph(g, g->t_init);
@@ -1298,7 +1299,7 @@ void resample_slots(kc_graph *g, const std::vector<int64_t> &slots, bool cond, i
             KC_CK(g, copy_sync(g, &err, g->d_err, sizeof(err), cudaMemcpyDeviceToHost));
             if (solo_retry(g, err)) pop = kPopNone;
         }
-        for (bool solo = use_solo(g); !pop; solo = false) {
+        for (bool solo = use_solo(g, b); !pop; solo = false) {
             KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
             if (cond) {
                 if (solo) init_queues(g, gv, w, c.sids, -1, g->stream);
@@ -1562,7 +1563,7 @@ void run_wave_reject(kc_graph *g, Plan &p, int64_t B, int64_t sid0) {
     KC_CK(g, launch_iota(c.sids, sid0, B, g->stream));
     reset_segtab(g, B);
     uint32_t hdr[2] = {0, 0};
-    for (bool solo = use_solo(g);; solo = false) {
+    for (bool solo = use_solo(g, B, true);; solo = false) {
         KC_CK(g, cudaMemsetAsync(g->d_err, 0, 2 * sizeof(uint32_t), g->stream));
         {
             Phase ph(g, g->t_init);
@@ -1679,7 +1680,8 @@ void do_sample_reject(kc_graph *g, int64_t ntrees) {
             }
             if (B > 1 && (B > p.BT || g->n >= (1 << 16))) {
                 try {
-                    if (!run_wave_pipelined(g, p, B, g->next_sid, true, use_solo(g)))
+                    if (!run_wave_pipelined(g, p, B, g->next_sid, true,
+                                            use_solo(g, B, true)))
                         run_wave_pipelined(g, p, B, g->next_sid, true, false);
                 } catch (Fail &) {
                     // let both streams drain before the workspace is reused
@@ -1847,7 +1849,7 @@ void do_sample_multi(kc_graph *const *gs, const int64_t *n_trees, int32_t count)
             // trees have launches of their own.
             std::vector<char> solo(G), pop(G);
             for (size_t k = 0; k < G; ++k) {
-                solo[k] = use_solo(gs[idx[k]]) ? 1 : 0;
+                solo[k] = use_solo(gs[idx[k]], 1) ? 1 : 0;  // else 32 walkers a tree
                 pop[k] = (char)use_pop(gs[idx[k]]);
                 if (pop[k] != kPopSmall && bs[k] > plans[(size_t)idx[k]].BT) pop[k] = kPopNone;
             }
@@ -2335,7 +2337,7 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
                          ? KC_WALK_LANE : KC_WALK_WARP;
         g->walker = walker;
         g->auto_walker = cfg.walker == KC_WALK_AUTO && !cfg.autotune;
-        if (!use_solo(g) && !use_pop(g)) start_order(g);
+        if (!use_solo(g, 1) && !use_pop(g)) start_order(g);
     } catch (Fail &f) {
         kc_graph_destroy(g);
         return f.st;

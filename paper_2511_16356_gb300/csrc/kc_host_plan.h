@@ -121,6 +121,18 @@ inline int queue_group(int64_t B, int64_t num_sms) {
     return per_sm > 32 && per_sm <= 48 ? 16 : 32;
 }
 
+// Whether the LANE walker's wave of B trees runs those kernels, a warp or half a warp a
+// tree, or (so many trees that lanes fill the GPU) a lane a tree.  The line, in trees an
+// SM, depends on how even the walks are: about 145 to 205 on graphs of low diameter, 260
+// and more on long-diameter ones, 180 there under a cap that ends long walks early.
+// GB300, ms of a lane / a warp a tree: random graph of 300 vertices, 16000 trees 2.3 / 1.9,
+// 128000 trees 7.2 / 13.3; of 2000, 32000 trees 25 / 25, 64000 trees 35 / 50; grid 10x10,
+// 32000 trees 1.9 / 1.7, 256000 trees 6.7 / 12.0; grid 60x60, 32000 trees 109 / 68; grid
+// 100x100 under a cap, 16000 accepted trees 162 / 149, 32000 trees 221 / 291.
+inline bool queue_serves(int64_t B, int64_t num_sms, bool bit, bool reject) {
+    return B < std::max<int64_t>(num_sms, 1) * (!bit ? 160 : (reject ? 184 : 320));
+}
+
 // Cycle popping in shared memory (k_pop_small): its bytes for n vertices (two
 // words, a volume and a 16-bit size each; vertex ids are 16 bits), the largest n
 // (227 KB a block, less its static part) and the threads of a block.

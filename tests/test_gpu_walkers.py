@@ -285,3 +285,29 @@ def test_many_small_trees_without_allocation_match_oracle(trees, cap):
     assert np.array_equal(got[~over], want[~over]) and np.all(got[over] == cap + 1)
     for k in [*np.flatnonzero(~over)[:2], *np.flatnonzero(~over)[-2:]]:
         assert np.array_equal(par[k].cpu().numpy(), O.tree(g, t0, 73, 2 + int(k)).parent)
+
+
+@pytest.mark.parametrize("name,variant,per_sm", [("K3", 1, 160), ("er300", 1, 160),
+                                                 ("er300", 2, 320), ("grid17x13", 2, 320)])
+def test_a_lane_per_tree_matches_oracle(name, variant, per_sm):
+    """So many trees that the LANE walker takes a lane for each, both variants of f."""
+    g, trees = SMALL[name](), per_sm * 152
+    with kc.KemenyGraph.from_graph(g, _cfg(walker=kc.KC_WALK_LANE, ttf_variant=variant)) as G:
+        G.sample(19, trees)
+        _check(g, G.samples(), 19, 0, trees)
+
+
+@pytest.mark.parametrize("variant", [1, 2])
+def test_a_lane_per_tree_under_rejection_matches_oracle(variant):
+    g = SMALL["grid17x13"]()
+    t0 = O.tau0(g)
+    _, st = O.sample_batch(g, t0, 31, 0, 256)
+    cap, trees = int(np.quantile(st, 0.6)), 184 * 152
+    ids, f_ref, st_ref = O.accepted_samples(lambda a, c: O.sample_batch(g, t0, 31, a, c), cap,
+                                            trees, block=2 * trees)
+    with kc.KemenyGraph.from_graph(g, _cfg(walker=kc.KC_WALK_LANE, reject_steps=cap,
+                                           ttf_variant=variant)) as G:
+        G.sample(31, trees)
+        got = G.samples()
+    assert np.array_equal(got["sid"], ids)
+    assert np.array_equal(got["steps"], st_ref) and np.array_equal(got["f"], f_ref)

@@ -24,6 +24,9 @@ extern "C" int64_t hq_trees_max(int contract) {
     return contract ? kc_host::kPopContractMax : kc_host::kPopTreesMax;
 }
 extern "C" int hq_pop_noalloc(int64_t n, int64_t t) { return kc_host::pop_noalloc(n, t); }
+extern "C" int hq_serves(int64_t B, int64_t sms, int bit, int reject) {
+    return kc_host::queue_serves(B, sms, bit, reject);
+}
 extern "C" int64_t hq_pop_max() { return kc_host::kPopSmallMax; }
 """
 
@@ -47,6 +50,7 @@ def queue(tmp_path_factory):
     for f in (lib.hq_pop_bytes, lib.hq_pop_threads, lib.hq_trees_bytes):
         f.argtypes = [ctypes.c_int64]
     lib.hq_pop.argtypes = [ctypes.c_int64] * 3
+    lib.hq_serves.argtypes = [ctypes.c_int64, ctypes.c_int64, ctypes.c_int, ctypes.c_int]
     lib.hq_pop_noalloc.argtypes = [ctypes.c_int64] * 2
     return lib
 
@@ -99,3 +103,11 @@ def test_many_trees_of_few_vertices_are_walked(queue):
     for n in (256, 2000, queue.hq_trees_max(0)):
         assert queue.hq_pop_noalloc(n, (8 << 20) // n)
     assert not queue.hq_pop_noalloc(queue.hq_trees_max(0) + 1, 1)
+
+
+@pytest.mark.parametrize("bit,reject,per_sm", [(0, 0, 160), (0, 1, 160), (1, 0, 320),
+                                               (1, 1, 184)])
+def test_waves_of_very_many_trees_take_a_lane_each(queue, bit, reject, per_sm):
+    assert queue.hq_serves(1, 152, bit, reject)
+    assert queue.hq_serves(per_sm * 152 - 1, 152, bit, reject)
+    assert not queue.hq_serves(per_sm * 152, 152, bit, reject)
