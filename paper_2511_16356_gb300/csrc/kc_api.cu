@@ -1350,8 +1350,17 @@ void transform_slots(kc_graph *g, const std::vector<int64_t> &slots, bool insert
         // DFN serves; cut-link picks the k-th crossing edge in the id-ordered
         // preorder, and its trees hold the edge that the graph has lost
         int nl = 0;
-        KC_CK(g, launch_traverse_parents(gv, w, ParTrees{g->d_parents, ub.slots}, !insert,
-                                         insert ? -1 : u, insert ? -1 : v, true, g->stream, &nl));
+        if (kc_host::transform_in_order(b, g->n, g->num_sms, p.bit)) {
+            KC_CK(g, launch_prepare_from_parents(g->n, b, g->root, g->d_parents, ub.slots, w,
+                                                 g->stream));
+            KC_CK(g, launch_traverse(gv, w, true, g->stream, &nl,
+                                     insert ? kTravChunked : kTravCanonical));
+            nl += 4;
+        } else {
+            KC_CK(g, launch_traverse_parents(gv, w, ParTrees{g->d_parents, ub.slots}, !insert,
+                                             insert ? -1 : u, insert ? -1 : v, true, g->stream,
+                                             &nl));
+        }
         KC_CK(g, launch_link_cut(g->d_row_off, g->d_col, w, ub.slots, g->d_parents, ub.factor,
                                  ub.cut, g->root, u, v, g->seed, (uint32_t)g->update_seq, insert,
                                  g->stream));

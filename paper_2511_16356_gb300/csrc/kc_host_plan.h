@@ -133,6 +133,19 @@ inline bool queue_serves(int64_t B, int64_t num_sms, bool bit, bool reject) {
     return B < std::max<int64_t>(num_sms, 1) * (!bit ? 160 : (reject ? 184 : 320));
 }
 
+// Whether the retained trees that an ISM operation transforms, B of n vertices, are
+// traversed by a warp a tree in a parent-first order (launch_prepare_from_parents,
+// k2_traverse.cu) or by the order-free passes (k2_parents.cu), whose time is that of all
+// vertices: the first where its warps fill the GPU.  GB300, tree part of an insertion and
+// its deletion in ms, ordered / order-free: random graph of 2000 vertices, some 500 trees
+// 5.6 / 5.1, 2000 trees 8.4 / 11.3, 5000 trees 18.4 / 25.2; of 16500, 500 trees 35 / 26,
+// 2000 trees 87 / 83; of 60000, 500 trees 119 / 66; grid 100x100, 120 trees 18 / 12, 600
+// trees 25.6 / 26.7, 4800 trees 100 / 144; grid 300x300, 120 trees 148 / 70, 600 trees
+// 174 / 180.
+inline bool transform_in_order(int64_t B, int64_t n, int64_t num_sms, bool bit) {
+    return B >= 4 * num_sms + (bit ? 0 : n / 10);
+}
+
 // Cycle popping in shared memory (k_pop_small): its bytes for n vertices (two
 // words, a volume and a 16-bit size each; vertex ids are 16 bits), the largest n
 // (227 KB a block, less its static part) and the threads of a block.

@@ -238,3 +238,31 @@ def test_batched_updates_equal_one_at_a_time():
     assert np.array_equal(s1["f"], s2["f"]) and np.array_equal(s1["w"], s2["w"])
     assert np.array_equal(t1["p0"], t2["p0"])
     assert all(np.array_equal(a, b) for a, b in zip(p1, p2))
+
+
+@pytest.mark.parametrize("variant", [kc.KC_TTF_SCAN, kc.KC_TTF_BIT])
+@pytest.mark.parametrize("T", [1200, 3600])
+def test_ism_of_many_trees_bit_exact(variant, T):
+    """Pools of which an operation transforms fewer trees than take the ordered passes
+    (608, and a tenth of the vertices under SCAN), and more."""
+    g = S.er_lcc(40, 0.12, 3)
+    D = DynamicOracle(g, 29, T)
+    cfg = kc.kc_config_default()
+    cfg.keep_trees = 1
+    cfg.r_source = kc.KC_R_GIVEN
+    cfg.ttf_variant = variant
+    moved = [0]
+    with kc.KemenyGraph.from_graph(g, cfg) as G:
+        G.sample(29, T)
+        for (a, b, op) in _ops(g, np.random.default_rng(2), 4):
+            if op == 0:
+                arr = np.array(sorted(D.edges | {(a, b)}))
+                R = O.resistance(S.csr_from_edges(g.n, arr[:, 0], arr[:, 1]), a, b)
+                D.insert(a, b, kc.KC_UPDATE_ISM, R=R)
+                G.update([(a, b, 0, R)], kc.KC_UPDATE_ISM)
+            else:
+                D.delete(a, b, kc.KC_UPDATE_ISM)
+                G.update([(a, b, 1)], kc.KC_UPDATE_ISM)
+            _compare(G, D, g.n)
+            moved.append(G.stats()["trees_resampled"])
+    assert all((k >= 611) == (T == 3600) for k in np.diff(moved))

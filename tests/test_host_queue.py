@@ -27,6 +27,9 @@ extern "C" int hq_pop_noalloc(int64_t n, int64_t t) { return kc_host::pop_noallo
 extern "C" int hq_serves(int64_t B, int64_t sms, int bit, int reject) {
     return kc_host::queue_serves(B, sms, bit, reject);
 }
+extern "C" int hq_in_order(int64_t B, int64_t n, int64_t sms, int bit) {
+    return kc_host::transform_in_order(B, n, sms, bit);
+}
 extern "C" int64_t hq_pop_max() { return kc_host::kPopSmallMax; }
 """
 
@@ -51,6 +54,7 @@ def queue(tmp_path_factory):
         f.argtypes = [ctypes.c_int64]
     lib.hq_pop.argtypes = [ctypes.c_int64] * 3
     lib.hq_serves.argtypes = [ctypes.c_int64, ctypes.c_int64, ctypes.c_int, ctypes.c_int]
+    lib.hq_in_order.argtypes = [ctypes.c_int64, ctypes.c_int64, ctypes.c_int64, ctypes.c_int]
     lib.hq_pop_noalloc.argtypes = [ctypes.c_int64] * 2
     return lib
 
@@ -111,3 +115,10 @@ def test_waves_of_very_many_trees_take_a_lane_each(queue, bit, reject, per_sm):
     assert queue.hq_serves(1, 152, bit, reject)
     assert queue.hq_serves(per_sm * 152 - 1, 152, bit, reject)
     assert not queue.hq_serves(per_sm * 152, 152, bit, reject)
+
+
+def test_many_transformed_trees_are_traversed_in_order(queue):
+    for n in (2, 40, 2000, 1000000):
+        assert not queue.hq_in_order(607, n, 152, 1) and queue.hq_in_order(608, n, 152, 1)
+        line = 608 + n // 10
+        assert not queue.hq_in_order(line - 1, n, 152, 0) and queue.hq_in_order(line, n, 152, 0)
