@@ -2245,14 +2245,14 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
         if (cfg.sample_id_base < 0 || cfg.sample_id_base >= ((int64_t)1 << 32))
             throw Fail{KC_ERR_INVALID_ARG};
         g->next_sid = cfg.sample_id_base;
-        // host copy of the CSR (validated layout, kept for updates)
+        // host copy of the CSR (validated layout, kept for updates), by copies on the
+        // stream: the caller's arrays may still be the target of work queued before the
+        // call (reading them in place instead saved 0.1 of 5.3 ms at 5 million edges)
+        const cudaMemcpyKind kind =
+            cfg.inputs_on_device ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost;
         auto take = [&](auto &dst, const auto *src, size_t count) {
-            if (!cfg.inputs_on_device) {
-                dst.assign(src, src + count);
-                return;
-            }
             dst.resize(count);
-            KC_CK(g, copy_sync(g, dst.data(), src, sizeof(*src) * count, cudaMemcpyDeviceToHost));
+            KC_CK(g, copy_sync(g, dst.data(), src, sizeof(*src) * count, kind));
         };
         take(g->h_row_off, row_off, (size_t)n + 1);
         if (g->h_row_off[0] != 0) throw Fail{KC_ERR_INVALID_ARG};

@@ -1,5 +1,7 @@
 """GPU tests of the walkers' waves against the CPU oracle: failed trees of a
 pipelined wave, segment tables across waves."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -311,3 +313,32 @@ def test_a_lane_per_tree_under_rejection_matches_oracle(variant):
         got = G.samples()
     assert np.array_equal(got["sid"], ids)
     assert np.array_equal(got["steps"], st_ref) and np.array_equal(got["f"], f_ref)
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+def test_creation_waits_for_copies_into_its_arrays(pinned):
+    """A handle from host arrays that an asynchronous copy queued before the call still
+    fills, and one from device arrays under the host flag: the runtime orders and finds both."""
+    torch = pytest.importorskip("torch")
+    g = SMALL["er300"]()
+    dev = [torch.from_numpy(x).cuda() for x in (g.row_off, g.col)]
+    src = dev
+    if pinned:
+        src = [torch.zeros(x.shape, dtype=x.dtype).pin_memory() for x in dev]
+    with kc.KemenyGraph.from_graph(g):  # sets the device up: no step of the next one waits
+        pass
+    torch.cuda.synchronize()
+    if pinned:
+        with torch.cuda.stream(torch.cuda.default_stream()):
+            torch.cuda._sleep(200_000_000)
+            for h, d in zip(src, dev):
+                h.copy_(d, non_blocking=True)
+    h, cfg = ctypes.c_void_p(), _cfg()
+    st = kc.load().kc_graph_create(g.n, src[0].data_ptr(), src[1].data_ptr(), ctypes.byref(cfg),
+                                   ctypes.byref(h))
+    assert kc.STATUS[st] == "KC_OK"
+    try:
+        kc.kc_sample(h, 17, 20)
+        _check(g, kc.kc_get_samples(h, 0, 20), 17, 0, 20)
+    finally:
+        kc.kc_graph_destroy(h)
