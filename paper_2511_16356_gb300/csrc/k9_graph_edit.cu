@@ -23,7 +23,8 @@
 namespace kc {
 namespace {
 
-// pos[0] = pa, pos[1] = pb, pos[2] = error (1: the edit does not apply)
+// pos[0] = pa, pos[1] = pb, pos[2] = error (1: the edit does not apply), pos[3] and
+// pos[4] = the degrees of a and b before it
 __global__ void k_edit_positions(const int64_t *row_off, const int32_t *col, int32_t a,
                                  int32_t b, int insert, int64_t *pos) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
@@ -39,6 +40,7 @@ __global__ void k_edit_positions(const int64_t *row_off, const int32_t *col, int
         const bool present = lo < row_off[row + 1] && col[lo] == key;
         if (present == (insert != 0)) ok = false;
         p[k] = lo;
+        pos[3 + k] = row_off[row + 1] - row_off[row];
     }
     pos[0] = p[0];
     pos[1] = p[1];
@@ -82,7 +84,7 @@ __global__ void k_edit_offsets(int64_t n, int64_t *row_off, int32_t a, int32_t b
 
 // Insert or delete the undirected edge (u, v) of an n-vertex CSR whose column
 // array holds 2m entries now (capacity >= 2m + 2 for an insert).  `scratch`
-// holds >= 2m + 2 int32 and `pos` 3 int64 of device memory.  Enqueued on s; a
+// holds >= 2m + 2 int32 and `pos` 5 int64 of device memory.  Enqueued on s; a
 // precondition failure (edge present on insert, absent on delete) leaves the
 // CSR unchanged and pos[2] = 1.
 cudaError_t launch_csr_edit(int64_t n, int64_t twom, int64_t *row_off, int32_t *col,

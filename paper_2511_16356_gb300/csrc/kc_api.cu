@@ -1134,24 +1134,24 @@ void edit_graph(kc_graph *g, int32_t u, int32_t v, bool insert) {
         dalloc(g, &g->d_edit, cap);
         g->edit_cap = cap;
     }
-    int64_t *pos = (int64_t *)g->d_scratch + 64;  // 3 words past the reduction sums
+    int64_t *pos = (int64_t *)g->d_scratch + 64;  // 5 words past the reduction sums
     KC_CK(g, launch_csr_edit(g->n, twom, g->d_row_off, g->d_col, g->d_edit, pos, u, v, insert,
                              g->stream));
-    int64_t hp[3] = {0, 0, 0};
+    int64_t hp[5] = {0, 0, 0, 0, 0};
     KC_CK(g, copy_sync(g, hp, pos, sizeof(hp), cudaMemcpyDeviceToHost));
     if (hp[2]) {
         g->last_error = "kc_update: the device graph does not match the validated batch";
         throw Fail{KC_ERR_CUDA};
     }
     g->m += insert ? 1 : -1;
-    g->max_deg += insert ? 1 : 0;
+    if (insert) g->max_deg = kc_host::max_degree_with_edge(g->max_deg, hp[3], hp[4]);
     g->host_csr_stale = true;
-    KC_CK(g, launch_build_records(view_of(g), g->d_rec, g->max_deg <= 4 ? g->d_rec4 : nullptr,
-                                  g->d_deg, g->stream));
+    KC_CK(g, launch_build_records(view_of(g), g->d_rec, g->d_rec4, g->d_deg, g->stream));
     g->t_update.launches += 4;
 }
 
-// the host copy of the CSR (batch validation reads it) from the device
+// the host copy of the CSR (batch validation reads it) from the device, and with it the
+// largest degree, which a batch's deletions may have lowered
 void sync_host_csr(kc_graph *g) {
     if (!g->host_csr_stale) return;
     const int64_t n = g->n;
@@ -1162,6 +1162,7 @@ void sync_host_csr(kc_graph *g) {
     g->h_col.resize((size_t)twom);
     KC_CK(g, copy_sync(g, g->h_col.data(), g->d_col, sizeof(int32_t) * (size_t)twom,
                        cudaMemcpyDeviceToHost));
+    g->max_deg = kc_host::max_degree(g->h_row_off.data(), n);
     g->host_csr_stale = false;
 }
 
@@ -2256,11 +2257,9 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
         };
         take(g->h_row_off, row_off, (size_t)n + 1);
         if (g->h_row_off[0] != 0) throw Fail{KC_ERR_INVALID_ARG};
-        for (int64_t v = 0; v < n; ++v) {
-            const int64_t d = g->h_row_off[v + 1] - g->h_row_off[v];
-            if (d < 0) throw Fail{KC_ERR_INVALID_ARG};
-            g->max_deg = std::max(g->max_deg, d);
-        }
+        for (int64_t v = 0; v < n; ++v)
+            if (g->h_row_off[v + 1] < g->h_row_off[v]) throw Fail{KC_ERR_INVALID_ARG};
+        g->max_deg = kc_host::max_degree(g->h_row_off.data(), n);
         const int64_t twom = g->h_row_off[n];
         if (twom % 2 != 0 || twom == 0) throw Fail{twom == 0 ? KC_ERR_DISCONNECTED : KC_ERR_NOT_SYMMETRIC};
         g->m = twom / 2;

@@ -285,13 +285,13 @@ struct kc_graph {
     int device = 0;
     cudaStream_t stream = nullptr;
     int64_t n = 0, m = 0;
-    int64_t max_deg = 0;  // largest degree (an upper bound after deletions)
+    int64_t max_deg = 0;  // largest degree (within a batch of updates an upper bound)
     // device graph
     int64_t *d_row_off = nullptr;
     int32_t *d_col = nullptr;
     int32_t *d_deg = nullptr;
     kc::VRec *d_rec = nullptr;
-    int4 *d_rec4 = nullptr;  // used while max_deg <= 4
+    int4 *d_rec4 = nullptr;  // null if some degree exceeded 4 at creation; used while max_deg <= 4
     int32_t root = -1, ecc = 0;
     int32_t *d_p0 = nullptr, *d_level0 = nullptr, *d_in0 = nullptr, *d_out0 = nullptr;
     int32_t ttf_variant = KC_TTF_SCAN;

@@ -25,6 +25,17 @@ inline uint64_t edge_key(int32_t a, int32_t b) {
     return ((uint64_t)(uint32_t)a << 32) | (uint64_t)(uint32_t)b;
 }
 
+inline int64_t max_degree(const int64_t *row_off, int64_t n) {
+    int64_t d = 0;
+    for (int64_t v = 0; v < n; ++v) d = std::max(d, row_off[v + 1] - row_off[v]);
+    return d;
+}
+
+// An upper bound on it after an insertion between vertices of degrees da and db.
+inline int64_t max_degree_with_edge(int64_t max_deg, int64_t da, int64_t db) {
+    return std::max(max_deg, std::max(da, db) + 1);
+}
+
 class OverlayGraph {
   public:
     // row_off[n + 1] and col[2m]: the base graph, rows sorted ascending; the

@@ -266,3 +266,33 @@ def test_ism_of_many_trees_bit_exact(variant, T):
             _compare(G, D, g.n)
             moved.append(G.stats()["trees_resampled"])
     assert all((k >= 611) == (T == 3600) for k in np.diff(moved))
+
+
+@pytest.mark.parametrize("walker", [kc.KC_WALK_LANE, kc.KC_WALK_WARP])
+def test_walks_follow_the_largest_degree_of_an_edited_graph(walker):
+    """A graph of degree at most 4 that an insertion takes to 5 and later batches back to 4,
+    with other neighbours than before: trees after each batch match the oracle."""
+    g = S.grid(9, 7)  # 9 columns: vertex 10 and its neighbours have degree 4
+    edges = {(int(a), int(b)) for a, b in g.edges()}
+    cfg = kc.kc_config_default()
+    cfg.keep_trees = 1
+    cfg.r_source = kc.KC_R_GIVEN
+    cfg.walker = walker
+    batches = [[(10, 20, 0)], [(10, 11, 1), (20, 21, 1)], [(0, 10, 0), (0, 10, 1), (0, 8, 0)]]
+    with kc.KemenyGraph.from_graph(g, cfg) as G:
+        G.sample(30, 8)
+        for k, batch in enumerate(batches):
+            for a, b, op in batch:
+                (edges.discard if op else edges.add)((a, b))
+            G.update([(a, b, op, 0.5) if op == 0 else (a, b, op) for a, b, op in batch],
+                     kc.KC_UPDATE_ISM)
+            arr = np.array(sorted(edges))
+            h = S.csr_from_edges(g.n, arr[:, 0], arr[:, 1])
+            tau = G.tau0()
+            t0 = O.tau0(h, tau["root"])
+            G.reset(31 + k)
+            G.sample(31 + k, 200)
+            _, st_ref = O.sample_batch(h, t0, 31 + k, 0, 200)
+            assert np.array_equal(G.samples()["steps"], st_ref)
+            for t in (0, 57, 199):
+                assert np.array_equal(G.tree(t)["parent"], O.tree(h, t0, 31 + k, t).parent)

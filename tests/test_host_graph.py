@@ -21,6 +21,10 @@ CSRC = os.path.join(ROOT, "paper_2511_16356_gb300", "csrc")
 
 SHIM = r"""
 #include "kc_host_graph.h"
+extern "C" int64_t hg_max_degree(int64_t n, const int64_t *ro) { return kc_host::max_degree(ro, n); }
+extern "C" int64_t hg_with_edge(int64_t d, int64_t da, int64_t db) {
+    return kc_host::max_degree_with_edge(d, da, db);
+}
 extern "C" int hg_run(int64_t n, const int64_t *ro, const int32_t *col, int64_t n_ops,
                       const int32_t *ops, int32_t *out) {
     kc_host::OverlayGraph og(ro, col, n);
@@ -160,3 +164,19 @@ def test_bridges_of_a_path_and_cycle_edges(shim):
     c = S.cycle(40)
     got = _run(shim, c, [(0, 1, 1), (20, 21, 1)])
     assert got[0].tolist() == [1, 1] and got[1].tolist() == [1, 0]  # the second cut splits C40
+
+
+def test_largest_degree_follows_the_edges(shim):
+    """Insertions and deletions that undo each other leave the bound within one batch, and
+    the value after it, where they were: it only grows with its own endpoints."""
+    shim.hg_max_degree.restype = shim.hg_with_edge.restype = ctypes.c_int64
+    shim.hg_max_degree.argtypes = [ctypes.c_int64, ctypes.c_void_p]
+    shim.hg_with_edge.argtypes = [ctypes.c_int64] * 3
+    g = S.grid(9, 7)
+    deg = np.diff(g.row_off)
+    top = shim.hg_max_degree(g.n, g.row_off.ctypes.data)
+    assert top == deg.max() == 4
+    for _ in range(100):  # the same corner edge again and again
+        top = shim.hg_with_edge(top, deg[0], deg[8])
+    assert top == 4
+    assert shim.hg_with_edge(4, 4, 2) == 5 and shim.hg_with_edge(4, 2, 4) == 5
