@@ -296,3 +296,29 @@ def test_walks_follow_the_largest_degree_of_an_edited_graph(walker):
             assert np.array_equal(G.samples()["steps"], st_ref)
             for t in (0, 57, 199):
                 assert np.array_equal(G.tree(t)["parent"], O.tree(h, t0, 31 + k, t).parent)
+
+
+@pytest.mark.parametrize("name", ["er20000", "cl20000", "cl50000"])
+def test_resampled_trees_of_every_popped_kind(name):
+    """BSM replacements, conditioned on the new edge and not, popped in shared memory: with
+    contracted rounds up to 38000 vertices and without them up to 56000."""
+    n = int(name[2:])
+    g = S.er_lcc(n, 8.0 / n, 9) if name[:2] == "er" else S.chung_lu(n, 2.1, 8.0, 5)
+    seed, T = 37, 6
+    D = DynamicOracle(g, seed, T)
+    cfg = kc.kc_config_default()
+    cfg.keep_trees = 1
+    cfg.r_source = kc.KC_R_GIVEN
+    rng = np.random.default_rng(11)
+    u, v = (int(x) for x in rng.choice(g.n, 2, replace=False))
+    a, b = min(u, v), max(u, v)
+    assert (a, b) not in D.edges
+    with kc.KemenyGraph.from_graph(g, cfg) as G:
+        G.sample(seed, T)
+        D.insert(a, b, kc.KC_UPDATE_BSM, R=0.9)
+        G.update([(a, b, 0, 0.9)], kc.KC_UPDATE_BSM)
+        _compare(G, D, g.n)
+        D.delete(a, b, kc.KC_UPDATE_BSM)
+        G.update([(a, b, 1)], kc.KC_UPDATE_BSM)
+        _compare(G, D, g.n)
+        assert G.stats()["trees_resampled"] >= 2 * 6

@@ -342,3 +342,102 @@ def test_creation_waits_for_copies_into_its_arrays(pinned):
         _check(g, kc.kc_get_samples(h, 0, 20), 17, 0, 20)
     finally:
         kc.kc_graph_destroy(h)
+
+
+@pytest.mark.parametrize("n", [40002, 70002])
+def test_lane_walker_without_queues_matches_oracle(n):
+    """Neighbour indices too wide for an arrow queue (a vertex of degree n - 2): a lane per
+    tree, in plain and (70002 vertices) pipelined waves, also rejecting and at the cap."""
+    g = S.complete_bipartite(2, n - 2)
+    t0 = O.tau0(g)
+    with kc.KemenyGraph.from_graph(g, _cfg(walker=kc.KC_WALK_LANE)) as G:
+        G.sample(53, 12)
+        _check(g, G.samples(), 53, 0, 12)
+    _, st = O.sample_batch(g, t0, 59, 0, 32)
+    cap = int(np.quantile(st, 0.6))
+    ids, f_ref, st_ref = O.accepted_samples(lambda a, c: O.sample_batch(g, t0, 59, a, c), cap,
+                                            10, block=32)
+    with kc.KemenyGraph.from_graph(g, _cfg(walker=kc.KC_WALK_LANE, reject_steps=cap)) as G:
+        G.sample(59, 10)
+        got = G.samples()
+    assert np.array_equal(got["sid"], ids)
+    assert np.array_equal(got["steps"], st_ref) and np.array_equal(got["f"], f_ref)
+    with kc.KemenyGraph.from_graph(g, _cfg(walker=kc.KC_WALK_LANE, step_cap=5000)) as G:
+        assert kc.STATUS[kc.kc_sample(G.h, 3, 8, check=False)] == "KC_ERR_STEP_LIMIT"
+        assert G.stats()["pool_trees"] == 0
+
+
+def _clique_on_a_path(k, length):
+    """K_k with a path of `length` edges from its vertex k - 1; its far end is the last id.
+    A clique vertex departs about k x length times from there on the way to that end."""
+    iu, iv = np.triu_indices(k, 1)
+    p = np.arange(k - 1, k + length - 1)
+    return S.csr_from_edges(k + length, np.r_[iu, p], np.r_[iv, p + 1])
+
+
+def test_pops_past_their_count_field_are_walked():
+    """More pops of one vertex (about 10000) than a popped tree counts (8191): the walkers
+    give the oracle's trees, through a handle and without allocation."""
+    torch = pytest.importorskip("torch")
+    g, trees = _clique_on_a_path(100, 100), 6
+    root = g.n - 1
+    t0 = O.tau0(g, root)
+    f_ref, st_ref = O.sample_batch(g, t0, 61, 0, trees)
+    with kc.KemenyGraph.from_graph(g, _cfg(keep_trees=1, root=root, ttf_variant=1)) as G:
+        G.sample(61, trees)
+        got = G.samples()
+        assert np.array_equal(got["steps"], st_ref) and np.array_equal(got["f"], f_ref)
+        assert np.array_equal(G.tree(3)["parent"], O.tree(g, t0, 61, 3).parent)
+    ro, co = torch.from_numpy(g.row_off).cuda(), torch.from_numpy(g.col).cuda()
+    par = torch.zeros((trees, g.n), dtype=torch.int32, device="cuda")
+    steps = torch.zeros(trees, dtype=torch.int64, device="cuda")
+    status = torch.full((1,), 5, dtype=torch.int32, device="cuda")
+    assert kc.load().kc_wilson_noalloc(g.n, ro.data_ptr(), co.data_ptr(), root, 61, 0, trees, 0,
+                                       par.data_ptr(), steps.data_ptr(), status.data_ptr(),
+                                       torch.cuda.current_stream().cuda_stream) == kc.KC_OK
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and np.array_equal(steps.cpu().numpy(), st_ref)
+    for k in range(trees):
+        assert np.array_equal(par[k].cpu().numpy(), O.tree(g, t0, 61, k).parent)
+
+
+def test_a_batched_wave_past_a_cap_is_drawn_again():
+    """One graph of a batched call passes its cap under popping, another under the queue
+    walk: the wave is repeated with 32 walkers, whose cap is per walker."""
+    graphs = [SMALL[k]() for k in ("er300", "cycle500", "cl3000", "K3")]
+    caps = []
+    for g in graphs:
+        _, st = O.sample_batch(g, O.tau0(g), 67, 0, 40)
+        caps.append(int(st.max()) - 1)
+    for capped in ([0], [1], [0, 1]):
+        Gs = [kc.KemenyGraph.from_graph(g, _cfg(step_cap=caps[k] if k in capped else 0))
+              for k, g in enumerate(graphs)]
+        try:
+            kc.kc_sample_multi([G.h for G in Gs], [67] * 4, [40] * 4)
+            for g, G in zip(graphs, Gs):
+                _check(g, G.samples(), 67, 0, 40)
+        finally:
+            for G in Gs:
+                G.close()
+
+
+def test_kept_trees_of_every_popped_kind_in_a_batched_call():
+    """In one call: trees in shared memory with and without f (16500 vertices, no hub), in
+    memory (20000, a hub), and the walkers' trees; f, step counts and kept trees."""
+    graphs = [SMALL["er300"](), S.er_lcc(16500, 8.0 / 16500, 9), S.chung_lu(20000, 2.1, 8.0, 5),
+              SMALL["grid17x13"](), S.er_lcc(40000, 8.0 / 40000, 9)]
+    Gs = [kc.KemenyGraph.from_graph(g, _cfg(keep_trees=1)) for g in graphs]
+    try:
+        for first in (0, 9):
+            kc.kc_sample_multi([G.h for G in Gs], [71] * 5, [9] * 5)
+            for g, G in zip(graphs, Gs):
+                _check(g, G.samples(first, 9), 71, first, 9)
+        for g, G in zip(graphs, Gs):
+            t0 = O.tau0(g)
+            for k in (0, 8, 9, 17):
+                tr, ref = G.tree(k), O.tree(g, t0, 71, k)
+                for key in ("parent", "depth", "din", "dout", "vol"):
+                    assert np.array_equal(tr[key], getattr(ref, key)), key
+    finally:
+        for G in Gs:
+            G.close()
