@@ -13,21 +13,34 @@ namespace {
 constexpr int kBlocks = 304;   // 2 per SM
 constexpr int kThreads = 256;
 
-// kLanes lanes a row: a thread a row made every product wait for the hubs' rows
-// (power-law graph of 100000 vertices, largest degree 1400: 125 us a product).
+// out = L p, a thread a row or (kLanes 8) 8 lanes a row.  A thread a row waits for the
+// hubs' rows; 8 lanes leave the short rows of the other graphs half empty (bound: the
+// random sectors of p).  GB300, one insertion's resistance in ms, 1 / 8 lanes: 1000x1000
+// grid 512 / 944, random graph of 10^6 vertices and mean degree 8 5.2 / 7.7; power-law
+// graphs of 300000 vertices 11.1 / 4.0, of 10^6 29 / 12, star of 20000 9.6 / 2.6.  32
+// lanes took 7.8 on the power-law graph of 300000 vertices.
+constexpr int kRowLanes = 8;
 template <int kLanes>
 __global__ void __launch_bounds__(kThreads) k_lap_spmv(GraphView g, const double *p, double *out) {
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kLanes;
-    const int lane = threadIdx.x & (kLanes - 1);
-    double acc = 0.0;
-    if (i < g.n) {
-        const int64_t end = g.row_off[i + 1];
+    if constexpr (kLanes == 1) {
+        if (i >= g.n) return;
+        double acc = (double)g.deg[i] * p[i];
+        for (int64_t e = g.row_off[i]; e < g.row_off[i + 1]; ++e) acc -= p[g.col[e]];
+        out[i] = acc;
+    } else {
+        const int lane = threadIdx.x & (kLanes - 1);
+        double acc = 0.0;
+        if (i < g.n) {
+            const int64_t end = g.row_off[i + 1];
 #pragma unroll 4
-        for (int64_t e = g.row_off[i] + lane; e < end; e += kLanes) acc += p[g.col[e]];
-    }
+            for (int64_t e = g.row_off[i] + lane; e < end; e += kLanes) acc += p[g.col[e]];
+        }
 #pragma unroll
-    for (int o = kLanes / 2; o > 0; o >>= 1) acc += __shfl_down_sync(0xFFFFFFFFu, acc, o, kLanes);
-    if (i < g.n && lane == 0) out[i] = (double)g.deg[i] * p[i] - acc;
+        for (int o = kLanes / 2; o > 0; o >>= 1)
+            acc += __shfl_down_sync(0xFFFFFFFFu, acc, o, kLanes);
+        if (i < g.n && lane == 0) out[i] = (double)g.deg[i] * p[i] - acc;
+    }
 }
 
 // partial[b] = sum over this block's grid-stride share of a_i * b_i
@@ -100,8 +113,8 @@ void cg_graph_release(CgGraph &c) {
     c = CgGraph{};
 }
 
-cudaError_t resistance_cg(const GraphView &g, int32_t u, int32_t v, double tol, int64_t max_iter,
-                          double *buf, double *R_out, int64_t *iters_out, int *launches,
+cudaError_t resistance_cg(const GraphView &g, bool by_lanes, int32_t u, int32_t v, double tol,
+                          int64_t max_iter, double *buf, double *R_out, int64_t *iters_out, int *launches,
                           cudaStream_t s, CgGraph *cache) {
     const int64_t n = g.n;
     cudaError_t e = cudaSuccess;
@@ -120,12 +133,11 @@ cudaError_t resistance_cg(const GraphView &g, int32_t u, int32_t v, double tol, 
     dot(r, z, sc + 0);
     // one CG iteration: 9 launches and a scalar copy, all on s
     auto iteration = [&]() -> cudaError_t {
-        if (g.twom > 12 * n)
-            k_lap_spmv<32><<<(unsigned)((n * 32 + kThreads - 1) / kThreads), kThreads, 0, cur>>>(
-                g, p, ap);
+        if (by_lanes)
+            k_lap_spmv<kRowLanes><<<(unsigned)((n * kRowLanes + kThreads - 1) / kThreads), kThreads,
+                                    0, cur>>>(g, p, ap);
         else
-            k_lap_spmv<8><<<(unsigned)((n * 8 + kThreads - 1) / kThreads), kThreads, 0, cur>>>(
-                g, p, ap);
+            k_lap_spmv<1><<<nb, kThreads, 0, cur>>>(g, p, ap);
         ++nl;
         dot(p, ap, sc + 1);
         k_cg_update_xr<<<nb, kThreads, 0, cur>>>(n, g.deg, sc, x, r, z, p, ap);

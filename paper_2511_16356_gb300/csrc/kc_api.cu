@@ -1405,8 +1405,8 @@ void apply_insert(kc_graph *g, int32_t u, int32_t v, int32_t mode, double r_give
         int nl = 0;
         int64_t iters = 0;
         if (!g->d_cg) dalloc(g, &g->d_cg, cg_scratch_doubles(g->n));
-        KC_CK(g, resistance_cg(view_of(g), u, v, 1e-13, 50 * g->n + 1000, g->d_cg, &R, &iters,
-                               &nl, g->stream, &g->cg_graph));
+        KC_CK(g, resistance_cg(view_of(g), g->cg_by_lanes, u, v, 1e-13, 50 * g->n + 1000, g->d_cg,
+                               &R, &iters, &nl, g->stream, &g->cg_graph));
         g->t_update.launches += nl;
         g->last_cg_iters = iters;
     }
@@ -2260,6 +2260,7 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
         for (int64_t v = 0; v < n; ++v)
             if (g->h_row_off[v + 1] < g->h_row_off[v]) throw Fail{KC_ERR_INVALID_ARG};
         g->max_deg = kc_host::max_degree(g->h_row_off.data(), n);
+        g->cg_by_lanes = kc_host::spmv_by_lanes(g->max_deg);
         const int64_t twom = g->h_row_off[n];
         if (twom % 2 != 0 || twom == 0) throw Fail{twom == 0 ? KC_ERR_DISCONNECTED : KC_ERR_NOT_SYMMETRIC};
         g->m = twom / 2;

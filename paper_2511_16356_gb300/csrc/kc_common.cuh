@@ -286,6 +286,8 @@ struct kc_graph {
     cudaStream_t stream = nullptr;
     int64_t n = 0, m = 0;
     int64_t max_deg = 0;  // largest degree (within a batch of updates an upper bound)
+    bool cg_by_lanes = false;  // kc_host::spmv_by_lanes at creation: R of an operation is the
+                               // same in a batch and on its own
     // device graph
     int64_t *d_row_off = nullptr;
     int32_t *d_col = nullptr;
@@ -594,9 +596,10 @@ cudaError_t launch_scatter_results(const int64_t *slot, int64_t B, const int64_t
 // in the cache for later calls on the same CSR, scratch and n.
 void cg_graph_release(CgGraph &c);
 size_t cg_scratch_doubles(int64_t n);
-cudaError_t resistance_cg(const GraphView &g, int32_t u, int32_t v, double tol, int64_t max_iter,
-                          double *scratch, double *R_out, int64_t *iters_out, int *launches,
-                          cudaStream_t s, CgGraph *cache = nullptr);
+// by_lanes: 8 lanes a row of the Laplacian, not a thread (another order of its sums)
+cudaError_t resistance_cg(const GraphView &g, bool by_lanes, int32_t u, int32_t v, double tol,
+                          int64_t max_iter, double *scratch, double *R_out, int64_t *iters_out,
+                          int *launches, cudaStream_t s, CgGraph *cache = nullptr);
 // one edge insert / delete of the device CSR, rows kept sorted (k9_graph_edit.cu)
 cudaError_t launch_csr_edit(int64_t n, int64_t twom, int64_t *row_off, int32_t *col,
                             int32_t *scratch, int64_t *pos, int32_t u, int32_t v, bool insert,

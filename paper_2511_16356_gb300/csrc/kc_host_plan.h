@@ -186,4 +186,10 @@ inline int pop_small_threads(int64_t n) {
     return n <= 1024 ? 128 : (n <= 4096 ? 256 : (n <= 8192 ? 512 : 1024));
 }
 
+// Whether a row of the Laplacian product (k8_resistance.cu) is added up by 8 lanes, not by
+// one thread: where some row is so long that the product would wait for its chain of
+// loads.  The rows of random graphs of mean degree 20 and less are shorter, the hubs of
+// power-law graphs longer (figures there).
+constexpr bool spmv_by_lanes(int64_t max_deg) { return max_deg > 64; }
+
 }  // namespace kc_host

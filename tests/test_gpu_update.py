@@ -322,3 +322,16 @@ def test_resampled_trees_of_every_popped_kind(name):
         G.update([(a, b, 1)], kc.KC_UPDATE_BSM)
         _compare(G, D, g.n)
         assert G.stats()["trees_resampled"] >= 2 * 6
+
+
+@pytest.mark.parametrize("k", [1, 7, 8, 62, 63, 64, 65, 1000])
+def test_cg_resistance_of_long_rows(k):
+    """The new edge joins the two vertices of degree k in K_{2,k}: R = 1 / (1 + k / 2).  Rows
+    shorter and longer than 8 lanes, and either side of the line between a thread and 8
+    lanes a row (degree 64)."""
+    g = S.complete_bipartite(2, k)
+    u, v = 0, 1
+    with kc.KemenyGraph.from_graph(g) as G:
+        G.sample(5, 8)
+        G.update([(u, v, 0)], kc.KC_UPDATE_BSM)
+        assert G.stats()["last_resistance"] == pytest.approx(1 / (1 + k / 2), rel=1e-11)
