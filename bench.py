@@ -284,19 +284,31 @@ def timed_sampling(G, T: int, steps: int, seed: int, stream, flush) -> list:
     return step_ms
 
 
-def walk_kernel(kc, st: dict, auto: bool) -> str:
-    """The kernel that draws the trees (auto: the library chose it by the graph)."""
+def walk_kernel(kc, st: dict, auto: bool, deg, reject: bool = False) -> str:
+    """The kernel that draws the trees (auto: the library chose it by the graph), by the rules
+    of csrc/kc_host_plan.h (queue_bits, queue_serves, pop_kind); deg: the degrees."""
     bit = st["ttf_variant"] == kc.KC_TTF_BIT
-    if st["walker"] == kc.KC_WALK_LANE or (auto and bit):
+    queues = int(deg.max()) <= 1 << 15
+    if st["walker"] == kc.KC_WALK_LANE:
+        line = 152 * (160 if not bit else (184 if reject else 320))
+        return "k_wilson_queue" if queues and st["trees_in_flight"] < line else "k_wilson"
+    if st["walker"] == kc.KC_WALK_HYBRID:
+        return "k_wilson+k_wilson_warp"
+    if auto and bit and queues:
         return "k_wilson_queue"
-    if auto:  # popped where a block's shared memory holds the tree or the root is a hub
-        return "k_pop_small" if st["n"] <= 38000 else "k_pop_rounds"
-    return {kc.KC_WALK_WARP: "k_wilson_warp",
-            kc.KC_WALK_HYBRID: "k_wilson+k_wilson_warp"}[st["walker"]]
+    if auto and not bit and not reject:
+        n, twom = st["n"], 2 * st["m"]
+        if n <= 16000 and twom < 1 << 32:
+            return "k_pop_small"
+        if 16 * (twom // max(int(deg[st["root"]]), 1)) <= n:
+            return "k_pop_rounds"
+        if n <= 38000:
+            return "k_pop_small"
+    return "k_wilson_warp"
 
 
 def phase_roofline(kc, st: dict, n: int, trees: int, steps_total: int, tot_ms: float,
-                   walker_traffic=None, auto=True) -> tuple:
+                   walker: str, walker_traffic=None) -> tuple:
     """The dominant phase of the timed steps (kc_stats' CUDA-event phase timers)
     and its roofline object: algorithmic bytes per launch over the mean launch
     time, against the measured HBM copy peak; plus the whole path's fraction."""
@@ -313,7 +325,7 @@ def phase_roofline(kc, st: dict, n: int, trees: int, steps_total: int, tot_ms: f
     per_launch_bytes = alg / max(1, dom_launches)
     per_launch_s = max(dom_ms, 1e-9) / 1000.0 / max(1, dom_launches)
     achieved = per_launch_bytes / per_launch_s / 1e9
-    kernel_name = {"wilson": walk_kernel(kc, st, auto),
+    kernel_name = {"wilson": walker,
                    "traverse": "traversal passes",
                    "ttf_bit": "k_ttf_bit", "ttf_scan": "k_ttf_scan"}[dom]
     traffic = None
@@ -391,7 +403,8 @@ def other_workload_leg(args, kc, stream, flush, name: str, T: int, steps: int, w
     st = G.stats()
     smp = G.samples(pool0, st["pool_trees"] - pool0)
     steps_total = int(smp["steps"].sum())
-    dom, roof, phase_ms = phase_roofline(kc, st, g.n, T * steps, steps_total, tot_ms)
+    walker = walk_kernel(kc, st, True, g.deg)
+    dom, roof, phase_ms = phase_roofline(kc, st, g.n, T * steps, steps_total, tot_ms, walker)
     G.close()
     out = {"workload": S.WORKLOADS.get(name, name), "n": g.n, "m": g.m, "ecc": st["ecc"],
            "trees_per_step": T, "steps": steps, "warmup": warmup,
@@ -399,7 +412,7 @@ def other_workload_leg(args, kc, stream, flush, name: str, T: int, steps: int, w
            "ms_per_step": tot_ms / steps, "roofline": roof, "phase_ms": phase_ms,
            "steps_per_tree": steps_total / (T * steps),
            "ttf": "BIT" if st["ttf_variant"] == kc.KC_TTF_BIT else "SCAN",
-           "walker": walk_kernel(kc, st, True)}
+           "walker": walker}
     out["time_to_eps"] = time_to_eps(kc, g, cfg, args.eps, delta, 1024, stream, name)
     return out
 
@@ -866,10 +879,11 @@ def main():
     steps_total = int(samples["steps"].sum())
     trees_timed = T * args.steps
     auto = args.walker == "auto"
-    traffic_per_step = (WALKER_GRID_DRAM_BYTES_PER_STEP.get(walk_kernel(kc, st, auto))
+    walker = walk_kernel(kc, st, auto, g.deg, reject is not None)
+    traffic_per_step = (WALKER_GRID_DRAM_BYTES_PER_STEP.get(walker)
                         if args.workload.startswith("grid") else None)
     dom, roof, phase_ms = phase_roofline(kc, st, n, trees_timed, steps_total, tot_ms,
-                                         traffic_per_step, auto)
+                                         walker, traffic_per_step)
     roof["traffic_basis"] = (None if roof["traffic"] is None else
                              "ncu dram bytes per departure on grid300x300 (1000 trees) x "
                              "departures")
@@ -887,7 +901,7 @@ def main():
                          f"{st['workspace_bytes'] / 1e9:.1f} GB",
                    "ttf": "BIT" if st["ttf_variant"] == kc.KC_TTF_BIT else "SCAN",
                    "walker": WALKER_NAMES[st["walker"]],
-                   "walk_kernel": walk_kernel(kc, st, auto),
+                   "walk_kernel": walker,
                    "trees_in_flight": st["trees_in_flight"]},
         "roofline": roof,
         "phase_ms": phase_ms,

@@ -138,3 +138,33 @@ def test_update_stream_is_valid_against_the_evolving_graph():
                 adj[v].discard(u)
                 assert connected(u, v)
     assert kinds == {0, 1}
+
+
+def test_the_named_walk_kernel_is_the_one_that_runs():
+    """The rules for the kernel's name: popping in shared memory up to 16000 vertices, or to
+    38000 without a hub; in memory where the root is one; else 32 walkers a tree."""
+    from paper_2511_16356_gb300 import kc
+
+    def name(n, m, root_deg, bit=False, walker=kc.KC_WALK_WARP, auto=True, top=None,
+             trees=1000, reject=False):
+        deg = np.array([root_deg, top if top is not None else root_deg])
+        st = {"n": n, "m": m, "root": 0, "walker": walker, "trees_in_flight": trees,
+              "ttf_variant": kc.KC_TTF_BIT if bit else kc.KC_TTF_SCAN}
+        return bench.walk_kernel(kc, st, auto, deg, reject)
+
+    assert name(16000, 64000, 20) == "k_pop_small"
+    assert name(16001, 64000, 2000) == "k_pop_rounds"
+    assert name(38000, 150000, 2000) == "k_pop_rounds"
+    assert name(38000, 150000, 20) == "k_pop_small"
+    assert name(38001, 150000, 20) == "k_wilson_warp"
+    assert name(4000000, 34000000, 8000) == "k_pop_rounds"
+    assert name(90000, 135000, 4, bit=True) == "k_wilson_queue"
+    assert name(90000, 135000, 4, bit=True, top=40000) == "k_wilson_warp"
+    assert name(2000, 8000, 20, auto=False) == "k_wilson_warp"
+    assert name(2000, 8000, 20, reject=True) == "k_wilson_warp"
+    lane = dict(walker=kc.KC_WALK_LANE, auto=False)
+    assert name(2000, 8000, 20, **lane) == "k_wilson_queue"
+    assert name(2000, 8000, 20, trees=30000, **lane) == "k_wilson"
+    assert name(90000, 135000, 4, bit=True, trees=30000, **lane) == "k_wilson_queue"
+    assert name(90000, 135000, 4, bit=True, trees=30000, reject=True, **lane) == "k_wilson"
+    assert name(2000, 8000, 20, top=40000, **lane) == "k_wilson"
