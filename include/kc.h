@@ -91,7 +91,8 @@ enum { KC_WALK_AUTO = 0,       /* by the graph.  Long diameter (the TTF variant 
                                   hub (16 x 2m / deg(root) <= n); else 32 walkers.
                                   Reported as WARP, or LANE under rejection by walk
                                   length on a BIT graph                                */
-       KC_WALK_LANE = 1,       /* one sequential walker per tree (one lane)              */
+       KC_WALK_LANE = 1,       /* one sequential walker per tree: a warp each, in waves of
+                                  very many trees a lane                               */
        KC_WALK_WARP = 2,       /* 32 concurrent walkers per tree popping cycles in any order */
        KC_WALK_HYBRID = 3 };   /* LANE for a prefix of the start order, then WARP for the
                                   rest; LANE trees still running when a share of the

@@ -165,7 +165,7 @@ __device__ __forceinline__ int32_t commit_path(unsigned gm, uint64_t *word, int3
 // departure with one tree per warp on an otherwise idle SM, of which 40 wait for
 // memory (L1 serves 95%); the 32 lockstep walkers of one tree (k_wilson_warp) take
 // about 650 cycles, a walker per lane (k_wilson) about 1100.  Walk of 500 trees of a
-// 40000-vertex grid: 348 (k_wilson_warp) -> 140 ms; of 4522 trees of the 350x350 grid
+// 40000-vertex grid: 299 (k_wilson_warp) -> 126 ms; of 4522 trees of the 350x350 grid
 // under a cap of 13 n departures: 1640 (k_wilson) -> 350 ms.  The word that held the
 // next target itself, with the queue behind it, made the load chain shorter and the
 // kernel slower: 52 instructions, 250 cycles.

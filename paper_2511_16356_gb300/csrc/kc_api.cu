@@ -406,9 +406,11 @@ int fast_traversal(const kc_graph *g) {
 // kernels with arrows drawn ahead (k1_solo.cu) in place of the handle's walker: for LANE
 // while they are faster than a lane per tree (kc_host::queue_serves), and under AUTO on
 // long-diameter graphs, where 32 walkers of a tree mostly wait for one another
-// (40000-vertex grid, walk in ms with 32 walkers / one: 64 trees 192 / 114, 500
-// trees 348 / 184, 4000 trees 590 / 316).  On graphs of low diameter the 32
-// walkers spread and stay faster (20000-vertex random graph: 24 / 28 ms).
+// (40000-vertex grid, walk in ms with 32 walkers / one: 64 trees 246 / 113, 500
+// trees 299 / 126, 4000 trees 523 / 221).  On graphs of low diameter the 32 walkers
+// spread and stay faster (random graphs of mean degree 8: 50000 vertices, 64 trees 44 / 69,
+// 500 trees 76 / 102; 200000, 64 trees 183 / 288, 500 trees 278 / 434; 10^6, 64 trees 987 /
+// 1795): those past popping keep them.
 bool fits_queues(const kc_graph *g) {
     return kc_host::queue_bits(g->max_deg) <= kc_host::kMaxQueueBits;
 }
@@ -1363,8 +1365,7 @@ void transform_slots(kc_graph *g, const std::vector<int64_t> &slots, bool insert
                                              &nl));
         }
         KC_CK(g, launch_link_cut(g->d_row_off, g->d_col, w, ub.slots, g->d_parents, ub.factor,
-                                 ub.cut, g->root, u, v, g->seed, (uint32_t)g->update_seq, insert,
-                                 g->stream));
+                                 ub.cut, u, v, g->seed, (uint32_t)g->update_seq, insert, g->stream));
         KC_CK(g, launch_scale_slots(g->d_w, ub.slots, ub.factor, b, g->stream));
         check_err(g, insert ? "link-cut" : "cut-link");
         g->t_update.launches += nl + 4;
@@ -2210,7 +2211,7 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
         cfg.hybrid_prefix_permille < 0 || cfg.hybrid_tail_permille < 0 ||
         cfg.tau0_kind < KC_TAU0_BFS || cfg.tau0_kind > KC_TAU0_WILSON)
         return KC_ERR_INVALID_ARG;
-    // rejection by walk length: the 32-walker kernel, static pools, and a cap a
+    // rejection by walk length: not the hybrid walker, static pools, and a cap a
     // tree can meet (every non-root vertex departs at least once)
     if (!(cfg.reject_accept_hint >= 0 && cfg.reject_accept_hint <= 1)) return KC_ERR_INVALID_ARG;
     if (cfg.ttf_segments < 0 || cfg.ttf_segments > 64) return KC_ERR_INVALID_ARG;
@@ -2331,15 +2332,11 @@ kc_status kc_graph_create(int64_t n, const int64_t *row_off, const int32_t *col,
         if (variant == KC_TTF_AUTO) variant = (g->ecc <= 2 * lg) ? KC_TTF_SCAN : KC_TTF_BIT;
         if (variant == KC_TTF_BIT && twom >= ((int64_t)1 << 31)) variant = KC_TTF_SCAN;
         g->ttf_variant = variant;
-        // Walkers: one sequential walker per tree leaves the GPU nearly idle
-        // whenever fewer trees fit in memory than it has warp slots, and a wave
-        // lasts as long as its slowest tree; 32 walkers per tree finish the
-        // long trees of road-shaped graphs about 4 steps per iteration, so they
-        // are the default.  Under rejection by walk length on a long-diameter
-        // graph (BIT variant) no tree walks past the cap, and one walker per
-        // tree keeps every tree of the wave in flight from the start (32-walker
-        // trees wait for one of the SMs' warp slots): the wave then lasts about
-        // cap x one walker's time per departure, which measured shorter.
+        // The handle's walker, which a wave falls back to; use_solo and use_pop say what
+        // AUTO's waves run instead.  32 walkers per tree finish the long trees of a wave
+        // sooner than one lane does.  Under rejection by walk length on a long-diameter
+        // graph (BIT variant) no tree walks past the cap, and one walker per tree keeps
+        // every tree of the wave in flight from the start.
         int walker = cfg.walker;
         if (walker == KC_WALK_AUTO || cfg.autotune)
             walker = (cfg.reject_steps > 0 && !cfg.autotune && variant == KC_TTF_BIT)

@@ -575,12 +575,12 @@ struct CutChoice {
     int32_t x, side;
     int64_t d_old;  // link-cut: length of the cycle less the new edge
 };
-// w.din, w.size and w.aux (preorder) of the trees at `slot` (launch_traverse_parents;
-// cut-link: by_id); w.vol is scratch
+// w.din, w.size and w.aux (preorder) of the trees at `slot` (either traversal; cut-link:
+// children in ascending id); w.vol is scratch
 cudaError_t launch_link_cut(const int64_t *row_off, const int32_t *col, WaveView w,
                             const int64_t *slot, int32_t *pool_parents, double *factor,
-                            CutChoice *choice, int32_t r, int32_t u, int32_t v, uint64_t seed,
-                            uint32_t seq, bool insert, cudaStream_t s);
+                            CutChoice *choice, int32_t u, int32_t v, uint64_t seed, uint32_t seq,
+                            bool insert, cudaStream_t s);
 cudaError_t launch_scale_slots(double *w, const int64_t *slot, const double *factor, int64_t B,
                                cudaStream_t s);
 cudaError_t launch_weight_rescale(double *w, const uint8_t *flag, int64_t P, double *sums,

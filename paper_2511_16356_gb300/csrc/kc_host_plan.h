@@ -115,7 +115,12 @@ constexpr int queue_slots(int bits) { return (31 - bits) / bits; }
 // all of them to be resident (32 an SM) and two trees per warp make them so (48).
 // 350x350 grid under a cap of 13 n departures, walk in ms for 32 / 16 / 8 lanes: 3044
 // trees 260 / 362 / 523, 4522 trees 345 / 397 / 546, 5991 trees 482 / 430 / 575, 8929
-// trees 628 / 742 / 620, 17672 trees 1133 / 1174 / 1204.
+// trees 628 / 742 / 620, 17672 trees 1133 / 1174 / 1204.  Without a cap, 32 / 16 lanes:
+// grid 200x200, 5400 trees 256 / 272, 6000 trees 296 / 286, 7290 trees 301 / 309; random
+// graph of 20000 vertices, 5400 trees 58 / 61, 6600 trees 67 / 62, 7290 trees 68 / 64, 7400
+// trees 70 / 83; power-law graph of 20000, 4800 trees 26 / 32, 4880 trees 37 / 32, 7290
+// trees 44 / 34, 7400 trees 44 / 51; K_300, 6000 trees 1.15 / 1.27.  The range pays from
+// about 40 trees an SM on, on hubs in all of it.
 inline int queue_group(int64_t B, int64_t num_sms) {
     const int64_t per_sm = (B + std::max<int64_t>(num_sms, 1) - 1) / std::max<int64_t>(num_sms, 1);
     return per_sm > 32 && per_sm <= 48 ? 16 : 32;
